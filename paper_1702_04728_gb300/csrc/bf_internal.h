@@ -21,6 +21,7 @@ constexpr int kSub = kUp / kFds; // 16 sub-channels
 constexpr int kFrame = kUp * kTds;   // 384 samples per frame
 constexpr int kInput = kCyl * kFeed * kPol;   // 2048 bytes per time sample
 constexpr int kBeams = kEw * kNs;    // 1024 intensity beams
+constexpr int kLaneTwLen = 32 * 16;     // twiddles between the FP32 form's two N-S stages
 constexpr int kInvLen = kBins + kNs;  // per table: first beam of each bin, next beam of each beam
 
 // Segments per launch (kernel-parameter space holds the descriptors).
@@ -53,7 +54,7 @@ struct Batch {
                              // next beam with the same bin (-1 ends a list)
     const int16_t* order;    // [n_tables][256]   FP32 form: beam taken by consumer slot (TMEM lane + 128 x half)
     const float2* ew;        // [n_tables][4 ew][4 cyl] E-W phases
-    const float2* tw512;     // [512] exp(-2 pi i e / 512)
+    const float2* twl;       // FP32 form: exp(-2 pi i n k / 512) at [n / 2][k][n & 1], n < 16, k < 32
     const float2* tw128;     // [128] exp(-2 pi i e / 128)
     float2* dump;            // debug: up-channelised voltages instead of detection
     int* status;                 // set non-zero by a kernel whose bounded wait expired
@@ -69,7 +70,7 @@ struct Batch {
 cudaError_t fused_fp32_launch(const Batch& b, int grid, cudaStream_t s);
 cudaError_t fused_fp32_dump_launch(const Batch& b, int grid, cudaStream_t s);
 cudaError_t debug_beams_launch(const uint8_t* vin, long long n_samples, const int16_t* lut,
-                               const float2* ew, const float2* tw512, float2* out, cudaStream_t s);
+                               const float2* ew, const float2* twl, float2* out, cudaStream_t s);
 cudaError_t debug_unpack_launch(const uint8_t* in, float* out, long long n, cudaStream_t s);
 int fused_fp32_max_grid(int device);   // CTAs that fit at once (1 per SM)
 

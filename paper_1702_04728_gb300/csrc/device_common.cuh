@@ -26,8 +26,6 @@ __device__ __forceinline__ float2 bc(float v) { return make_float2(v, v); }
 
 __device__ __forceinline__ cp cadd(cp a, cp b) { return {add2(a.re, b.re), add2(a.im, b.im)}; }
 __device__ __forceinline__ cp csub(cp a, cp b) { return {sub2(a.re, b.re), sub2(a.im, b.im)}; }
-// a * (-i)
-__device__ __forceinline__ cp cmul_neg_i(cp a) { return {a.im, mul2(a.re, bc(-1.f))}; }
 // a * (C + i S), C and S pairs (per element of the pair)
 __device__ __forceinline__ cp cmulp(cp a, float2 C, float2 S) {
     return {fma2(a.im, make_float2(-S.x, -S.y), mul2(a.re, C)), fma2(a.re, S, mul2(a.im, C))};
@@ -37,34 +35,6 @@ __device__ __forceinline__ cp ld_cp(const float4* p) {
     return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
 }
 __device__ __forceinline__ void st_cp(float4* p, cp a) { *p = make_float4(a.re.x, a.re.y, a.im.x, a.im.y); }
-
-// cos(2 pi e / 32), e = 0..31, rounded from double precision.
-__device__ __forceinline__ constexpr float cos32(int e) {
-    constexpr float t[32] = {
-        1.000000000e+00f, 9.807852804e-01f, 9.238795325e-01f, 8.314696123e-01f,
-        7.071067812e-01f, 5.555702330e-01f, 3.826834324e-01f, 1.950903220e-01f,
-        0.0f, -1.950903220e-01f, -3.826834324e-01f, -5.555702330e-01f,
-        -7.071067812e-01f, -8.314696123e-01f, -9.238795325e-01f, -9.807852804e-01f,
-        -1.000000000e+00f, -9.807852804e-01f, -9.238795325e-01f, -8.314696123e-01f,
-        -7.071067812e-01f, -5.555702330e-01f, -3.826834324e-01f, -1.950903220e-01f,
-        0.0f, 1.950903220e-01f, 3.826834324e-01f, 5.555702330e-01f,
-        7.071067812e-01f, 8.314696123e-01f, 9.238795325e-01f, 9.807852804e-01f};
-    return t[e & 31];
-}
-__device__ __forceinline__ constexpr float sin32(int e) { return cos32(e - 8); }
-
-// a * exp(-2 pi i e / N) for N | 32 and a compile-time e (after unrolling).
-template <int N>
-__device__ __forceinline__ cp twiddle(cp a, int e) {
-    const int k = (e * (32 / N)) & 31;               // angle in units of 2 pi / 32
-    switch (k) {
-        case 0: return a;
-        case 8: return cmul_neg_i(a);
-        case 16: return {mul2(a.re, bc(-1.f)), mul2(a.im, bc(-1.f))};
-        case 24: return {mul2(a.im, bc(-1.f)), a.re};
-        default: return cmulp(a, bc(cos32(k)), bc(-sin32(k)));
-    }
-}
 
 __device__ __forceinline__ void dft4(cp& a0, cp& a1, cp& a2, cp& a3) {
     const cp s02 = cadd(a0, a2), d02 = csub(a0, a2), s13 = cadd(a1, a3);
@@ -76,46 +46,67 @@ __device__ __forceinline__ void dft4(cp& a0, cp& a1, cp& a2, cp& a3) {
     a3 = csub(d02, d13);
 }
 
+// A packed multiply-add whose three operands are all registers of their own takes 3.7 cycles of a
+// scheduler, one that shares a constant or uniform operand 2.3 and a packed add 2.1 (measured, 2 or
+// more warps); hence compile-time twiddles where the transform allows them, and plain products
+// before an add-only first stage where the twiddles differ per lane.
+//
 // Radix-2 butterfly with a twiddle, factored for fused multiply-adds: with
 // w = c (1 + i t), (a, b) -> (a + w b, a - w b) as p = (1 + i t) b (two FMA)
 // and a +- c p (four FMA), six operations instead of a complex product and two
-// complex additions (eight).  E = e in units of 2 pi / 16, w = exp(-2 pi i E / 16);
-// c = cos(2 pi E / 16), t = -tan(2 pi E / 16), rounded from double precision.
+// complex additions (eight).  kRot: the twiddle is -i w, by exchanging p's parts.
+// t = Im w / c with c as rounded, so both parts of w carry one rounding; the two
+// roundings of p and the sums are relative to |b|, whatever the size of t.
+template <bool kRot>
+__device__ __forceinline__ void bfly_ct(cp& a, cp& b, float c, float t) {
+    const float2 pre = fma2(b.im, bc(-t), b.re), pim = fma2(b.re, bc(t), b.im);
+    if constexpr (kRot) {
+        b = {fma2(pim, bc(-c), a.re), fma2(pre, bc(c), a.im)};
+        a = {fma2(pim, bc(c), a.re), fma2(pre, bc(-c), a.im)};
+    } else {
+        b = {fma2(pre, bc(-c), a.re), fma2(pim, bc(-c), a.im)};
+        a = {fma2(pre, bc(c), a.re), fma2(pim, bc(c), a.im)};
+    }
+}
+
+// cos and sin of 2 pi e / 32, e = 0..8
+__device__ __forceinline__ constexpr double cos32(int e) {
+    constexpr double t[9] = {1.0, 0.98078528040323044913, 0.92387953251128675613, 0.83146961230254523708,
+                             0.70710678118654752440, 0.55557023301960222474, 0.38268343236508977173,
+                             0.19509032201612826785, 0.0};
+    return t[e];
+}
+__device__ __forceinline__ constexpr double sin32(int e) { return cos32(8 - e); }
+
+// The butterfly with w = exp(-2 pi i E / 32), 0 <= E < 16 (E >= 8: -i times E - 8).
 template <int E>
-__device__ __forceinline__ void bfly_tw(cp& a, cp& b) {
-    constexpr float kc[8] = {1.f, 9.238795325e-01f, 7.071067812e-01f, 3.826834324e-01f,
-                             0.f, -3.826834324e-01f, -7.071067812e-01f, -9.238795325e-01f};
-    constexpr float kt[8] = {0.f, -4.142135624e-01f, -1.0f, -2.414213562e+00f,
-                             0.f, 2.414213562e+00f, 1.0f, 4.142135624e-01f};
+__device__ __forceinline__ void bfly(cp& a, cp& b) {
+    static_assert(E >= 0 && E < 16, "angle out of range");
     if constexpr (E == 0) {
         const cp y = cadd(a, b), z = csub(a, b);
         a = y;
         b = z;
-    } else if constexpr (E == 4) {
+    } else if constexpr (E == 8) {
         // w = -i: a - i b = (a.re + b.im, a.im - b.re)
         const cp y = {add2(a.re, b.im), sub2(a.im, b.re)};
         const cp z = {sub2(a.re, b.im), add2(a.im, b.re)};
         a = y;
         b = z;
     } else {
-        const float c = kc[E], t = kt[E];
-        const float2 pre = fma2(b.im, bc(-t), b.re), pim = fma2(b.re, bc(t), b.im);
-        const cp y = {fma2(pre, bc(c), a.re), fma2(pim, bc(c), a.im)};
-        const cp z = {fma2(pre, bc(-c), a.re), fma2(pim, bc(-c), a.im)};
-        a = y;
-        b = z;
+        constexpr float c = (float)cos32(E & 7), t = (float)(-sin32(E & 7) / (double)c);
+        bfly_ct<(E >= 8)>(a, b, c, t);
     }
 }
 
 // forward DFT8 (2 x 4), natural order in and out; the last stage's twiddles
-// W8^k = W16^{2k} fused into its butterflies
+// W8^k fused into its butterflies
 __device__ __forceinline__ void dft8(cp (&x)[8]) {
     dft4(x[0], x[2], x[4], x[6]);
     dft4(x[1], x[3], x[5], x[7]);
-    bfly_tw<0>(x[0], x[1]);
-    bfly_tw<2>(x[2], x[3]);
-    bfly_tw<4>(x[4], x[5]);
-    bfly_tw<6>(x[6], x[7]);
+    bfly<0>(x[0], x[1]);
+    bfly<4>(x[2], x[3]);
+    bfly<8>(x[4], x[5]);
+    bfly<12>(x[6], x[7]);
     // X[k] = x[2k], X[k + 4] = x[2k + 1]
     cp y[8];
 #pragma unroll
@@ -127,35 +118,47 @@ __device__ __forceinline__ void dft8(cp (&x)[8]) {
     for (int k = 0; k < 8; ++k) x[k] = y[k];
 }
 
-// second-stage group k1 of dft16: the four inputs x[4 k1 + n2] with their
-// twiddles W16^{n2 k1} folded into three factored radix-2 levels
-template <int K1>
-__device__ __forceinline__ void dft16_group(cp& x0, cp& x1, cp& x2, cp& x3) {
-    bfly_tw<(2 * K1) & 15>(x0, x2);          // x0 + w2 x2, x0 - w2 x2
-    bfly_tw<(2 * K1) & 15>(x1, x3);          // u = x1 + w2 x3, v = x1 - w2 x3
-    bfly_tw<K1>(x0, x1);                     // out0 = s + w1 u, out2 = s - w1 u
-    bfly_tw<(K1 + 4) & 15>(x2, x3);          // out1 = d - i w1 v, out3 = d + i w1 v
-}
-
-// forward DFT16 (4 x 4), natural order in and out
-__device__ __forceinline__ void dft16(cp (&x)[16]) {
-#pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) dft4(x[n2], x[4 + n2], x[8 + n2], x[12 + n2]);
-    dft16_group<0>(x[0], x[1], x[2], x[3]);
-    dft16_group<1>(x[4], x[5], x[6], x[7]);
-    dft16_group<2>(x[8], x[9], x[10], x[11]);
-    dft16_group<3>(x[12], x[13], x[14], x[15]);
-    // group k1 holds (out0, out2, out1, out3) in its slots (0, 1, 2, 3); X[k1 + 4 k2] = out_k2
+// dft16 leaves X[k + 8 (l & 1) + 4 (l >> 1)] in slot 4 r + l, with (r, k) = (0, 0), (1, 2),
+// (2, 1), (3, 3): put them in natural order.
+__device__ __forceinline__ void dft16_order(cp (&x)[16]) {
     cp y[16];
 #pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) {
-        y[k1] = x[4 * k1];
-        y[k1 + 8] = x[4 * k1 + 1];
-        y[k1 + 4] = x[4 * k1 + 2];
-        y[k1 + 12] = x[4 * k1 + 3];
+    for (int r = 0; r < 4; ++r) {
+        const int k = r == 1 ? 2 : r == 2 ? 1 : r;
+#pragma unroll
+        for (int l = 0; l < 4; ++l) y[k + 8 * (l & 1) + 4 * (l >> 1)] = x[4 * r + l];
     }
 #pragma unroll
     for (int k = 0; k < 16; ++k) x[k] = y[k];
+}
+
+// One radix-4 group of dft16's second stage: inputs in slots 4 r + b, twiddle V^b with
+// V = exp(-2 pi i E / 32).
+template <int E>
+__device__ __forceinline__ void dft16_group(cp& x0, cp& x1, cp& x2, cp& x3) {
+    bfly<2 * E>(x0, x2);
+    bfly<2 * E>(x1, x3);
+    bfly<E>(x0, x1);                         // out 0 and 2
+    bfly<E + 8>(x2, x3);                     // out 1 and 3
+}
+
+// forward DFT16 (4 x 4) of x[n] exp(-2 pi i S n / 32), natural order in and out: S = 0 is the
+// plain transform; S = 1 (the odd bins of a zero-padded DFT32) carries its input twiddles
+// inside the butterflies (176 operations against 148, where a separate product takes 60 more)
+template <int S = 0>
+__device__ __forceinline__ void dft16(cp (&x)[16]) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        bfly<8 * S>(x[b], x[8 + b]);
+        bfly<8 * S>(x[4 + b], x[12 + b]);
+        bfly<4 * S>(x[b], x[4 + b]);         // k = 0, 2
+        bfly<4 * S + 8>(x[8 + b], x[12 + b]);    // k = 1, 3
+    }
+    dft16_group<S>(x[0], x[1], x[2], x[3]);
+    dft16_group<S + 4>(x[4], x[5], x[6], x[7]);
+    dft16_group<S + 2>(x[8], x[9], x[10], x[11]);
+    dft16_group<S + 6>(x[12], x[13], x[14], x[15]);
+    dft16_order(x);
 }
 
 // ---------------------------------------------------------------------------
@@ -172,43 +175,26 @@ __device__ __forceinline__ float2 nib2(uint32_t g0, uint32_t g1) {
     return fma2(make_float2(f0, f1), bc(s), bc(-(8388608.0f * s + 8.0f)));
 }
 
-__device__ __forceinline__ uint32_t word_of(const uint4& v, int k) {
-    return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
-}
-
-// swizzles that make the 128-bit shared accesses conflict-free
-__device__ __forceinline__ int ysw(int n2, int n1) { return n2 * 16 + (n1 ^ ((n2 & 7) ^ ((n2 >> 3) << 2))); }
-__device__ __forceinline__ int tsw(int r, int c) { return r * 16 + (c ^ (r & 7)); }
+// bin rows: swizzle that makes the 128-bit shared accesses conflict-free
 __device__ __forceinline__ int bsw(int L) { return L ^ ((L >> 3) & 1); }
-
-__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" :: "r"(id) : "memory"); }
-
-// Per-lane twiddles of the N-S FFT: exp(-2 pi i n2 (2 k1 + h) / 512), k1 = 0..15.
-struct PostTw {
-    float2 C[16], S[16];
-};
-
-__device__ __forceinline__ void load_post(const float2* __restrict__ tw512, int n2, int h, PostTw& pt) {
-#pragma unroll
-    for (int k1 = 0; k1 < 16; ++k1) {
-        const float2 w = tw512[(n2 * (2 * k1 + h)) & (kBins - 1)];
-        pt.C[k1] = bc(w.x);
-        pt.S[k1] = bc(w.y);
-    }
-}
 
 // E-W weights of cylinders 1..3 for one beam (cylinder 0 is the phase origin, weight 1).
 struct EwW {
     float2 R[3], I[3], NI[3];
 };
 
+// The same bits in a uniform register (every lane holds x): an operand that costs no register read.
+__device__ __forceinline__ float uniform(float x) {
+    return __uint_as_float(__reduce_or_sync(0xffffffffu, __float_as_uint(x)));
+}
+
 __device__ __forceinline__ void load_ew(const float2* __restrict__ ew, int table, int j, EwW& w) {
 #pragma unroll
     for (int c = 1; c < kCyl; ++c) {
         const float2 v = ew[(table * kEw + j) * kCyl + c];
-        w.R[c - 1] = bc(v.x);
-        w.I[c - 1] = bc(v.y);
-        w.NI[c - 1] = bc(-v.y);
+        w.R[c - 1] = bc(uniform(v.x));
+        w.I[c - 1] = bc(uniform(v.y));
+        w.NI[c - 1] = bc(uniform(-v.y));
     }
 }
 
@@ -220,12 +206,6 @@ __device__ __forceinline__ void load_ew_frame(const Seg& sg, const float2* __res
     } else {
         load_ew(ew, sg.table, j, w);
     }
-}
-
-__device__ __forceinline__ void load_row(const uint8_t* p, int lane, uint4 (&in)[kCyl]) {
-#pragma unroll
-    for (int c = 0; c < kCyl; ++c)
-        in[c] = __ldg(reinterpret_cast<const uint4*>(p + c * (kFeed * kPol) + 16 * lane));
 }
 
 // ---------------------------------------------------------------------------

@@ -6,15 +6,19 @@
 // structure-of-arrays form: every value is a pair of two time samples (or two
 // fine channels) that go through identical operations.
 //
-//  phase A, warps 0-7 (8 iterations per pass, 16 time samples each)
-//    * warp w takes the row pair tau = 16 w + 2 it + {0, 1}, staged in shared
-//      memory by cp.async, unpacks the 4+4-bit nibbles (Table 1) exactly and
-//      forms E-W beam j (Sec. 3) -- applied before the N-S transform, legal
-//      because both are linear and the phases do not depend on the feed;
-//    * lanes 0-15 compute the even bins (FFT256 of y), lanes 16-31 the odd
-//      bins (FFT256 of y exp(-i pi n / 256)) of the zero-padded 512-point N-S
-//      FFT (Sec. 3.1), each as 16 x 16 with one shared-memory transpose; all
-//      512 bins of the row pair land in the warp's row of a bin buffer;
+//  phase A, warps 0-7 in two teams of four; a team's iteration is 16 time samples
+//    * a warp takes two row pairs (four time rows, staged in shared memory by
+//      cp.async) and loads them with transposing ldmatrix, so that lane (n2, row
+//      pair) receives the bytes of feeds 16 n1 + n2 for all 16 n1 of every
+//      cylinder, both rows and both polarisations of a feed in one word; it
+//      unpacks the 4+4-bit nibbles (Table 1) exactly and forms E-W beam j
+//      (Sec. 3) in registers -- applied before the N-S transform, legal because
+//      both are linear and the phases do not depend on the feed;
+//    * the zero-padded 512-point N-S FFT (Sec. 3.1) is 32 x 16: every lane runs
+//      the DFT32 over n1 of its 16 values (two DFT16, the odd bins' twiddles at
+//      compile time), one shared-memory transpose, then the twiddles
+//      exp(-2 pi i n2 k / 512) and a DFT16 over n2; all 512 bins of a row pair
+//      land in its row of the team's bin buffer;
 //  gather + first up-channel pass, warps 8-11 (thread = N-S beams m, m + 128)
 //    * bin L(m) of the clamp table (Eq. 1) is picked from the 8 rows of each
 //      time residue pair, an 8-point DFT runs in registers, and the twiddled
@@ -35,35 +39,37 @@
 namespace chimebf {
 namespace {
 
-constexpr int kWarps = 8;                   // phase-A (producer) warps: warp w loads row pair a = w
+constexpr int kWarps = 8;                   // phase-A (producer) warps: two teams of four
+constexpr int kTeam = 4;                    // team q takes the iterations it = q mod 2, warp w of it row pairs 2w, 2w + 1
 constexpr int kCons = 4;                    // gather / up-channel (consumer) warps, one per TMEM lane quarter
 constexpr int kThreads = 32 * (kWarps + kCons);
 
-// named barriers: 0 = whole CTA; FULL of bin buffer b; consumers only.  The release of a
-// bin buffer (EMPTY) is an mbarrier the consumer warps arrive on, so producer warps wait
-// for the consumers without waiting for each other.
+// named barriers: 0 = whole CTA; FULL of bin buffer b (one team and the consumers); consumers
+// only.  The release of a bin buffer (EMPTY) is an mbarrier the consumer warps arrive on, so
+// producer warps wait for the consumers without waiting for each other.
 constexpr int kBarFull = 1, kBarCons = 3;
+constexpr int kFullThreads = 32 * (kTeam + kCons);
 
 // Register split (setmaxnreg): the launch gives every warp kRegLaunch registers per
 // thread; the producer warpgroups (warps 0-7) raise theirs to kRegProd and the
 // consumer warpgroup (warps 8-11) lowers its to kRegCons, within the same total.
-constexpr int kRegLaunch = 168, kRegProd = 176, kRegCons = 152;
+constexpr int kRegLaunch = 168, kRegProd = 184, kRegCons = 136;
 static_assert(kWarps * kRegProd + kCons * kRegCons <= (kWarps + kCons) * kRegLaunch,
               "the register split must fit in the launch's register file share");
 
-// shared memory (float4 = one SoA pair: re0, re1, im0, im1)
-constexpr int kBinsF4 = kWarps * kBins;             // 8 row pairs x 512 bins (one of two buffers)
-constexpr int kYscF4 = kFeed;                        // per warp: its row pair's 256 phased feed lines
-constexpr int kTbF4 = 2 * kFeed;                     // per warp: 2 halves x 16 x 16 (inside its own bin row)
-constexpr int kRawB = 2 * kInput;                    // per producer warp and buffer: its two raw rows
-constexpr size_t kSmemBins = 2 * (size_t)kBinsF4 * 16;   // double-buffered across iterations
-constexpr size_t kSmemYsc = (size_t)kWarps * kYscF4 * 16;
+// shared memory (a bin is one SoA pair of 16 bytes: re0, re1, im0, im1)
+constexpr int kRows = 8;                             // row pairs of a bin buffer (16 time samples)
+constexpr int kBinsF4 = kRows * kBins;               // 8 row pairs x 512 bins (one of two buffers)
+constexpr int kRowB = kBins * 16;                    // bytes of a row pair's bins, before that of its transpose
+constexpr int kRawRow = kInput + 32;                 // raw row stride: four rows in distinct bank groups
+constexpr int kRawB = 4 * kRawRow;                   // per producer warp: its two row pairs
+constexpr size_t kSmemBins = 2 * (size_t)kBinsF4 * 16;   // one buffer per team
 constexpr size_t kSmemRaw = (size_t)kWarps * kRawB;      // raw rows (cp.async), one iteration ahead
 constexpr size_t kSmemLut = 2 * kNs * sizeof(int);   // bins and beams in gather order
 constexpr size_t kSmemTw = 8 * 8 * 16;               // pair twiddles of the first up-channel pass
+constexpr size_t kSmemTwl = kLaneTwLen * sizeof(float2);           // exp(-2 pi i n2 k / 512), [8][32 k] x 2 n2
 constexpr size_t kSmemPark = (size_t)kSub * kNs * sizeof(float);   // first half of the current item
-constexpr size_t kSmemTotal = kSmemBins + kSmemYsc + kSmemRaw + kSmemLut + kSmemTw + kSmemPark;
-static_assert(kTbF4 == kBins, "a warp's transpose scratch is exactly its bin row");
+constexpr size_t kSmemTotal = kSmemBins + kSmemRaw + kSmemLut + kSmemTw + kSmemTwl + kSmemPark;
 
 __device__ __forceinline__ uint32_t smem_sa(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -82,101 +88,127 @@ __device__ __forceinline__ cp lds_cp(uint32_t addr) {
     return a;
 }
 
-// Phase A for one warp and its row pair (two time rows as SoA pairs):
-//   in0/in1   the two raw rows
-//   sel       byte permutation selecting polarisation pol of two feeds
-//   ysc       this warp's phased feed lines [16 n2][16 n1] (swizzled, 4 KB)
-//   tb        this warp's transpose scratch [2 halves][16][16] (8 KB; may be the bin row)
-//   row_bins  the row pair's 512 bins (8 KB)
-// Lanes 0-15 compute the even bins (FFT256 of y), lanes 16-31 the odd bins
-// (FFT256 of y exp(-i pi n / 256)) of the zero-padded 512-point N-S FFT, lane
-// n2 = lane & 15 in each half; `pt` holds that lane's twiddles.  Only warp-level
-// synchronisation: no other warp touches this warp's scratch.
-// Hooks: `after_ew` runs once in0/in1 have been consumed, `before_tb` before
-// the transpose scratch is first written, `after_tb` after the transposed
-// values are loaded (a slot for work that overlaps the last DFT).
-template <class AfterEw, class BeforeTb, class AfterTb>
-__device__ __forceinline__ void phase_a(const uint4 (&in0)[kCyl], const uint4 (&in1)[kCyl], uint32_t sel,
-                                        const EwW& w, const PostTw& pt, uint32_t ysc, uint32_t tb, uint32_t row_bins,
-                                        int lane, AfterEw after_ew, BeforeTb before_tb, AfterTb after_tb) {
-    // unpack + E-W: lane holds feeds 8 lane .. 8 lane + 7 of both rows.  Feed n = 8 lane + 2k (+1)
-    // sits at n2 = n & 15 = 8 (lane & 1) + 2k (+1), n1 = n >> 4 = lane >> 1; ysw(n2, n1) =
-    // 16 n2 + (n1 ^ (n2 & 7) ^ 4 (n2 >> 3)) = 16 n2 + (((lane >> 1) ^ 4 (lane & 1)) ^ (n2 & 7)).
-    const uint32_t yw = ysc + 16u * (uint32_t)(16 * 8 * (lane & 1) + (((lane >> 1) ^ (4 * (lane & 1)))));
+// Four 8 x 8 matrices of 16-bit elements, transposed: lane i gets, from matrix m (row addresses
+// in lanes 8 m .. 8 m + 7), rows 2 (i & 3) (low half) and 2 (i & 3) + 1 (high half) of column i >> 2.
+__device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+
+// The nibbles of one polarisation in a byte pair (low byte polarisation 0): masks and the exact
+// rescaling of the nibble's place in the mantissa of 2^23 (see nib2).
+struct PolSel {
+    uint32_t mi, mr;
+    float si, bi, sr, br;
+};
+__device__ __forceinline__ PolSel pol_sel(int pol) {
+    const float s = pol ? 1.f / 256.f : 1.f;
+    return {pol ? 0xF00u : 0xFu, pol ? 0xF000u : 0xF0u, s, -(8388608.f * s + 8.f), s * 0.0625f,
+            -(524288.f * s + 8.f)};
+}
+__device__ __forceinline__ float2 nibm(uint32_t g0, uint32_t g1, uint32_t m, float s, float b) {
+    return fma2(make_float2(__uint_as_float((g0 & m) | 0x4B000000u), __uint_as_float((g1 & m) | 0x4B000000u)),
+                bc(s), bc(b));
+}
+
+// Lane i of a producer warp stands for row pair R = i & 1 of the warp's two and for
+// n2 = (i >> 2) + 8 H, H = (i >> 1) & 1, until the transpose.
+//
+// Address that the lane passes to ldsm4t: matrix = cylinder i >> 3, matrix row i & 7 = 2 x + e,
+// x = R + 2 H: time row e of row pair R, feeds 8 H .. 8 H + 7 (+ 16 n1, 32 bytes each).  Rows of
+// kRawRow bytes put the eight 16-byte matrix rows in distinct bank groups.
+__device__ __forceinline__ uint32_t raw_lane(uint32_t raw, int lane) {
+    const int x = (lane >> 1) & 3, e = lane & 1;
+    return raw + (uint32_t)((2 * (x & 1) + e) * kRawRow + (lane >> 3) * (kFeed * kPol) + 16 * (x >> 1));
+}
+
+// Transpose slot (16 bytes) of n2 within row k of row pair R: n2 = 8 H + 4 b2 + 2 b1 + b0 goes to
+// 8 b2 + ((4 (b1 ^ R) + 2 H + b0) ^ (k & 7)): the eight lanes that a 128-bit store serves at once
+// (two n2, both H, both R) and the eight rows that a load serves fall in distinct bank groups.
+__device__ __forceinline__ constexpr uint32_t tslot(int n2, int R) {
+    return (uint32_t)(8 * ((n2 >> 2) & 1) + (4 * (((n2 >> 1) & 1) ^ R) + 2 * (n2 >> 3) + (n2 & 1)));
+}
+
+// Phase A for one warp and its two row pairs (SoA pairs of time rows):
+//   raw    the lane's ldsm4t address (raw_lane)
+//   twl    shared address of the lane's first entry of the [8][32] twiddle table
+//   rows   the two row pairs' bins (2 x 8 KB; the transpose runs in place)
+// Only warp-level synchronisation.  Hooks: `after_ew` runs once the raw rows have been read,
+// `before_tb` before the bin rows are first written.
+//
+// Bound: the FMA pipe with the register reads of its operands, 530 packed operations per row pair
+// here and 178 in the consumers.  Two warps per scheduler at 184 registers; one row pair per warp
+// and three warps at 128 registers (lane-dependent twiddles in both transforms) took 1.67 ms against
+// 1.57 ms here for 4 channels x 49152 samples.  The unpack straight from the transposing loads
+// replaced a store and two loads of the phased feeds per row pair and the odd half's divergent
+// twiddles (1.64 ms).
+template <class AfterEw, class BeforeTb>
+__device__ __forceinline__ void phase_a(uint32_t raw, const PolSel& ps, const EwW& w, uint32_t twl,
+                                        uint32_t rows, int lane, AfterEw after_ew, BeforeTb before_tb) {
+    cp y[16];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        cp yA, yB;
+    for (int n1 = 0; n1 < 16; ++n1) {
+        uint32_t g[4];
+        ldsm4t(raw + 32u * n1, g);
 #pragma unroll
         for (int c = 0; c < kCyl; ++c) {
-            const uint32_t g0 = __byte_perm(word_of(in0[c], k), 0u, sel);
-            const uint32_t g1 = __byte_perm(word_of(in1[c], k), 0u, sel);
-            const float2 xiA = nib2<0>(g0, g1), xrA = nib2<1>(g0, g1);
-            const float2 xiB = nib2<2>(g0, g1), xrB = nib2<3>(g0, g1);
+            const uint32_t h = g[c] >> 16;
+            const float2 xi = nibm(g[c], h, ps.mi, ps.si, ps.bi), xr = nibm(g[c], h, ps.mr, ps.sr, ps.br);
             if (c == 0) {
-                yA = {xrA, xiA};
-                yB = {xrB, xiB};
+                y[n1] = {xr, xi};
             } else {
-                yA.re = fma2(xiA, w.NI[c - 1], fma2(xrA, w.R[c - 1], yA.re));
-                yA.im = fma2(xrA, w.I[c - 1], fma2(xiA, w.R[c - 1], yA.im));
-                yB.re = fma2(xiB, w.NI[c - 1], fma2(xrB, w.R[c - 1], yB.re));
-                yB.im = fma2(xrB, w.I[c - 1], fma2(xiB, w.R[c - 1], yB.im));
+                y[n1].re = fma2(xi, w.NI[c - 1], fma2(xr, w.R[c - 1], y[n1].re));
+                y[n1].im = fma2(xr, w.I[c - 1], fma2(xi, w.R[c - 1], y[n1].im));
             }
         }
-        // rows n2 = 2k and 2k + 1 of this lane's half: + 256 n2 bytes, low slot bits ^ n2
-        sts_cp((yw ^ (uint32_t)(16 * (2 * k))) + 256u * (2 * k), yA);
-        sts_cp((yw ^ (uint32_t)(16 * (2 * k + 1))) + 256u * (2 * k + 1), yB);
     }
     after_ew();
-    __syncwarp();
-
-    // half h = lane >> 4 of the padded FFT, lane handles n2 (both halves read the same lines):
-    // ysw(n2, n1) = 16 n2 + (n1 ^ f), f = (n2 & 7) ^ 4 (n2 >> 3)
-    const int h = lane >> 4, n2 = lane & 15;
-    const uint32_t yr = ysc + 16u * (uint32_t)(16 * n2 + ((n2 & 7) ^ (4 * (n2 >> 3))));
-    // loads in the order the first radix-4 stage of dft16 consumes them
-    cp v[16];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        const int n1 = 4 * (q & 3) + (q >> 2);
-        v[n1] = lds_cp(yr ^ (uint32_t)(16 * n1));
-    }
-    if (h) {
-        // odd bins: input times exp(-i pi n / 256) = exp(-2 pi i n1 / 32) * exp(-2 pi i n2 / 512);
-        // the second factor is folded into the per-lane twiddles
-#pragma unroll
-        for (int n1 = 1; n1 < 16; ++n1) v[n1] = twiddle<32>(v[n1], n1);
-    }
-    dft16(v);
-#pragma unroll
-    for (int k1 = 0; k1 < 16; ++k1) v[k1] = cmulp(v[k1], pt.C[k1], pt.S[k1]);
-    // the transpose scratch may share memory with bins still being read elsewhere
-    before_tb();
-    // transpose through tb (one 4 KB block per half): tsw(r, c) = 16 r + (c ^ (r & 7))
-    const uint32_t tbl = tb + 16u * (uint32_t)(h * kFeed);
     {
-        const uint32_t tw_ = tbl + 256u * (uint32_t)n2 + 16u * (uint32_t)(n2 & 7);
+        const int n2 = (lane >> 2) + 4 * (lane & 2), R = lane & 1;
+        const uint32_t tw_ = rows + (uint32_t)(R * kRowB) + 16u * tslot(n2, R);
+        cp v[16];
 #pragma unroll
-        for (int k1 = 0; k1 < 16; ++k1) sts_cp(tw_ ^ (uint32_t)(16 * k1), v[k1]);
+        for (int n1 = 0; n1 < 16; ++n1) v[n1] = y[n1];
+        dft16<0>(v);                                     // even outputs: k = 2 k1
+        // the bin rows may still be read as the previous bins
+        before_tb();
+#pragma unroll
+        for (int k1 = 0; k1 < 16; ++k1) sts_cp((tw_ ^ (uint32_t)(16 * ((2 * k1) & 7))) + 256u * (2 * k1), v[k1]);
+        dft16<1>(y);                                     // odd outputs: k = 2 k1 + 1
+#pragma unroll
+        for (int k1 = 0; k1 < 16; ++k1)
+            sts_cp((tw_ ^ (uint32_t)(16 * ((2 * k1 + 1) & 7))) + 256u * (2 * k1 + 1), y[k1]);
     }
     __syncwarp();
-    const int k1 = n2;
-    {
-        const uint32_t tr_ = tbl + 16u * (uint32_t)k1;
+    // lane = k: twiddles and DFT16 over n2, bins L = 32 k2 + k; bsw(L) = 32 k2 + bsw(k).  The twiddles
+    // are read here, not held through the first half, whose registers are all taken.
+    float2 tw[16];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const cp t = lds_cp(twl + 512u * i);
+        tw[2 * i] = t.re;
+        tw[2 * i + 1] = t.im;
+    }
+#pragma unroll
+    for (int R = 0; R < 2; ++R) {
+        const uint32_t row = rows + (uint32_t)(R * kRowB);
+        const uint32_t tr_ = row + 256u * (uint32_t)lane + 16u * (uint32_t)(lane & 7);
+        cp v[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
-            const int r = 4 * (q & 3) + (q >> 2);
-            v[r] = lds_cp((tr_ ^ (uint32_t)(16 * (r & 7))) + 256u * r);
+            const int n2 = 4 * (q & 3) + (q >> 2);       // in the order dft16 consumes them
+            const uint32_t sl = tslot(n2, R);
+            v[n2] = lds_cp((tr_ ^ (16u * (sl & 7))) + 16u * (sl & 8));
         }
-    }
-    after_tb();
-    dft16(v);
-    // every lane is done with the scratch before the bins (which may share its memory) are written
-    __syncwarp();
-    // bin of the 512-point padded FFT: L = 2 (k1 + 16 k2) + h = 32 k2 + (2 k1 + h), and
-    // bsw(L) = 32 k2 + bsw(2 k1 + h) because bit 3 of L does not depend on k2
-    const uint32_t row = row_bins + 16u * (uint32_t)bsw(2 * k1 + h);
 #pragma unroll
-    for (int k2 = 0; k2 < 16; ++k2) sts_cp(row + 16u * 32u * k2, v[k2]);
+        for (int n2 = 1; n2 < 16; ++n2) v[n2] = cmulp(v[n2], bc(tw[n2].x), bc(tw[n2].y));
+        dft16(v);
+        // every lane has read the row before the bins are written over it
+        __syncwarp();
+        const uint32_t bw = row + 16u * (uint32_t)bsw(lane);
+#pragma unroll
+        for (int k2 = 0; k2 < 16; ++k2) sts_cp(bw + 512u * k2, v[k2]);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -193,40 +225,32 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
 
-__device__ __forceinline__ uint4 lds_u4(uint32_t addr) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr)
-                 : "memory");
-    return v;
-}
-
 // Warps 0-7 (producers) run phase A for their row pairs; warps 8-11 (consumers,
 // one per TMEM lane quarter) gather the clamped bins, run the first up-channel
 // pass into TMEM and, after each block, the second pass and the detection for
-// two bins each (m and m + 128).  The bin rows are double-buffered: producers
-// arrive on the named barrier FULL[b] after writing buffer b, consumers arrive on
-// the mbarrier EMPTY[b] after reading it, so phase A of iteration g + 1 overlaps
-// the gather of iteration g and the second up-channel pass.  A producer can only
-// be two iterations ahead of the slowest consumer and one FULL phase behind
-// the others, so no barrier phase ever mixes iterations.  The EMPTY waits are
-// bounded; on expiry the kernel carries on (keeping every barrier matched) and
-// reports through the status word.
+// two bins each (m and m + 128).  Each team of producers owns one bin buffer and
+// every other iteration: it arrives on the named barrier FULL[b] after writing
+// its buffer, the consumers arrive on the mbarrier EMPTY[b] after reading it, so
+// phase A of an iteration overlaps the gather of the one before and the second
+// up-channel pass.  A team's warp is at most one iteration of its buffer ahead
+// of the slowest consumer, so no barrier phase ever mixes iterations.  The EMPTY
+// waits are bounded; on expiry the kernel carries on (keeping every barrier
+// matched) and reports through the status word.
 template <bool kDump>
 __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_constant__ Batch bt) {
     extern __shared__ __align__(256) unsigned char smem[];   // the swizzles XOR address bits 4-7
     float4* bins_all = reinterpret_cast<float4*>(smem);
-    float4* ysc_all = reinterpret_cast<float4*>(smem + kSmemBins);
-    unsigned char* raw_all = smem + kSmemBins + kSmemYsc;
-    int* lut_s = reinterpret_cast<int*>(smem + kSmemBins + kSmemYsc + kSmemRaw);
+    unsigned char* raw_all = smem + kSmemBins;
+    int* lut_s = reinterpret_cast<int*>(smem + kSmemBins + kSmemRaw);
     int* beam_s = lut_s + kNs;
-    float4* tw_s = reinterpret_cast<float4*>(smem + kSmemBins + kSmemYsc + kSmemRaw + kSmemLut);
-    float* park_s = reinterpret_cast<float*>(smem + kSmemBins + kSmemYsc + kSmemRaw + kSmemLut + kSmemTw);
+    float4* tw_s = reinterpret_cast<float4*>(smem + kSmemBins + kSmemRaw + kSmemLut);
+    float4* twl_s = tw_s + kSmemTw / 16;
+    float* park_s = reinterpret_cast<float*>(smem + kSmemBins + kSmemRaw + kSmemLut + kSmemTw + kSmemTwl);
     __shared__ uint32_t tmem_base_s;
     __shared__ __align__(8) uint64_t empty_s[2];
     __shared__ int expired_s;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    constexpr int kAll = kThreads;
     const uint32_t empty0 = smem_sa(&empty_s[0]);
 
     if (warp == 0) {
@@ -241,6 +265,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
         const float2 w1 = bt.tw128[((2 * it + 1) * c) & (kUp - 1)];
         tw_s[i] = make_float4(w0.x, w1.x, w0.y, w1.y);
     }
+    for (int i = tid; i < kLaneTwLen / 2; i += kThreads) twl_s[i] = reinterpret_cast<const float4*>(bt.twl)[i];
     if (tid == 0) {
         for (int i = 0; i < 2; ++i)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(empty0 + 8u * i), "n"(kCons) : "memory");
@@ -258,11 +283,13 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
     if (warp < kWarps) {
         // ---------------------------------- producers ----------------------------------
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(kRegProd) : "memory");
-        const uint32_t ysc_sa = smem_sa(ysc_all + warp * kYscF4);
-        const uint32_t raw_sa = smem_sa(raw_all) + (uint32_t)(warp * kRawB) + 16u * lane;
-        PostTw pt;
-        load_post(bt.tw512, lane & 15, lane >> 4, pt);
-        uint32_t g = 0;                                   // iterations done by this CTA
+        const int team = warp / kTeam, tw = warp % kTeam;
+        const uint32_t raw_sa = smem_sa(raw_all) + (uint32_t)(warp * kRawB);
+        const uint32_t raw_ld = raw_lane(raw_sa, lane);
+        const uint32_t rows = smem_sa(bins_all + team * kBinsF4 + 2 * tw * kBins);
+        const uint32_t empty = empty0 + 8u * (uint32_t)team;
+        const uint32_t twl = smem_sa(twl_s) + 16u * lane;
+        uint32_t g = 0;                                   // this team's iterations so far
         for (int un = blockIdx.x; un < units.n_units; un += gridDim.x) {
             int item, ps0, ps1, half;
             unit_of(units, un, item, ps0, ps1, half);
@@ -273,61 +300,42 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
             const int F = local >> 2, j = local & 3;
             EwW w;
             load_ew_frame(sg, bt.ew, F, j, w);
-            const long long row0 = (long long)F * kFrame + 16 * warp;
-            // this warp's two rows of iteration (ps, it) into its raw buffer (own bytes only)
+            // time rows 16 a + 2 it + {0, 1} of row pairs a = 2 tw, 2 tw + 1
+            const long long row0 = (long long)F * kFrame + 32 * tw;
+            // this warp's four rows of iteration (ps, it) into its raw buffer
             auto fetch = [&](int ps, int it) {
                 const long long r = row0 + (ps >> 1) * kUp + 2 * it;
-                const uint8_t* p0 = frame_row(sg, r) + 16 * lane;
-                const uint8_t* p1 = frame_row(sg, r + 1) + 16 * lane;
 #pragma unroll
-                for (int c = 0; c < kCyl; ++c) {
-                    cp16(raw_sa + c * (kFeed * kPol), p0 + c * (kFeed * kPol));
-                    cp16(raw_sa + kInput + c * (kFeed * kPol), p1 + c * (kFeed * kPol));
+                for (int k = 0; k < 4; ++k) {
+                    const uint8_t* p = frame_row(sg, r + 16 * (k >> 1) + (k & 1)) + 16 * lane;
+                    const uint32_t d = raw_sa + (uint32_t)(k * kRawRow) + 16u * lane;
+#pragma unroll
+                    for (int c = 0; c < kCyl; ++c) cp16(d + c * (kFeed * kPol), p + c * (kFeed * kPol));
                 }
                 cp_commit();
             };
-            auto load_raw = [&](uint4 (&r0)[kCyl], uint4 (&r1)[kCyl]) {
-#pragma unroll
-                for (int c = 0; c < kCyl; ++c) {
-                    r0[c] = lds_u4(raw_sa + c * (kFeed * kPol));
-                    r1[c] = lds_u4(raw_sa + kInput + c * (kFeed * kPol));
-                }
-            };
-            // The current iteration's raw words are in registers.  Once the unpack has
-            // consumed them, the next iteration's rows are copied into the raw buffer, and
-            // they are read into registers during this iteration's last DFT.
-            uint4 in0[kCyl], in1[kCyl];
-            fetch(ps0, 0);
-            cp_wait<0>();
-            load_raw(in0, in1);
+            fetch(ps0, team);
             for (int ps = ps0; ps < ps1; ++ps) {
-                const int pol = ps & 1;
-                const uint32_t sel = 0x4400u | ((2u + pol) << 4) | (uint32_t)pol;
-                // two iterations per loop body give the scheduler room across the
-                // iteration boundary (measured: unroll 1 / 2 / 4 = 1.652 / 1.632 / 1.652 ms)
-#pragma unroll 2
-                for (int it = 0; it < 8; ++it, ++g) {
-                    const uint32_t b = g & 1u;
-                    const bool more = it < 7 || ps + 1 < ps1;
-                    const uint32_t row_bins = smem_sa(bins_all + b * kBinsF4 + warp * kBins);
-                    phase_a(in0, in1, sel, w, pt, ysc_sa, row_bins, row_bins, lane,
+                const PolSel sel = pol_sel(ps & 1);
+#pragma unroll 1
+                for (int it = team; it < 8; it += 2, ++g) {
+                    cp_wait<0>();
+                    __syncwarp();
+                    phase_a(raw_ld, sel, w, twl, rows, lane,
                             [&] {
-                                if (more) fetch(it < 7 ? ps : ps + 1, it < 7 ? it + 1 : 0);
+                                // every lane has its words: the next iteration's rows may replace them
+                                __syncwarp();
+                                if (it < 6)
+                                    fetch(ps, it + 2);
+                                else if (ps + 1 < ps1)
+                                    fetch(ps + 1, team);
                             },
                             [&] {
-                                // buffer b is free once the consumers gathered it two iterations ago
-                                // (release number g / 2 - 1 of buffer b)
-                                if (g >= 2 && !mbar_wait(empty0 + 8u * b, ((g >> 1) + 1u) & 1u, wlim))
-                                    expired_s = 1;
-                            },
-                            [&] {
-                                // in0 / in1 were consumed by the unpack: the next rows replace them
-                                if (more) {
-                                    cp_wait<0>();
-                                    load_raw(in0, in1);
-                                }
+                                // the buffer is free once the consumers gathered this team's last
+                                // iteration (release number g - 1)
+                                if (g >= 1 && !mbar_wait(empty, (g - 1u) & 1u, wlim)) expired_s = 1;
                             });
-                    bar_arrive_n(kBarFull + (int)b, kAll);
+                    bar_arrive_n(kBarFull + team, kFullThreads);
                 }
             }
         }
@@ -370,7 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
 #pragma unroll 1
                 for (int it = 0; it < 8; ++it, ++g) {
                     const uint32_t b = g & 1u;
-                    bar_sync_n(kBarFull + (int)b, kAll);
+                    bar_sync_n(kBarFull + (int)b, kFullThreads);
                     const float4* bins = bins_all + b * kBinsF4;
                     // gather + 8-point DFT over a (tau = 16 a + b, b = 2 it, 2 it + 1), both bin halves
 #pragma unroll
@@ -473,30 +481,29 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
 // inspection kernels sharing the device code above
 // ---------------------------------------------------------------------------
 
-// Stages 1+2 of 4 consecutive rows per CTA (one warp pair), then the clamp gather.
-__global__ void __launch_bounds__(64) debug_beams_kernel(const uint8_t* __restrict__ vin, long long T,
+// Stages 1+2 of 4 consecutive rows per CTA (one warp: two row pairs), then the clamp gather.
+__global__ void __launch_bounds__(32) debug_beams_kernel(const uint8_t* __restrict__ vin, long long T,
                                                           const int16_t* __restrict__ lut,
-                                                          const float2* __restrict__ ew, const float2* __restrict__ tw512,
+                                                          const float2* __restrict__ ew, const float2* __restrict__ twl,
                                                           float2* __restrict__ out) {
-    __shared__ __align__(256) float4 ysc[2 * kYscF4];     // 256-byte rows: the swizzles XOR address bits 4-7
-    __shared__ __align__(256) float4 tbs[2][kTbF4];
-    __shared__ __align__(256) float4 bins2[2 * kBins];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, e = warp;
+    __shared__ __align__(256) float4 bins2[2 * kBins];    // 256-byte rows: the swizzles XOR address bits 4-7
+    __shared__ __align__(256) unsigned char raw[kRawB];
+    const int lane = threadIdx.x;
     const long long t0 = (long long)blockIdx.x * 4;
     const int pol = blockIdx.y & 1, j = blockIdx.y >> 1;
-    PostTw pt;
-    load_post(tw512, lane & 15, lane >> 4, pt);
+    __shared__ float4 twl_s[kLaneTwLen / 2];
+    for (int i = lane; i < kLaneTwLen / 2; i += 32) twl_s[i] = reinterpret_cast<const float4*>(twl)[i];
     EwW w;
     load_ew(ew, 0, j, w);
-    uint4 in0[kCyl], in1[kCyl];
-    const long long ra = min(t0 + 2 * e, T - 1), rb = min(t0 + 2 * e + 1, T - 1);
-    load_row(vin + ra * kInput, lane, in0);
-    load_row(vin + rb * kInput, lane, in1);
-    const uint32_t sel = 0x4400u | ((2u + pol) << 4) | (uint32_t)pol;
-    phase_a(in0, in1, sel, w, pt, smem_sa(ysc + e * kYscF4), smem_sa(tbs[warp]), smem_sa(bins2 + e * kBins), lane,
-            [] {}, [] {}, [] {});
-    __syncthreads();
-    for (int i = threadIdx.x; i < 4 * kNs; i += 64) {
+    for (int k = 0; k < 4; ++k) {
+        const uint4* p = reinterpret_cast<const uint4*>(vin + min(t0 + k, T - 1) * kInput);
+        for (int i = lane; i < kInput / 16; i += 32) *reinterpret_cast<uint4*>(raw + k * kRawRow + 16 * i) = __ldg(p + i);
+    }
+    __syncwarp();
+    phase_a(raw_lane(smem_sa(raw), lane), pol_sel(pol), w, smem_sa(twl_s) + 16u * lane, smem_sa(bins2), lane, [] {},
+            [] {});
+    __syncwarp();
+    for (int i = lane; i < 4 * kNs; i += 32) {
         const int r = i >> 8, mm = i & 255;          // r: row 0..3 = slot (r >> 1), element (r & 1)
         const long long t = t0 + r;
         if (t >= T) continue;
@@ -566,10 +573,10 @@ int fused_fp32_max_grid(int device) {
 }
 
 cudaError_t debug_beams_launch(const uint8_t* vin, long long T, const int16_t* lut, const float2* ew,
-                               const float2* tw512, float2* out, cudaStream_t s) {
+                               const float2* twl, float2* out, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     dim3 grid((unsigned)((T + 3) / 4), kPol * kEw);
-    debug_beams_kernel<<<grid, 64, 0, s>>>(vin, T, lut, ew, tw512, out);
+    debug_beams_kernel<<<grid, 32, 0, s>>>(vin, T, lut, ew, twl, out);
     return cudaGetLastError();
 }
 

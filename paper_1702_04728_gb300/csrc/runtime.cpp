@@ -121,7 +121,7 @@ struct bf_plan_s {
     int16_t* d_lut = nullptr;
     int16_t* d_order = nullptr;               // FP32 form: gather order of the beams per table
     float2* d_ew = nullptr;
-    float2* d_tw512 = nullptr;
+    float2* d_twl = nullptr;
     float2* d_tw128 = nullptr;
     // Per-frequency table slots (clamp table, gather order, E-W phases and, for the
     // tensor-core form, the FP16 twiddle image).  A slot is referenced by every open
@@ -479,7 +479,7 @@ Batch make_batch(const bf_plan_s* p) {
     b.inv = p->d_inv;
     b.order = p->d_order;
     b.ew = p->d_ew;
-    b.tw512 = p->d_tw512;
+    b.twl = p->d_twl;
     b.tw128 = p->d_tw128;
     b.status = p->d_status;
     b.part = p->d_part;
@@ -898,7 +898,7 @@ int bf_plan(const bf_config* cfg, bf_plan_t* out) {
     CK(cudaMalloc(&p->d_lut, (size_t)p->table_cap * kNs * sizeof(int16_t)));
     CK(cudaMalloc(&p->d_order, (size_t)p->table_cap * kNs * sizeof(int16_t)));
     CK(cudaMalloc(&p->d_ew, (size_t)p->table_cap * kEw * kCyl * sizeof(float2)));
-    CK(cudaMalloc(&p->d_tw512, kBins * sizeof(float2)));
+    CK(cudaMalloc(&p->d_twl, kLaneTwLen * sizeof(float2)));
     CK(cudaMalloc(&p->d_tw128, kUp * sizeof(float2)));
     if (p->dft512) {
         CK(cudaMalloc(&p->d_inv, (size_t)p->table_cap * kInvLen * sizeof(int16_t)));
@@ -909,10 +909,13 @@ int bf_plan(const bf_config* cfg, bf_plan_t* out) {
         CK(cudaMalloc(&p->d_a512, img.size() * sizeof(__half)));
         CK(cudaMemcpy(p->d_a512, img.data(), img.size() * sizeof(__half), cudaMemcpyHostToDevice));
     }
-    std::vector<float2> tw(kBins);
-    for (int e = 0; e < kBins; ++e)
-        tw[e] = make_float2((float)std::cos(-2.0 * kPi * e / kBins), (float)std::sin(-2.0 * kPi * e / kBins));
-    CK(cudaMemcpy(p->d_tw512, tw.data(), kBins * sizeof(float2), cudaMemcpyHostToDevice));
+    std::vector<float2> tw(kLaneTwLen);
+    for (int n = 0; n < 16; ++n)
+        for (int k = 0; k < 32; ++k)
+            tw[((n >> 1) * 32 + k) * 2 + (n & 1)] = make_float2((float)std::cos(-2.0 * kPi * (n * k) / kBins),
+                                                                (float)std::sin(-2.0 * kPi * (n * k) / kBins));
+    CK(cudaMemcpy(p->d_twl, tw.data(), kLaneTwLen * sizeof(float2), cudaMemcpyHostToDevice));
+    tw.resize(kUp);
     for (int e = 0; e < kUp; ++e)
         tw[e] = make_float2((float)std::cos(-2.0 * kPi * e / kUp), (float)std::sin(-2.0 * kPi * e / kUp));
     CK(cudaMemcpy(p->d_tw128, tw.data(), kUp * sizeof(float2), cudaMemcpyHostToDevice));
@@ -1090,7 +1093,7 @@ int bf_destroy(bf_plan_t p) {
     cudaFree(p->d_lut);
     cudaFree(p->d_order);
     cudaFree(p->d_ew);
-    cudaFree(p->d_tw512);
+    cudaFree(p->d_twl);
     cudaFree(p->d_tw128);
     cudaFree(p->d_part);
     cudaFree(p->d_part_tok);
@@ -1253,7 +1256,7 @@ int bf_debug_beams(bf_plan_t p, double freq_hz, const uint8_t* d_vin, int64_t n_
     if (rc) return rc;
     const int tab = hold.idx;
     CK(debug_beams_launch(d_vin, n_samples, p->d_lut + (size_t)tab * kNs, p->d_ew + (size_t)tab * kEw * kCyl,
-                          p->d_tw512, reinterpret_cast<float2*>(d_out), p->stream));
+                          p->d_twl, reinterpret_cast<float2*>(d_out), p->stream));
     CK(cudaStreamSynchronize(p->stream));
     return BF_OK;
 }
