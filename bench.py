@@ -40,7 +40,7 @@ FORM_NAMES = {"BF_FP32_FFT": "fp32_fft", "BF_TC_DFT256": "tc_dft256_3term",
 # tensor flop per input-sample of each tensor-core form: 8 real flop per (row, feed) and
 # term, over the 256 clamped rows or all 512 rows of the zero-padded transform
 TC_FLOP = {"tc_dft256_3term": 3 * 2048, "tc_dft256_2term": 2 * 2048, "tc_dft256_1term": 2048,
-           "tc_dft512_1term": 4096}
+           "tc_dft512_1term": 2048}      # of the 512 rows only the 256 that the clamp keeps
 
 
 def bench_config(form: str) -> dict:
@@ -53,12 +53,11 @@ def bench_config(form: str) -> dict:
 KERNEL_SOURCES = {
     "fused_fp32_kernel": ["fused_fp32.cu", "device_common.cuh", "bf_internal.h"],
     "fused_tc_kernel": ["fused_tc.cu", "device_common.cuh", "bf_internal.h"],
-    "fused_tc_pair_kernel": ["fused_tc_pair.cu", "device_common.cuh", "bf_internal.h"],
 }
 # the kernel that runs each form's detecting launches
 FORM_KERNEL = {"fp32_fft": "fused_fp32_kernel", "tc_dft256_3term": "fused_tc_kernel",
-               "tc_dft256_2term": "fused_tc_kernel", "tc_dft256_1term": "fused_tc_pair_kernel",
-               "tc_dft512_1term": "fused_tc_pair_kernel"}
+               "tc_dft256_2term": "fused_tc_kernel", "tc_dft256_1term": "fused_tc_kernel",
+               "tc_dft512_1term": "fused_tc_kernel"}
 
 
 def kernel_hash(kernel: str) -> str:

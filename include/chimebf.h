@@ -48,14 +48,14 @@ extern "C" {
  * clamped zero-padded FFT (Sec. 3.1, Eq. 1) as the equivalent DFT over the 256
  * kept rows on tcgen05 (FP16 operands, FP32 accumulation); the E-W phased feed
  * line is split into FP16 hi + lo, the twiddles are FP16 hi (+ lo).
- * BF_TC_DFT512 evaluates all 512 rows of the zero-padded transform (the 512
- * redundant beams of Sec. 3.1) with one GEMM term and applies the clamp to the
- * result: the same output as BF_TC_DFT256_X1 at twice the GEMM and
- * up-channelisation work.  Its plans refuse the stage dumps and the stall
- * check (BF_EINVAL). */
+ * BF_TC_DFT512 is the clamp applied to all 512 rows of the zero-padded
+ * transform (the 512 redundant beams of Sec. 3.1) with one GEMM term.  Rows that
+ * no pointing keeps reach no output, so they are not computed: it runs the
+ * BF_TC_DFT256_X1 kernel and gives its output bit for bit.  Its plans refuse
+ * the stage dumps (BF_EINVAL). */
 #define BF_FP32_FFT      0 /* FP32 zero-padded FFT on the CUDA cores                */
 #define BF_TC_DFT256     1 /* 3 GEMM terms: twiddles hi+lo x data hi+lo             */
-#define BF_TC_DFT512     2 /* all 512 padded rows, 1 GEMM term, clamp at the output */
+#define BF_TC_DFT512     2 /* clamp of all 512 padded rows, 1 GEMM term             */
 #define BF_TC_DFT256_X2  3 /* 2 GEMM terms: twiddles hi x data hi+lo                */
 #define BF_TC_DFT256_X1  4 /* 1 GEMM term: twiddles hi x data hi                    */
 
@@ -277,10 +277,8 @@ int bf_debug_gemm(bf_plan_t p, double freq_hz, const uint8_t* d_vin, int64_t n_s
  * paper): runs a tensor-core kernel on one frame (d_vin: device, 384 x 2048
  * bytes, 16-byte aligned) with its MMA thread idle, so no pipeline stage is
  * ever released, and every mbarrier wait bounded by wait_ns (1 .. 2e9).  The
- * kernel is the plan's own for the 1-term and 512-row forms (one cluster of
- * two or four CTAs, which also exchange data-tile copies before their waits
- * run out) and the single-CTA tensor-core kernel for every other form.  It
- * neither traps nor spins unbounded: its waits run out, it frees its tensor
+ * kernel is the 1-term tensor-core kernel (one cluster of two CTAs), whatever
+ * the plan's form.  It neither traps nor spins unbounded: its waits run out, it frees its tensor
  * memory and reports through the plan's status word, and the call returns
  * BF_ETIMEDOUT, after which the plan and the CUDA context remain usable.
  * BF_OK would mean a wait did not expire.  Any plan form may call it; it

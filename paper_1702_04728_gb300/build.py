@@ -1,6 +1,6 @@
 """Build the in-tree CUDA library ``_lib/libchimebf.so`` for sm_103a.
 
-Two translation units are compiled in parallel with nvcc and linked into one
+The translation units are compiled in parallel with nvcc and linked into one
 shared library (static CUDA runtime).  Run as ``python -m
 paper_1702_04728_gb300.build`` or through ``__graft_entry__.build()``.
 """
@@ -18,7 +18,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIBDIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(LIBDIR, "libchimebf.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["fused_fp32.cu", "fused_tc.cu", "fused_tc_pair.cu", "post.cu", "runtime.cpp"]
+SOURCES = ["fused_fp32.cu", "fused_tc.cu", "post.cu", "runtime.cpp"]
 
 
 def nvcc() -> str:

@@ -22,7 +22,6 @@ constexpr int kFrame = kUp * kTds;   // 384 samples per frame
 constexpr int kInput = kCyl * kFeed * kPol;   // 2048 bytes per time sample
 constexpr int kBeams = kEw * kNs;    // 1024 intensity beams
 constexpr int kLaneTwLen = 32 * 16;     // twiddles between the FP32 form's two N-S stages
-constexpr int kInvLen = kBins + kNs;  // per table: first beam of each bin, next beam of each beam
 
 // Segments per launch (kernel-parameter space holds the descriptors).
 constexpr int kMaxSegs = 160;
@@ -46,12 +45,36 @@ struct Seg {
     const unsigned char* a_img;  // tensor-core form: FP16 twiddle image(s) of this segment's table
 };
 
+// Work units of a launch whose items (six passes each) go to `slots` CTAs or CTA pairs in turn: whole
+// items, and the items of a last round that would not fill the slots in parts of g passes, g chosen
+// for the fewest passes of any slot (of equals the largest).  Every output adds the six passes' sums in
+// one fixed order, whether or not its item was split, so the result does not depend on how a request
+// was batched.
+struct PassUnits {
+    int n_full;     // items run whole: 0 .. n_full - 1
+    int g;          // passes of a part of the others (1, 2, 3; 6: none is split)
+    int n_units;    // n_full + (6 / g) x (split items)
+};
+inline PassUnits pass_units(int n_items, int slots, bool split) {
+    constexpr int kPasses = kTds * kPol;
+    PassUnits u{n_items, kPasses, n_items};
+    const int rem = n_items % slots;
+    if (!split || rem == 0) return u;
+    int best = kPasses;
+    for (int g = 3; g >= 1; --g) {
+        const int cost = (rem * (kPasses / g) + slots - 1) / slots * g;
+        if (cost < best) {
+            best = cost;
+            u = {n_items - rem, g, n_items - rem + rem * (kPasses / g)};
+        }
+    }
+    return u;
+}
+
 struct Batch {
     int n_segs;
     int n_items;
     const int16_t* lut;      // [n_tables][256]   clamp table, Eq. (1)
-    const int16_t* inv;      // [n_tables][kInvLen] 512-row form: first beam of each bin, then the
-                             // next beam with the same bin (-1 ends a list)
     const int16_t* order;    // [n_tables][256]   FP32 form: beam taken by consumer slot (TMEM lane + 128 x half)
     const float2* ew;        // [n_tables][4 ew][4 cyl] E-W phases
     const float2* twl;       // FP32 form: exp(-2 pi i n k / 512) at [n / 2][k][n & 1], n < 16, k < 32
@@ -59,10 +82,10 @@ struct Batch {
     float2* dump;            // debug: up-channelised voltages instead of detection
     int* status;                 // set non-zero by a kernel whose bounded wait expired
     unsigned long long wait_ns;  // bound on each device-side wait (0: the default, 2 s)
-    float* part;                 // halves of split items [grid / 2 + 1][2][16][256] (null: no split)
-    unsigned long long* part_tok;    // [grid / 2 + 1][256] handshake tokens (2 x epoch + half)
+    PassUnits units;             // tensor-core form: work units of the launch
+    float* part;                 // sums of split items' passes [grid][6][16][256] (null: no split)
+    unsigned long long* part_tok;    // [grid][256] handshake tokens
     unsigned long long epoch;        // this launch's number within the plan (from 1)
-    float* park;                 // tensor-core form: first half of each CTA's item [grid][16][256]
     Seg segs[kMaxSegs];
 };
 
@@ -74,21 +97,14 @@ cudaError_t debug_beams_launch(const uint8_t* vin, long long n_samples, const in
 cudaError_t debug_unpack_launch(const uint8_t* in, float* out, long long n, cudaStream_t s);
 int fused_fp32_max_grid(int device);   // CTAs that fit at once (1 per SM)
 
-// Tensor-core form: `terms` = 1, 2 or 3 GEMM terms; mode 0 = detect,
-// 1 = dump up-channelised voltages, 2 = dump the N-S/E-W beams of the GEMM,
-// 3 = stall check (1 term only): the MMA warp stays idle, so the producers'
-// bounded waits run out and the kernel reports through `status`.
-cudaError_t fused_tc_launch(const Batch& b, int terms, int mode, int grid, cudaStream_t s);
-// Tensor-core form, 1 term, detection: clusters of two CTAs (grid even, at most one
-// CTA per SM), each CTA 128 of the 256 bins of every item; no item is split.
-cudaError_t fused_tc_pair_launch(const Batch& b, int grid, cudaStream_t s);
-// The 512-row form (all bins of the zero-padded transform, clamp at the output) on clusters
-// of four CTAs; the grid is the clusters that fit at once.
-cudaError_t fused_tc_dft512_launch(const Batch& b, cudaStream_t s);
-// Stall check of the cluster kernel (cluster 2 or 4 CTAs, one cluster): the MMA thread stays
-// idle, the other waits run out against b.wait_ns and the kernel reports through b.status.
-cudaError_t fused_tc_pair_stall_launch(const Batch& b, int cluster, cudaStream_t s);
+// Tensor-core form on `pairs` clusters of two CTAs over b.units: `terms` = 1, 2 or 3 GEMM terms; mode
+// 0 = detect, 1 = dump up-channelised voltages, 2 = dump the N-S/E-W beams of the GEMM, 3 = stall check
+// (1 term only): the MMA thread stays idle, so the other waits run out and the kernel reports through
+// `status`.
+cudaError_t fused_tc_launch(const Batch& b, int terms, int mode, int pairs, cudaStream_t s);
 size_t tc_a_bytes(int terms);    // bytes of one table's twiddle image(s)
+// byte offset in an image of cos (part 0) or sin (part 1) of 2 pi n L(m) / 512, FP16; the lo image follows
+size_t tc_a_offset(int m, int n, int part);
 cudaError_t skymap_launch(const float* in, int n_beams, long long per_beam, float* map, cudaStream_t s);
 cudaError_t dedisperse_launch(const float* in, const int* delays, int n_sub, long long nf, long long n_out,
                               float* out, cudaStream_t s);
@@ -99,7 +115,6 @@ constexpr int kMaxDevices = 64;
 cudaError_t dedisperse_static_table(int device, int** table);
 cudaError_t rescale_u8_launch(const float* in, long long rows, long long nf, uint8_t* codes, float* stats,
                               cudaStream_t s);
-int tc_chunk_k(int terms);       // K elements per shared-memory chunk
 // FP32 FMA-pipe probe: 4 CTAs per SM (at most n_sink / 256) of 256 threads, each
 // thread `iters` (rounded up to 4) x 16 FFMA2 (paired) or 32 scalar FMA; *flop = flops issued.
 cudaError_t fma_probe_launch(bool paired, long long iters, float* sink, long long n_sink, int sms, double* flop,

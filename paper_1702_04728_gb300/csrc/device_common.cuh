@@ -162,17 +162,24 @@ __device__ __forceinline__ void dft16(cp (&x)[16]) {
 }
 
 // ---------------------------------------------------------------------------
-// 4+4-bit unpack (Table 1) of the same byte position in two rows.  The nibble
-// (already shifted by 4 q bits) sits in the mantissa of 2^23; one FFMA2 scales
-// it back by 16^-q and removes 2^23 and the +8 offset -- exact throughout.
+// 4+4-bit unpack (Table 1) of the same byte position in two words.  A nibble at bit q of a word sits
+// in the mantissa of 2^23; one FFMA2 scales it back by 2^-q and removes 2^23 and the +8 offset --
+// exact throughout.
 // ---------------------------------------------------------------------------
-template <int Q>
-__device__ __forceinline__ float2 nib2(uint32_t g0, uint32_t g1) {
-    constexpr uint32_t mask = 0xFu << (4 * Q);
-    constexpr float s = 1.0f / float(1u << (4 * Q));
-    const float f0 = __uint_as_float((g0 & mask) | 0x4B000000u);
-    const float f1 = __uint_as_float((g1 & mask) | 0x4B000000u);
-    return fma2(make_float2(f0, f1), bc(s), bc(-(8388608.0f * s + 8.0f)));
+// The nibbles of one polarisation in a byte pair (low byte polarisation 0): masks and the
+// constants of the exact rescaling.
+struct PolSel {
+    uint32_t mi, mr;
+    float si, bi, sr, br;
+};
+__device__ __forceinline__ PolSel pol_sel(int pol) {
+    const float s = pol ? 1.f / 256.f : 1.f;
+    return {pol ? 0xF00u : 0xFu, pol ? 0xF000u : 0xF0u, s, -(8388608.f * s + 8.f), s * 0.0625f,
+            -(524288.f * s + 8.f)};
+}
+__device__ __forceinline__ float2 nibm(uint32_t g0, uint32_t g1, uint32_t m, float s, float b) {
+    return fma2(make_float2(__uint_as_float((g0 & m) | 0x4B000000u), __uint_as_float((g1 & m) | 0x4B000000u)),
+                bc(s), bc(b));
 }
 
 // bin rows: swizzle that makes the 128-bit shared accesses conflict-free
@@ -328,6 +335,38 @@ __device__ __forceinline__ bool second_half(unsigned long long* tok, unsigned lo
     return true;
 }
 
+// Pass units (see PassUnits): item and pass range [ps0, ps1) of unit `un`.
+__device__ __forceinline__ void pass_unit(const PassUnits& u, int un, int& item, int& ps0, int& ps1) {
+    constexpr int kPasses = kTds * kPol;
+    if (un < u.n_full) {
+        item = un;
+        ps0 = 0;
+        ps1 = kPasses;
+    } else {
+        const int v = un - u.n_full, parts = kPasses / u.g;
+        item = u.n_full + v / parts;
+        ps0 = (v % parts) * u.g;
+        ps1 = ps0 + u.g;
+    }
+}
+
+// A thread of a split item has published the sums of n passes: true for the one that completes the
+// six (all of them are then visible to it).  The token holds the launch's epoch and the passes
+// counted so far, so a launch that was abandoned leaves nothing to clean up, and nothing waits.
+__device__ __forceinline__ bool add_passes(unsigned long long* tok, unsigned long long epoch, unsigned n) {
+    __threadfence();                                   // the published sums before the token
+    unsigned long long seen = *(volatile unsigned long long*)tok, next;
+    for (;;) {
+        next = ((seen >> 3) == epoch ? seen : epoch << 3) + n;
+        const unsigned long long was = atomicCAS(tok, seen, next);
+        if (was == seen) break;                        // else another part's thread has counted: try again
+        seen = was;
+    }
+    if ((next & 7u) != (unsigned)(kTds * kPol)) return false;
+    __threadfence();                                   // the other parts' sums after their tokens
+    return true;
+}
+
 // CTA barrier that also orders tensor-memory accesses across it.
 __device__ __forceinline__ void cta_sync() {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -457,9 +496,9 @@ __device__ __forceinline__ void tmem_ld32f(uint32_t taddr, float (&v)[32]) {
 
 // First up-channel pass in place on the split layout (t = 16 a + b): 8-point
 // DFT over a for the residue pair (b0, b0 + 1), twiddled by exp(-2 pi i b c / 128).
-__device__ __forceinline__ void upchan_pass1_split(uint32_t base, const float4* tw_s, int sub, int nsub) {
+__device__ __forceinline__ void upchan_pass1_split(uint32_t base, const float4* tw_s) {
 #pragma unroll 1
-    for (int bp = sub; bp < 8; bp += nsub) {
+    for (int bp = 0; bp < 8; ++bp) {
         const int b0 = 2 * bp;
         cp z[8];
         tmem_ld_p1(base + b0, z);
@@ -477,10 +516,9 @@ __device__ __forceinline__ void upchan_pass1_split(uint32_t base, const float4* 
 }
 
 // Second pass on the split layout: Re of (c, b) at 16 c + b, Im at 128 + 16 c + b.
-__device__ __forceinline__ void upchan_pass2_split(uint32_t base, float2 (&acc)[kSub], float2* dump, int sub,
-                                                   int nsub) {
+__device__ __forceinline__ void upchan_pass2_split(uint32_t base, float2 (&acc)[kSub], float2* dump) {
 #pragma unroll 1
-    for (int cpi = sub; cpi < 4; cpi += nsub) {
+    for (int cpi = 0; cpi < 4; ++cpi) {
         float re[32], im[32];
         tmem_ld32f(base + 32 * cpi, re);
         tmem_ld32f(base + 128 + 32 * cpi, im);

@@ -95,22 +95,6 @@ __device__ __forceinline__ void ldsm4t(uint32_t addr, uint32_t (&r)[4]) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
 
-// The nibbles of one polarisation in a byte pair (low byte polarisation 0): masks and the exact
-// rescaling of the nibble's place in the mantissa of 2^23 (see nib2).
-struct PolSel {
-    uint32_t mi, mr;
-    float si, bi, sr, br;
-};
-__device__ __forceinline__ PolSel pol_sel(int pol) {
-    const float s = pol ? 1.f / 256.f : 1.f;
-    return {pol ? 0xF00u : 0xFu, pol ? 0xF000u : 0xF0u, s, -(8388608.f * s + 8.f), s * 0.0625f,
-            -(524288.f * s + 8.f)};
-}
-__device__ __forceinline__ float2 nibm(uint32_t g0, uint32_t g1, uint32_t m, float s, float b) {
-    return fma2(make_float2(__uint_as_float((g0 & m) | 0x4B000000u), __uint_as_float((g1 & m) | 0x4B000000u)),
-                bc(s), bc(b));
-}
-
 // Lane i of a producer warp stands for row pair R = i & 1 of the warp's two and for
 // n2 = (i >> 2) + 8 H, H = (i >> 1) & 1, until the transpose.
 //
@@ -515,9 +499,9 @@ __global__ void __launch_bounds__(32) debug_beams_kernel(const uint8_t* __restri
 __global__ void debug_unpack_kernel(const uint8_t* __restrict__ in, float2* __restrict__ out, long long n) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    // byte i goes through the same path as a polarisation-0 byte of a feed A
-    const uint32_t g = __byte_perm((uint32_t)in[i], 0u, 0x4420u);
-    const float2 re = nib2<1>(g, g), im = nib2<0>(g, g);
+    const uint32_t g = in[i];                            // as a polarisation-0 byte
+    const PolSel ps = pol_sel(0);
+    const float2 re = nibm(g, g, ps.mr, ps.sr, ps.br), im = nibm(g, g, ps.mi, ps.si, ps.bi);
     out[i] = make_float2(re.x, im.x);
 }
 

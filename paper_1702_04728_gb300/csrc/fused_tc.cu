@@ -1,33 +1,44 @@
-// Tensor-core form of the fan-beam path for sm_103a (arXiv 1702.04728, Sec. 3).
+// Tensor-core forms of the fan-beam path for sm_103a (arXiv 1702.04728, Sec. 3 and 3.1).
 //
-// Same work decomposition as the FP32 kernel -- one CTA per SM owns
-// (channel segment, frame F, E-W beam j) and makes six passes (3 blocks x 2
-// pols) -- but the N-S stage (Sec. 3.1: zero-padded FFT kept at the 256 bins
-// of Eq. 1) is evaluated as the equivalent dense DFT over the clamped rows on
-// the tcgen05 tensor cores:
+// The N-S stage (zero-padded FFT kept at the 256 bins of Eq. 1) is evaluated as the equivalent
+// dense DFT over the clamped rows on tcgen05:
 //
 //   X[m][t] = sum_n exp(-2 pi i n L(m) / 512) y_j[n][t],   m < 256, n < 256,
 //
-// with y_j the E-W phased feed line (Sec. 3) of block time t.  As a real GEMM:
-// rows = bins m (two M = 128 tiles), columns = (t, re/im) (N = 256), K = (n,
-// re/im) = 512.  With A[m][2n] = cos, A[m][2n+1] = sin (of 2 pi n L / 512) the
-// column t of B holds (yr, yi) and column 128 + t holds (yi, -yr), so the two
-// halves give Re and Im of X with one A.  The accumulator lands in tensor
-// memory where the up-channel passes read it: lane = bin (m, m + 128), columns
-// [0, 128) = Re X(t), [128, 256) = Im X(t) of each 256-column bin half.
+// with y_j the E-W phased feed line (Sec. 3) of block time t.  With C = cos, S = sin of
+// 2 pi n L(m) / 512 and y = yr + i yi this is four real products,
 //
-// Precision: FP16 operands, FP32 accumulation.  y is split y = y_hi + y_lo in
-// FP16 (22 bits together); the twiddles are FP16 (hi) and, for three terms,
-// also lo.  Terms: 1 = A_hi y_hi, 2 = + A_hi y_lo, 3 = + A_lo y_hi.
+//   Re X = C yr + S yi,   Im X = C yi - S yr,
 //
-// Pipeline per pass: K is streamed in chunks through two shared-memory stages.
-// Thread 0 starts the bulk copy (TMA engine) of each twiddle chunk one chunk
-// ahead; all warps build the B chunk (unpack, E-W, FP16 split) from raw bytes
-// prefetched into registers one chunk ahead and arrive on the stage's "B full"
-// mbarrier; thread 0 waits for B and twiddles, issues the MMAs and commits
-// them to the stage's "empty" mbarrier, which the producers wait on before
-// reusing the stage.  No CTA barrier sits inside the chunk loop.  Every wait is
-// bounded by %globaltimer; on expiry the kernel records an error and leaves.
+// so one FP16 image of C and S and one copy of yr and yi serve both parts (the minus sign is the
+// instruction's operand negation).  FP16 operands, FP32 accumulation; y is split y = hi + lo (22
+// bits together) and the twiddles are hi, for three terms hi + lo.  Terms: 1 = T_hi y_hi,
+// 2 = + T_hi y_lo, 3 = + T_lo y_hi.
+//
+// A cluster of two CTAs on neighbouring SMs owns a work item (channel segment, frame F, E-W beam j)
+// and its six passes (3 blocks x 2 pols), one tcgen05 pair (cta_group::2, M = 256, N = 128, K = 16)
+// per step:
+//   * CTA r keeps the hi twiddles of bins 128 r .. 128 r + 127 for all feeds in shared memory
+//     (128 KB), reloaded only when the item's channel changes;
+//   * CTA r builds yr and yi of block times 64 r .. 64 r + 63 (unpack, E-W toward beam j, FP16), its
+//     half of the pair's N = 128 columns; the tensor cores of both SMs read both halves, so nothing
+//     is copied between the CTAs.  The lo twiddles of the 3-term form stream through the ring;
+//   * the accumulator of a pass is 128 bins x (128 Re + 128 Im) columns per CTA, half of tensor
+//     memory, so passes alternate between the halves and the MMAs of pass p + 1 overlap the
+//     up-channel passes (Sec. 3.2) of pass p.
+//
+// Per CTA: warps 0-7 build (one (time, 8 feeds) task per thread and 32-feed chunk, the next chunk's
+// raw rows prefetched into registers), warps 8-11 (one per tensor-memory lane quarter) run the
+// up-channel passes and detection for one bin per thread, warp 12 loads the twiddles and, in the first
+// CTA, issues the MMAs of the pair.  Hand-offs are mbarriers only; every wait is bounded
+// by %globaltimer, and on expiry the CTA records the failure and leaves its loops (the other CTA's
+// waits then expire too).
+//
+// Bound: the builders' unpack and E-W arithmetic (FP32 pipe) and the latency of two builder warps per
+// scheduler; the tensor pipe needs 512 x terms cycles of a chunk (3 terms: it and the shared-memory
+// reads of its operands).  Per 4 x 49152-sample request on 152 SMs: 1.02 / 1.36 / 1.75 ms for 1 / 2 / 3
+// terms, where one CTA with streamed twiddles took 1.89 (2) and 2.55 (3) and CTAs that copied the data
+// tile to each other 1.36 (1).
 #include "device_common.cuh"
 
 #include <cuda_fp16.h>
@@ -38,452 +49,507 @@
 namespace chimebf {
 namespace {
 
+constexpr int kTFeeds = 32;                       // feeds per chunk
+constexpr int kTNch = kFeed / kTFeeds;            // 8 chunks per pass
+constexpr int kTTw = 128 * kTFeeds * 2;           // 8 KB: C or S of 128 bins for one chunk
+// Operands are K-major without swizzle: 8-row x 16-byte core matrices, k-groups (8 feeds) *Lbo and
+// 8-row groups *Sbo bytes apart.
+constexpr int kTALbo = 128, kTASbo = kTFeeds / 8 * kTALbo;
+constexpr int kTBuild = 8;                        // builder warps
+constexpr int kTUp = 4;                           // up-channel warps
+constexpr int kTMma = kTBuild + kTUp;             // the MMA / twiddle warp
+constexpr int kTThreads = 32 * (kTMma + 1);
+// Register split (setmaxnreg): builders kTRegBuild, up-channel warps kTRegUp, the MMA warp keeps the
+// launch count; the launcher checks that the launch gives enough (with fewer, the up-channel warps'
+// increase could never be granted).
+constexpr int kTRegBuild = 104, kTRegUp = 176;
 
 template <int TERMS>
 struct TcCfg {
-    static constexpr int KC = TERMS == 3 ? 32 : 64;              // K elements (FP16) per chunk
-    static constexpr int NCH = 2 * kFeed / KC;                    // chunks per pass
-    static constexpr int SBO = KC / 8 * 128;                      // bytes between 8-row groups
-    static constexpr int OPER = 256 * KC * 2;                     // bytes of one 256-row operand chunk
-    static constexpr bool A_LO = TERMS == 3;
-    static constexpr bool B_LO = TERMS >= 2;
-    static constexpr int A_STAGE = OPER * (A_LO ? 2 : 1);         // twiddle ring stage
-    static constexpr int B_STAGE = OPER * (B_LO ? 2 : 1);         // data ring stage
-    static constexpr int NA = 2;                                  // twiddle ring depth (a smaller shared-memory
-                                                                  // footprint leaves L1 for the raw loads)
-    static constexpr int NOCT = KC / 16;                          // 8-feed octets per chunk
-    static constexpr int NT = 288;                                // 8 producer warps + 1 MMA warp
-    static constexpr int NPROD = 256;                             // producer threads
-    static constexpr size_t SMEM = (size_t)NA * A_STAGE + 2ull * B_STAGE + 8 * 8 * 16 + 8 * (6 + 2 * NA);
+    static constexpr bool A_LO = TERMS == 3, B_LO = TERMS >= 2;
+    // data: yr and yi (hi, then lo) of a k-group side by side, 128 bytes each, and a pad that puts the
+    // eight lanes of a 128-bit store (two times, four k-groups, see the builders) in distinct bank
+    // groups; for three terms there is room for half of it, a store then takes two passes
+    static constexpr int B_LBO = (B_LO ? 512 : 256) + (A_LO ? 16 : 32), B_SBO = kTFeeds / 8 * B_LBO;
+    static constexpr int B_STAGE = 8 * B_SBO;                          // 64 times
+    static constexpr int STAGE = B_STAGE + (A_LO ? 2 * kTTw : 0);      // and the chunk's lo twiddles
+    static constexpr int NB = TERMS == 1 ? 6 : TERMS == 2 ? 5 : 3;     // ring stages
+    // arrivals on "stage full" in the first CTA: the builder warps of both CTAs; 3 terms: both
+    // CTAs' lo twiddles
+    static constexpr int FULL = 2 * kTBuild + (A_LO ? 2 : 0);
+    static constexpr int BARS = 3 * NB + 7;
+    static constexpr size_t SM_A = (size_t)kTNch * 2 * kTTw;           // 128 KB
+    static constexpr size_t SM_RING = (size_t)NB * STAGE;
+    static constexpr size_t SM_TW = 8 * 8 * 16;
+    static constexpr size_t SMEM = SM_A + SM_RING + SM_TW + 8 * BARS;
+    static_assert(SMEM + 128 <= 227 * 1024, "dynamic and static shared memory");
 };
 
-// Byte offset of element (row r, k) in a K-major operand chunk without
-// swizzle: 8 x 16-byte core matrices, k-groups 128 B apart, row groups SBO apart.
-template <int SBO>
-__device__ __forceinline__ int core_off(int r, int kgroup) {
-    return (r >> 3) * SBO + kgroup * 128 + (r & 7) * 16;
-}
+// instruction descriptor: kind::f16, A = B = F16, D = F32, both K-major, M = 256 (the pair), N = 128;
+// bit 13 negates A
+constexpr uint32_t kTIdesc = (1u << 4) | ((128u >> 3) << 17) | ((256u >> 4) << 24);
+constexpr uint32_t kTIdescNeg = kTIdesc | (1u << 13);
 
 // shared-memory matrix descriptor (no swizzle, version 1)
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
+__device__ __forceinline__ uint64_t tdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
 }
+__device__ __forceinline__ uint64_t adesc(uint32_t saddr) { return tdesc(saddr, kTALbo, kTASbo); }
 
-// instruction descriptor: kind::f16, A = B = F16, D = F32, both K-major, M = 128, N = 256
-constexpr uint32_t kIdesc = (1u << 4) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
-
-__device__ __forceinline__ void mma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t accum) {
+__device__ __forceinline__ void tmma(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(dtmem), "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accum)
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        :: "r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(accum)
         : "memory");
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(mbar)
-                 : "memory");
+// commit of this thread's outstanding MMAs to the same mbarrier in both CTAs
+__device__ __forceinline__ void tcommit(uint32_t mbar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 :: "r"(mbar), "h"((uint16_t)3) : "memory");
 }
 
-__device__ __forceinline__ uint32_t h2u(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
-
-// Producer tasks (t, octet): 8 feeds x 2 pols of every cylinder, one 16-byte
-// load each.  Lanes run over t so the B stores of a quarter warp fill one
-// 128-byte line.
-template <int TERMS>
-struct RawB {
-    static constexpr int TASKS = kUp * TcCfg<TERMS>::NOCT / TcCfg<TERMS>::NPROD;   // 2 (KC 64) or 1 (KC 32)
-    static_assert(TASKS >= 1, "fewer producer tasks than threads");
-    uint4 v[TASKS][kCyl];
-};
-
-// Lane bits 0-2 pick the time row within a group of 8, the next bits the
-// octet, the rest (with the warp and the task index) the group: one warp load
-// instruction then reads whole 32-byte sectors (all octets of 8 rows), and each
-// quarter warp stores 8 distinct 16-byte rows of a core matrix (no conflicts).
-template <int TERMS>
-__device__ __forceinline__ void task_of(int tid, int i, int& t, int& oct) {
-    using C = TcCfg<TERMS>;
-    constexpr int RPW = 32 / C::NOCT;                 // time rows per warp and task (8 or 16)
-    const int lane = tid & 31, warp = tid >> 5;
-    oct = (lane >> 3) % C::NOCT;
-    t = (lane & 7) + 8 * (lane / (8 * C::NOCT)) + RPW * warp + i * (C::NPROD / C::NOCT);
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
 }
-
-template <int TERMS>
-__device__ __forceinline__ void load_b(const Seg& sg, long long row0, int kc, int tid, RawB<TERMS>& r) {
-    using C = TcCfg<TERMS>;
-#pragma unroll
-    for (int i = 0; i < RawB<TERMS>::TASKS; ++i) {
-        int t, oct;
-        task_of<TERMS>(tid, i, t, oct);
-        const int n0 = (C::KC / 2) * kc + 8 * oct;
-        const uint8_t* rp = frame_row(sg, row0 + t) + 2 * n0;
-#pragma unroll
-        for (int c = 0; c < kCyl; ++c) r.v[i][c] = __ldg(reinterpret_cast<const uint4*>(rp + c * (kFeed * kPol)));
-    }
+__device__ __forceinline__ uint32_t cluster_id() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
+    return r;
 }
-
-// Build the B chunk: unpack, E-W toward beam j, split into FP16 hi (+ lo), and
-// store row t = (yr, yi) per feed and row 128 + t = (yi, -yr).
-template <int TERMS>
-__device__ __forceinline__ void build_b(const RawB<TERMS>& r, uint32_t sel, const EwW& w, unsigned char* bhi,
-                                        unsigned char* blo, int tid) {
-    using C = TcCfg<TERMS>;
-#pragma unroll
-    for (int i = 0; i < RawB<TERMS>::TASKS; ++i) {
-        int t, oct;
-        task_of<TERMS>(tid, i, t, oct);
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {           // feeds 4 half .. 4 half + 3 of the octet
-            cp y0, y1;                                    // SoA: (n, n + 2) and (n + 1, n + 3)
-#pragma unroll
-            for (int c = 0; c < kCyl; ++c) {
-                const uint32_t w0 = half ? r.v[i][c].z : r.v[i][c].x, w1 = half ? r.v[i][c].w : r.v[i][c].y;
-                const uint32_t g0 = __byte_perm(w0, 0u, sel), g1 = __byte_perm(w1, 0u, sel);
-                const float2 xi0 = nib2<0>(g0, g1), xr0 = nib2<1>(g0, g1);
-                const float2 xi1 = nib2<2>(g0, g1), xr1 = nib2<3>(g0, g1);
-                if (c == 0) {
-                    y0 = {xr0, xi0};
-                    y1 = {xr1, xi1};
-                } else {
-                    y0.re = fma2(xi0, w.NI[c - 1], fma2(xr0, w.R[c - 1], y0.re));
-                    y0.im = fma2(xr0, w.I[c - 1], fma2(xi0, w.R[c - 1], y0.im));
-                    y1.re = fma2(xi1, w.NI[c - 1], fma2(xr1, w.R[c - 1], y1.re));
-                    y1.im = fma2(xr1, w.I[c - 1], fma2(xi1, w.R[c - 1], y1.im));
-                }
-            }
-            const float yr[4] = {y0.re.x, y1.re.x, y0.re.y, y1.re.y};
-            const float yi[4] = {y0.im.x, y1.im.x, y0.im.y, y1.im.y};
-            __half2 hr[4];
-            uint32_t vre[4], vim[4];
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                hr[f] = __floats2half2_rn(yr[f], yi[f]);
-                vre[f] = h2u(hr[f]);
-                vim[f] = h2u(__floats2half2_rn(yi[f], -yr[f]));
-            }
-            const int kg = 2 * oct + half;
-            const int off_re = core_off<C::SBO>(t, kg), off_im = core_off<C::SBO>(128 + t, kg);
-            *reinterpret_cast<uint4*>(bhi + off_re) = make_uint4(vre[0], vre[1], vre[2], vre[3]);
-            *reinterpret_cast<uint4*>(bhi + off_im) = make_uint4(vim[0], vim[1], vim[2], vim[3]);
-            if constexpr (C::B_LO) {
-#pragma unroll
-                for (int f = 0; f < 4; ++f) {
-                    const float2 back = __half22float2(hr[f]);
-                    const float lr = yr[f] - back.x, li = yi[f] - back.y;
-                    vre[f] = h2u(__floats2half2_rn(lr, li));
-                    vim[f] = h2u(__floats2half2_rn(li, -lr));
-                }
-                *reinterpret_cast<uint4*>(blo + off_re) = make_uint4(vre[0], vre[1], vre[2], vre[3]);
-                *reinterpret_cast<uint4*>(blo + off_im) = make_uint4(vim[0], vim[1], vim[2], vim[3]);
-            }
-        }
-    }
+__device__ __forceinline__ uint32_t n_clusters() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
+    return r;
 }
-
-// One-thread bulk copy (TMA engine) of `bytes` into shared memory, completing
-// on an mbarrier that expects that many bytes.
+// address in CTA `cta` of the cluster of a local shared-memory address
+__device__ __forceinline__ uint32_t cta_addr(uint32_t a, uint32_t cta) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(cta));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Arrival on an mbarrier of any CTA of the cluster (shared::cluster address).  What it announces was
+// written for the asynchronous proxy (fence.proxy.async) or to tensor memory (tcgen05.fence), so no
+// cluster-wide release is needed; one here costs a memory barrier and an L1 invalidation per chunk
+// (1.83 ms per 4 x 49152-sample request against 1.30).
+__device__ __forceinline__ void arrive_cluster(uint32_t mbar) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" :: "r"(mbar) : "memory");
+}
+__device__ __forceinline__ void expect_tx(uint32_t mbar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(mbar), "r"(bytes) : "memory");
+}
+// bulk copy global -> this CTA's shared memory
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  :: "r"(dst), "l"(src), "r"(bytes), "r"(mbar) : "memory");
 }
+__device__ __forceinline__ uint32_t h2(float lo, float hi) {
+    const __half2 h = __floats2half2_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float2 unh2(uint32_t u) { return __half22float2(*reinterpret_cast<const __half2*>(&u)); }
 
-__device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(mbar), "r"(bytes) : "memory");
+struct RawT {
+    uint4 v[kCyl];
+};
+// the thread's 8 feeds x 2 pols of every cylinder at chunk kc (p: its row at feed octet 0 of chunk 0)
+__device__ __forceinline__ void load_raw(const uint8_t* p, int kc, RawT& r) {
+#pragma unroll
+    for (int c = 0; c < kCyl; ++c)
+        r.v[c] = __ldg(reinterpret_cast<const uint4*>(p + kc * (kTFeeds * kPol) + c * (kFeed * kPol)));
 }
 
+// One task: unpack 8 feeds of one time, E-W toward beam j in FP32, FP16 hi (+ lo) of yr and yi; dst is
+// the task's 16-byte place in yr, yi 128 bytes on, lo 256.
+template <int TERMS>
+__device__ __forceinline__ void build(const RawT& raw, const PolSel& ps, const EwW& w, unsigned char* dst) {
+    uint32_t vr[4], vi[4], lr[4], li[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {                        // feeds 2k, 2k + 1 as a SoA pair
+        cp y;
+#pragma unroll
+        for (int c = 0; c < kCyl; ++c) {
+            const uint32_t g = k == 0 ? raw.v[c].x : k == 1 ? raw.v[c].y : k == 2 ? raw.v[c].z : raw.v[c].w;
+            const uint32_t h = g >> 16;
+            const float2 xi = nibm(g, h, ps.mi, ps.si, ps.bi), xr = nibm(g, h, ps.mr, ps.sr, ps.br);
+            if (c == 0) {
+                y = {xr, xi};
+            } else {
+                y.re = fma2(xi, w.NI[c - 1], fma2(xr, w.R[c - 1], y.re));
+                y.im = fma2(xr, w.I[c - 1], fma2(xi, w.R[c - 1], y.im));
+            }
+        }
+        vr[k] = h2(y.re.x, y.re.y);
+        vi[k] = h2(y.im.x, y.im.y);
+        if constexpr (TERMS >= 2) {
+            const float2 br = unh2(vr[k]), bi = unh2(vi[k]);
+            lr[k] = h2(y.re.x - br.x, y.re.y - br.y);
+            li[k] = h2(y.im.x - bi.x, y.im.y - bi.y);
+        }
+    }
+    *reinterpret_cast<uint4*>(dst) = make_uint4(vr[0], vr[1], vr[2], vr[3]);
+    *reinterpret_cast<uint4*>(dst + 128) = make_uint4(vi[0], vi[1], vi[2], vi[3]);
+    if constexpr (TERMS >= 2) {
+        *reinterpret_cast<uint4*>(dst + 256) = make_uint4(lr[0], lr[1], lr[2], lr[3]);
+        *reinterpret_cast<uint4*>(dst + 384) = make_uint4(li[0], li[1], li[2], li[3]);
+    }
+}
 
-// MODE: 0 = detect and integrate, 1 = dump up-channelised voltages,
-//       2 = dump the N-S/E-W beams of the GEMM (stage dump), 3 = stall check
-//       (the MMA warp stays idle; the producers' bounded waits must run out).
-//
-// Warps 0-7 produce B chunks and run the up-channel passes out of TMEM; warp 8
-// streams the twiddle chunks (bulk copies, NA-deep ring) and issues the MMAs.
-// Chunks are numbered globally per CTA (item, pass, kc) so every barrier
-// phase is consumed exactly once in order.
+// MODE: 0 = detect and integrate, 1 = dump up-channelised voltages, 2 = dump the N-S/E-W beams of
+//       the GEMM, 3 = stall check (the MMA thread stays idle, so no stage is ever released and
+//       every other wait runs out against the launch's bound).
 template <int TERMS, int MODE>
-__global__ void __launch_bounds__(TcCfg<TERMS>::NT, 1) fused_tc_kernel(const __grid_constant__ Batch bt) {
+__global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_constant__ Batch bt) {
     using C = TcCfg<TERMS>;
-    constexpr int NA = C::NA;
-    extern __shared__ __align__(1024) unsigned char smem[];
+    constexpr int NB = C::NB;
+    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
-    unsigned char* a_ring = smem;                                  // NA x A_STAGE
-    unsigned char* b_ring = smem + NA * C::A_STAGE;                // 2 x B_STAGE
-    float4* tw_s = reinterpret_cast<float4*>(b_ring + 2 * C::B_STAGE);
-    uint64_t* mbar_s = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(tw_s) + 8 * 8 * 16);
+    unsigned char* ring = smem + C::SM_A;
+    float4* tw_s = reinterpret_cast<float4*>(ring + C::SM_RING);
+    uint64_t* mbar_s = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(tw_s) + C::SM_TW);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool producer = warp < 8;
-    const int ell = 32 * (warp & 3) + lane;           // TMEM lane (quarter = warp & 3)
-    const int hh = (warp >> 2) & 1;                    // bin half: m = ell + 128 hh
-    const int m = ell + 128 * hh;
+    const uint32_t rank = cluster_rank();
     const uint32_t smem0 = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
     const uint32_t bar0 = static_cast<uint32_t>(__cvta_generic_to_shared(&mbar_s[0]));
-    // barriers: bfull[2] (8 producer warps), bempty[2] (MMA commit), afull[NA] (bulk copy),
-    //           aempty[NA] (MMA commit), accfull (pass's last commit), tfree (8 producer warps)
-    auto bfull = [&](int s) { return bar0 + 8u * (uint32_t)s; };
-    auto bempty = [&](int s) { return bar0 + 8u * (uint32_t)(2 + s); };
-    auto afull = [&](int a) { return bar0 + 8u * (uint32_t)(4 + a); };
-    auto aempty = [&](int a) { return bar0 + 8u * (uint32_t)(4 + NA + a); };
-    const uint32_t accfull = bar0 + 8u * (uint32_t)(4 + 2 * NA);
-    const uint32_t tfree = accfull + 8u;
+    auto bfull = [&](int s) { return bar0 + 8u * (uint32_t)s; };               // first CTA: stage s of both CTAs
+    auto bempty = [&](int s) { return bar0 + 8u * (uint32_t)(NB + s); };       // MMA commit
+    auto lofull = [&](int s) { return bar0 + 8u * (uint32_t)(2 * NB + s); };   // second CTA's lo twiddles
+    auto accfull = [&](int b) { return bar0 + 8u * (uint32_t)(3 * NB + b); };  // last commit of a pass
+    auto tfree = [&](int b) { return bar0 + 8u * (uint32_t)(3 * NB + 2 + b); };    // first CTA: both CTAs' up-channel warps
+    const uint32_t afull = bar0 + 8u * (uint32_t)(3 * NB + 4);                 // this CTA's resident twiddles
+    const uint32_t aother = afull + 8u, adone = afull + 16u;
 
     if (warp == 0) {
         const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&tmem_base_s));
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" :: "r"(dst) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" :: "r"(dst) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
+        auto init = [](uint32_t b, uint32_t n) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(b), "r"(n) : "memory");
+        };
+        for (int i = 0; i < NB; ++i) {
+            init(bfull(i), C::FULL);
+            init(bempty(i), 1);
+            init(lofull(i), 1);
+        }
         for (int i = 0; i < 2; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" :: "r"(bfull(i)) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(bempty(i)) : "memory");
+            init(accfull(i), 1);
+            init(tfree(i), 2 * kTUp);
         }
-        for (int i = 0; i < NA; ++i) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(afull(i)) : "memory");
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(aempty(i)) : "memory");
-        }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(accfull) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 8;" :: "r"(tfree) : "memory");
+        init(afull, 1);
+        init(aother, 1);
+        init(adone, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         abort_s = 0;
     }
-    for (int i = tid; i < 64; i += C::NT) {
+    for (int i = tid; i < 64; i += kTThreads) {
         const int it = i >> 3, c = i & 7;
         const float2 w0 = bt.tw128[(2 * it * c) & (kUp - 1)];
         const float2 w1 = bt.tw128[((2 * it + 1) * c) & (kUp - 1)];
         tw_s[i] = make_float4(w0.x, w1.x, w0.y, w1.y);
     }
-    cta_sync();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    cluster_sync();                        // both CTAs' barriers exist before any remote arrival
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base_s;
-    constexpr int PASSES = kTds * kPol;
     const unsigned long long wlim = bt.wait_ns ? bt.wait_ns : kWaitNs;
-    // Tail items are split for the 1- and 3-term forms; the 2-term form, whose builders are
-    // the most register- and L1-bound, measured slower with the extra epilogue.
-    constexpr bool SPLIT = MODE == 0 && TERMS != 2;
-    const Units units = make_units(bt.n_items, (int)gridDim.x, SPLIT);
-    // this CTA's units are blockIdx.x + k gridDim.x: whole items first, then at most one half
-    auto my_count = [&](int n) { return n > (int)blockIdx.x ? (n - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0; };
-    const int n_my_whole = my_count(units.n_full), n_my_units = my_count(units.n_units);
+    const int pair = (int)cluster_id(), npairs = (int)n_clusters();
+    const PassUnits units = bt.units;
 
-    if (!producer) {
-        // ------------------------------ MMA / copy warp ------------------------------
-        // (MODE 3, the stall check: this warp stays idle, so no chunk is ever consumed)
+    if (warp == kTMma) {
+        // ------------------------------ twiddle loads and MMAs ------------------------------
         if (lane == 0 && MODE != 3) {
-            uint32_t p_bfull = 0, p_afull = 0, p_aempty = 0, p_tfree = 0;
-            long long c = 0;                                  // global chunk number
-            long long c_copy = 0;                             // next twiddle chunk to copy
-            const long long whole_chunks = (long long)n_my_whole * PASSES * C::NCH;
-            const long long total = whole_chunks + (long long)(n_my_units - n_my_whole) * (PASSES / 2) * C::NCH;
-            // twiddle image of the item that chunk cc belongs to; items only move forward,
-            // so the segment search resumes where the previous lookup stopped
-            int seg_cursor = 0;
-            auto image_of = [&](long long cc) {
-                const int k = cc < whole_chunks
-                                  ? (int)(cc / (PASSES * C::NCH))
-                                  : n_my_whole + (int)((cc - whole_chunks) / ((PASSES / 2) * C::NCH));
-                int it, ps0, ps1, half;
-                unit_of(units, (int)blockIdx.x + k * (int)gridDim.x, it, ps0, ps1, half);
-                while (seg_cursor + 1 < bt.n_segs && bt.segs[seg_cursor + 1].item_begin <= it) ++seg_cursor;
-                return bt.segs[seg_cursor].a_img;
-            };
-            auto issue_copy = [&](long long cc) {
-                const int a = (int)(cc % NA), kc = (int)(cc % C::NCH);
-                const unsigned char* a_hi = image_of(cc);
-                unsigned char* st = a_ring + a * C::A_STAGE;
-                mbar_expect(afull(a), C::A_STAGE);
-                bulk_g2s(smem0 + (uint32_t)(st - smem), a_hi + (size_t)kc * C::OPER, C::OPER, afull(a));
-                if constexpr (C::A_LO)
-                    bulk_g2s(smem0 + (uint32_t)(st + C::OPER - smem), a_hi + (size_t)(C::NCH + kc) * C::OPER,
-                             C::OPER, afull(a));
-            };
+            uint32_t p_bfull = 0, p_tfree = 0, p_a = 0, p_lo = 0;
+            const unsigned char* a_cur = nullptr;
+            uint32_t s = 0, pass = 0;
             bool ok = true;
-            // prologue: the first NA - 1 twiddle chunks
-            for (; c_copy < total && c_copy < NA - 1; ++c_copy) issue_copy(c_copy);
-            for (; c < total && ok; ++c) {
-                const int s = (int)(c & 1), a = (int)(c % NA), kc = (int)(c % C::NCH);
-                if (kc == 0 && c > 0) {
-                    // the previous pass's accumulator has been read by the producers
-                    if (!mbar_wait(tfree, p_tfree, wlim)) ok = false;
-                    p_tfree ^= 1u;
-                }
-                if (!mbar_wait(bfull(s), (p_bfull >> s) & 1u, wlim)) ok = false;
-                p_bfull ^= 1u << s;
-                if (!mbar_wait(afull(a), (p_afull >> a) & 1u, wlim)) ok = false;
-                p_afull ^= 1u << a;
-                if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t ahi = smem0 + (uint32_t)(a_ring + a * C::A_STAGE - smem), alo = ahi + C::OPER;
-                const uint32_t bhi = smem0 + (uint32_t)(b_ring + s * C::B_STAGE - smem), blo = bhi + C::OPER;
-#pragma unroll
-                for (int ks = 0; ks < C::KC / 16; ++ks) {
-#pragma unroll
-                    for (int mt = 0; mt < 2; ++mt) {
-                        const uint32_t d = tmem + mt * 256;
-                        const uint32_t aoff = mt * 16 * C::SBO + ks * 256;
-                        const uint64_t da = smem_desc(ahi + aoff, 128, C::SBO);
-                        const uint64_t db = smem_desc(bhi + ks * 256, 128, C::SBO);
-                        mma_f16(d, da, db, (kc | ks) ? 1u : 0u);
-                        if constexpr (C::B_LO) mma_f16(d, da, smem_desc(blo + ks * 256, 128, C::SBO), 1u);
-                        if constexpr (C::A_LO) mma_f16(d, smem_desc(alo + aoff, 128, C::SBO), db, 1u);
+            int seg_cursor = 0;
+            for (int un = pair; un < units.n_units && ok; un += npairs) {
+                int item, ps0, ps1;
+                pass_unit(units, un, item, ps0, ps1);
+                while (seg_cursor + 1 < bt.n_segs && bt.segs[seg_cursor + 1].item_begin <= item) ++seg_cursor;
+                const unsigned char* a_img = bt.segs[seg_cursor].a_img;
+                if (a_img != a_cur) {
+                    if (a_cur) {
+                        // the MMAs that read the old twiddles are complete before they are replaced
+                        if (rank == 0) tcommit(adone);
+                        ok = mbar_wait(adone, (p_a >> 1) & 1u, wlim) && ok;
+                        p_a ^= 2u;
                     }
-                }
-                mma_commit(bempty(s));
-                mma_commit(aempty(a));
-                if (kc == C::NCH - 1) mma_commit(accfull);
-                // refill: chunk c + NA - 1 goes into the stage of chunk c - 1 once its MMAs are done
-                if (c_copy < total) {
-                    if (c_copy >= NA) {
-                        const int ra = (int)(c_copy % NA);
-                        if (!mbar_wait(aempty(ra), (p_aempty >> ra) & 1u, wlim)) ok = false;
-                        p_aempty ^= 1u << ra;
+                    expect_tx(afull, (uint32_t)C::SM_A);
+#pragma unroll 1
+                    for (int kc = 0; kc < kTNch; ++kc)
+                        bulk_g2s(smem0 + (uint32_t)(kc * 2 * kTTw), a_img + (size_t)(kc * 2 + (int)rank) * (2 * kTTw),
+                                 2 * kTTw, afull);
+                    ok = mbar_wait(afull, p_a & 1u, wlim) && ok;
+                    if (rank == 1) {
+                        arrive_cluster(cta_addr(aother, 0));
+                    } else {
+                        ok = mbar_wait(aother, p_a & 1u, wlim) && ok;
                     }
-                    issue_copy(c_copy);
-                    ++c_copy;
+                    p_a ^= 1u;
+                    a_cur = a_img;
                 }
-                if (abort_s) ok = false;
+                for (int ps = ps0; ps < ps1 && ok; ++ps, ++pass) {
+                    if (rank == 1 && !C::A_LO) continue;
+                    const uint32_t buf = pass & 1u;
+                    if (rank == 0 && pass >= 2) {
+                        // the up-channel warps of both CTAs have read this accumulator half (pass - 2)
+                        ok = mbar_wait(tfree((int)buf), (p_tfree >> buf) & 1u, wlim) && ok;
+                        p_tfree ^= 1u << buf;
+                    }
+                    for (int kc = 0; kc < kTNch && ok; ++kc) {
+                        if (rank == 1) {
+                            // 3 terms: this CTA's lo twiddles of the stage have landed
+                            ok = mbar_wait(lofull((int)s), (p_lo >> s) & 1u, wlim);
+                            p_lo ^= 1u << s;
+                            if (ok) arrive_cluster(cta_addr(bfull((int)s), 0));
+                        } else {
+                            ok = mbar_wait(bfull((int)s), (p_bfull >> s) & 1u, wlim) && ok;
+                            p_bfull ^= 1u << s;
+                            if (!ok) break;
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint32_t a0 = smem0 + (uint32_t)(kc * 2 * kTTw);
+                            const uint32_t b0 = smem0 + (uint32_t)C::SM_A + s * (uint32_t)C::STAGE;
+                            const uint32_t re = tmem + 256u * buf, im = re + 128u;
+                            auto bdesc = [](uint32_t saddr) { return tdesc(saddr, C::B_LBO, C::B_SBO); };
+#pragma unroll
+                            for (int ks = 0; ks < kTFeeds / 16; ++ks) {
+                                const uint64_t c = adesc(a0 + ks * 2 * kTALbo), sn = adesc(a0 + kTTw + ks * 2 * kTALbo);
+                                const uint32_t bk = b0 + ks * 2 * C::B_LBO;
+                                const uint64_t yr = bdesc(bk), yi = bdesc(bk + 128);
+                                const uint32_t more = (kc | ks) ? 1u : 0u;
+                                tmma(re, c, yr, kTIdesc, more);
+                                tmma(im, c, yi, kTIdesc, more);
+                                tmma(re, sn, yi, kTIdesc, 1u);
+                                tmma(im, sn, yr, kTIdescNeg, 1u);
+                                if constexpr (C::B_LO) {
+                                    const uint64_t zr = bdesc(bk + 256), zi = bdesc(bk + 384);
+                                    tmma(re, c, zr, kTIdesc, 1u);
+                                    tmma(im, c, zi, kTIdesc, 1u);
+                                    tmma(re, sn, zi, kTIdesc, 1u);
+                                    tmma(im, sn, zr, kTIdescNeg, 1u);
+                                }
+                                if constexpr (C::A_LO) {
+                                    const uint32_t l0 = b0 + (uint32_t)C::B_STAGE;
+                                    const uint64_t cl = adesc(l0 + ks * 2 * kTALbo), sl = adesc(l0 + kTTw + ks * 2 * kTALbo);
+                                    tmma(re, cl, yr, kTIdesc, 1u);
+                                    tmma(im, cl, yi, kTIdesc, 1u);
+                                    tmma(re, sl, yi, kTIdesc, 1u);
+                                    tmma(im, sl, yr, kTIdescNeg, 1u);
+                                }
+                            }
+                            tcommit(bempty((int)s));
+                            if (kc == kTNch - 1) tcommit(accfull((int)buf));
+                        }
+                        if (++s == (uint32_t)NB) s = 0;
+                    }
+                    if (*(volatile int*)&abort_s) ok = false;
+                }
             }
+            // every issued MMA is complete before shared and tensor memory are released
+            if (rank == 0) tcommit(adone);
+            if (!mbar_wait(adone, (p_a >> 1) & 1u, wlim)) ok = false;
             if (!ok) abort_s = 1;
         }
         __syncwarp();
-    } else {
-        // ------------------------------ producer warps ------------------------------
-        const uint32_t tlane = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + hh * 256;
-        uint32_t p_bempty = 0, p_acc = 0;
-        long long c = 0;
-        bool ok = true;
-        for (int k = 0; k < n_my_units && ok; ++k) {
-            int item, ps0, ps1, half;
-            unit_of(units, (int)blockIdx.x + k * (int)gridDim.x, item, ps0, ps1, half);
-            int sgi = 0;
+    } else if (warp < kTBuild) {
+        // ------------------------------ builders ------------------------------
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kTRegBuild) : "memory");
+        // lane bits 0-1 take the four feed octets of a chunk, bits 2-4 eight times: a quarter warp loads 64
+        // contiguous bytes of two rows (lanes on eight different lines at one offset instead take a
+        // pass of the L1 data banks each: 1.29 ms per 4 x 49152-sample request against 1.16)
+        const int t = 64 * (int)rank + 8 * warp + (lane >> 2), oct = lane & 3;
+        unsigned char* dst0 = ring + warp * C::B_SBO + oct * C::B_LBO + (lane >> 2) * 16;
+        const uint32_t full0 = cta_addr(bar0, 0);                      // the first CTA's bfull(0)
+        // this thread's row at chunk 0 of pass ps of an item
+        auto row_of = [&](const Seg& sg, int F, int ps) {
+            return frame_row(sg, (long long)F * kFrame + (ps >> 1) * kUp + t) + 16 * oct;
+        };
+        uint32_t p_bempty = 0, s = 0;
+        bool wrapped = false, ok = true;
+        int sgi = 0;
+        for (int un = pair; un < units.n_units && ok; un += npairs) {
+            int item, ps0, ps1;
+            pass_unit(units, un, item, ps0, ps1);
             while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
             const Seg& sg = bt.segs[sgi];
             const int local = item - sg.item_begin;
             const int F = local >> 2, j = local & 3;
             EwW w;
             load_ew_frame(sg, bt.ew, F, j, w);
-            float2 acc[kSub];
-#pragma unroll
-            for (int q = 0; q < kSub; ++q) acc[q] = make_float2(0.f, 0.f);
-            RawB<TERMS> raw;
-            load_b<TERMS>(sg, (long long)F * kFrame + (ps0 >> 1) * kUp, 0, tid, raw);
+            const uint8_t* p = row_of(sg, F, ps0);
+            RawT raw;
+            load_raw(p, 0, raw);
             for (int ps = ps0; ps < ps1 && ok; ++ps) {
-                const int blk = ps >> 1, pol = ps & 1;
-                const uint32_t sel = 0x4400u | ((2u + pol) << 4) | (uint32_t)pol;
-                for (int kc = 0; kc < C::NCH && ok; ++kc, ++c) {
-                    const int s = (int)(c & 1);
-                    if (c >= 2) {
-                        if (!mbar_wait(bempty(s), (p_bempty >> s) & 1u, wlim)) ok = false;
+                const PolSel sel = pol_sel(ps & 1);
+                // four chunks per loop body: the raw rows alternate between registers without copies
+                // (1.16 ms with a copy per chunk, 1.02 ms without)
+#pragma unroll 4
+                for (int kc = 0; kc < kTNch; ++kc) {
+                    if (wrapped) {
+                        // the MMAs have read stage s in both CTAs
+                        if (!mbar_wait(bempty((int)s), (p_bempty >> s) & 1u, wlim)) ok = false;
                         p_bempty ^= 1u << s;
                     }
-                    unsigned char* sb_hi = b_ring + s * C::B_STAGE;
-                    unsigned char* sb_lo = sb_hi + C::OPER;
-                    RawB<TERMS> cur = raw;
-                    const bool last = kc + 1 == C::NCH;
-                    if (!last || ps + 1 < ps1) {
-                        const int nblk = last ? ((ps + 1) >> 1) : blk;
-                        load_b<TERMS>(sg, (long long)F * kFrame + nblk * kUp, last ? 0 : kc + 1, tid, raw);
+                    // the warp stops as one (a wait expired in any lane)
+                    if (!__all_sync(0xffffffffu, ok)) {
+                        ok = false;
+                        break;
                     }
-                    build_b<TERMS>(cur, sel, w, sb_hi, sb_lo, tid);
+                    if constexpr (C::A_LO) {
+                        if (tid == 0) {
+                            // the chunk's lo twiddles (second half of the image) into the stage
+                            const uint32_t bar = rank == 0 ? bfull((int)s) : lofull((int)s);
+                            expect_tx(bar, 2 * kTTw);
+                            bulk_g2s(smem0 + (uint32_t)C::SM_A + s * (uint32_t)C::STAGE + (uint32_t)C::B_STAGE,
+                                     sg.a_img + 2 * C::SM_A + (size_t)(kc * 2 + (int)rank) * (2 * kTTw), 2 * kTTw, bar);
+                        }
+                    }
+                    const RawT cur = raw;
+                    if (kc + 1 < kTNch) {
+                        load_raw(p, kc + 1, raw);
+                    } else if (ps + 1 < ps1) {
+                        p = row_of(sg, F, ps + 1);
+                        load_raw(p, 0, raw);
+                    }
+                    build<TERMS>(cur, sel, w, dst0 + s * (uint32_t)C::STAGE);
+                    // the generic-proxy stores are visible to the tensor cores
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bfull(s));
-                    if (abort_s) ok = false;
+                    if (lane == 0) arrive_cluster(full0 + 8u * s);
+                    if (++s == (uint32_t)NB) {
+                        s = 0;
+                        wrapped = true;
+                    }
                 }
-                if (!ok) break;
-                if (!mbar_wait(accfull, p_acc, wlim)) ok = false;
-                p_acc ^= 1u;
-                if (!ok) break;
+                if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;   // the warp stops as one
+            }
+        }
+        if (!ok) abort_s = 1;
+    } else {
+        // ------------------------------ up-channel warps ------------------------------
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(kTRegUp) : "memory");
+        const int q4 = warp & 3;                                     // tensor-memory lane quarter
+        const int ell = 32 * q4 + lane, m = 128 * (int)rank + ell;   // this thread's bin
+        const uint32_t free0 = cta_addr(tfree(0), 0);
+        uint32_t p_acc = 0, pass = 0;
+        bool ok = true;
+        int sgi = 0;
+        for (int un = pair; un < units.n_units && ok; un += npairs) {
+            int item, ps0, ps1;
+            pass_unit(units, un, item, ps0, ps1);
+            while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
+            const Seg& sg = bt.segs[sgi];
+            const int local = item - sg.item_begin;
+            const int F = local >> 2, j = local & 3;
+            const bool whole = ps1 - ps0 == kTds * kPol;
+            // sums of the item's passes of each polarisation
+            float acc0[kSub], acc1[kSub];
+#pragma unroll
+            for (int q = 0; q < kSub; ++q) acc0[q] = acc1[q] = 0.f;
+            for (int ps = ps0; ps < ps1 && ok; ++ps, ++pass) {
+                const uint32_t buf = pass & 1u;
+                const uint32_t base = tmem + (static_cast<uint32_t>(32 * q4) << 16) + 256u * buf;
+                if (!mbar_wait(accfull((int)buf), (p_acc >> buf) & 1u, wlim)) ok = false;
+                p_acc ^= 1u << buf;
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    break;
+                }
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                float2 pw[kSub];
+#pragma unroll
+                for (int q = 0; q < kSub; ++q) pw[q] = make_float2(0.f, 0.f);
+                float2* dump = MODE == 1 || MODE == 2
+                                   ? bt.dump + ((((long long)(F * kTds + (ps >> 1)) * kPol + (ps & 1)) * kEw + j) * kNs + m) * kUp
+                                   : nullptr;
                 if constexpr (MODE == 2) {
-                    float2* d = bt.dump + ((((long long)(F * kTds + blk) * kPol + pol) * kEw + j) * kNs + m) * kUp;
                     for (int c4 = 0; c4 < 4; ++c4) {
                         float re[32], im[32];
-                        tmem_ld32f(tlane + 32 * c4, re);
-                        tmem_ld32f(tlane + 128 + 32 * c4, im);
-                        for (int b = 0; b < 32; ++b) d[32 * c4 + b] = make_float2(re[b], im[b]);
+                        tmem_ld32f(base + 32 * c4, re);
+                        tmem_ld32f(base + 128 + 32 * c4, im);
+                        for (int b = 0; b < 32; ++b) dump[32 * c4 + b] = make_float2(re[b], im[b]);
                     }
                 } else {
-                    upchan_pass1_split(tlane, tw_s, 0, 1);
+                    upchan_pass1_split(base, tw_s);
                     tmem_wait_st();
-                    upchan_pass2_split(tlane, acc,
-                                       MODE == 1 ? bt.dump + ((((long long)(F * kTds + blk) * kPol + pol) * kEw + j) * kNs + m) * kUp
-                                                 : nullptr,
-                                       0, 1);
+                    upchan_pass2_split(base, pw, MODE == 1 ? dump : nullptr);
                 }
-                // this warp's TMEM reads of the pass are done
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) mbar_arrive(tfree);
-                if constexpr (SPLIT) {
-                    if (half < 0 && ps == PASSES / 2 - 1) {
-                        // whole item: H0 (passes 0-2) parks in this CTA's slot (coalesced)
-                        // until H1 is done
-                        float* pk = bt.park + (size_t)blockIdx.x * (kSub * kNs) + m;
+                if (lane == 0) arrive_cluster(free0 + 8u * buf);
+                if constexpr (MODE == 0) {
+                    if (whole) {
 #pragma unroll
                         for (int q = 0; q < kSub; ++q) {
-                            pk[q * kNs] = acc[q].x + acc[q].y;
-                            acc[q] = make_float2(0.f, 0.f);
+                            const float v = pw[q].x + pw[q].y;
+                            if (ps & 1)
+                                acc1[q] += v;
+                            else
+                                acc0[q] += v;
+                        }
+                    } else {
+                        // part of an item: publish the pass; the thread that completes the six adds them
+                        const int slot = item - units.n_full;
+                        float* o = bt.part + ((size_t)slot * (kTds * kPol) + ps) * (kSub * kNs) + m;
+#pragma unroll
+                        for (int q = 0; q < kSub; ++q) o[q * kNs] = pw[q].x + pw[q].y;
+                        if (add_passes(bt.part_tok + (size_t)slot * kNs + m, bt.epoch, 1)) {
+                            const float* in = bt.part + (size_t)slot * (kTds * kPol) * (kSub * kNs) + m;
+                            float* out = sg.out + (long long)(kNs * j + m) * sg.beam_stride + F;
+#pragma unroll
+                            for (int q = 0; q < kSub; ++q) {
+                                float v[kTds * kPol];
+#pragma unroll
+                                for (int k = 0; k < kTds * kPol; ++k) v[k] = __ldcg(in + (size_t)k * (kSub * kNs) + q * kNs);
+                                out[(long long)q * sg.sub_stride] = ((v[0] + v[2]) + v[4]) + ((v[1] + v[3]) + v[5]);
+                            }
                         }
                     }
                 }
+                if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;   // the warp stops as one
             }
             if constexpr (MODE == 0) {
-                if (ok) {
-                    // forms that split items: each output is H0 + H1 (H = the two fine channels
-                    // of a pair added first), split or not; the 2-term form: the running sum
-                    float h1[kSub];
+                if (whole && ok) {
+                    float* out = sg.out + (long long)(kNs * j + m) * sg.beam_stride + F;
 #pragma unroll
-                    for (int q = 0; q < kSub; ++q) h1[q] = acc[q].x + acc[q].y;
-                    float* o = sg.out + (long long)(kNs * j + m) * sg.beam_stride + F;
-                    if (!SPLIT) {
-#pragma unroll
-                        for (int q = 0; q < kSub; ++q) o[(long long)q * sg.sub_stride] = h1[q];
-                    } else if (half < 0) {
-                        const float* pk = bt.park + (size_t)blockIdx.x * (kSub * kNs) + m;
-                        float h0[kSub];
-#pragma unroll
-                        for (int q = 0; q < kSub; ++q) h0[q] = pk[q * kNs];
-#pragma unroll
-                        for (int q = 0; q < kSub; ++q) o[(long long)q * sg.sub_stride] = h0[q] + h1[q];
-                    } else {
-                        const int slot = item - units.n_full;
-                        float* mine = bt.part + ((size_t)slot * 2 + half) * (kSub * kNs) + m;
-#pragma unroll
-                        for (int q = 0; q < kSub; ++q) mine[q * kNs] = h1[q];
-                        if (second_half(bt.part_tok + (size_t)slot * kNs + m, bt.epoch, half)) {
-                            const float* other = bt.part + ((size_t)slot * 2 + (half ^ 1)) * (kSub * kNs) + m;
-                            float h0[kSub];
-#pragma unroll
-                            for (int q = 0; q < kSub; ++q) h0[q] = __ldcg(other + q * kNs);
-#pragma unroll
-                            for (int q = 0; q < kSub; ++q) o[(long long)q * sg.sub_stride] = h0[q] + h1[q];
-                        }
-                    }
+                    for (int q = 0; q < kSub; ++q) out[(long long)q * sg.sub_stride] = acc0[q] + acc1[q];
                 }
             }
         }
         if (!ok) abort_s = 1;
     }
 
-    cta_sync();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    // both CTAs are done with each other's barriers and, in a run that completed, with the MMAs
+    cluster_sync();
     if (abort_s && tid == 0 && bt.status) atomicExch(bt.status, 1);
     if (warp == 0) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" :: "r"(tmem) : "memory");
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" :: "r"(tmem) : "memory");
     }
 }
 
+// Once per device and kernel: the register split must fit in what the kernel was launched with
+// (else the up-channel warps' increase could never be granted: such a build is refused), and the
+// shared-memory size is set.
 template <int TERMS, int MODE>
-cudaError_t launch_tc(const Batch& b, int grid, cudaStream_t s) {
+cudaError_t launch_tc(const Batch& b, int pairs, cudaStream_t s) {
     if (b.n_items <= 0) return cudaSuccess;
-    // the detecting 1- and 3-term kernels park and split: they need the plan's buffers
-    if (MODE == 0 && TERMS != 2 && (!b.part || !b.park || !b.part_tok || grid > 2 * kMaxSplit))
-        return cudaErrorInvalidValue;
-    const int smem = (int)TcCfg<TERMS>::SMEM;
-    // shared-memory opt-in, once per device (the outcome is kept and returned on every launch)
+    if (pairs < 1 || (b.units.g < kTds * kPol && (!b.part || !b.part_tok))) return cudaErrorInvalidValue;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -491,35 +557,58 @@ cudaError_t launch_tc(const Batch& b, int grid, cudaStream_t s) {
     static std::once_flag once[kMaxDevices];
     static cudaError_t result[kMaxDevices];
     std::call_once(once[dev], [&] {
-        result[dev] = cudaFuncSetAttribute(fused_tc_kernel<TERMS, MODE>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncAttributes fa;
+        cudaError_t r = cudaFuncGetAttributes(&fa, fused_tc_kernel<TERMS, MODE>);
+        if (r == cudaSuccess && kTBuild * kTRegBuild + kTUp * kTRegUp > kTMma * fa.numRegs) r = cudaErrorInvalidConfiguration;
+        if (r == cudaSuccess)
+            r = cudaFuncSetAttribute(fused_tc_kernel<TERMS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)TcCfg<TERMS>::SMEM);
+        result[dev] = r;
     });
     if (result[dev] != cudaSuccess) return result[dev];
-    fused_tc_kernel<TERMS, MODE><<<grid, TcCfg<TERMS>::NT, smem, s>>>(b);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    cfg.blockDim = dim3(kTThreads);
+    cfg.dynamicSmemBytes = TcCfg<TERMS>::SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, fused_tc_kernel<TERMS, MODE>, b);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
 }  // namespace
 
 size_t tc_a_bytes(int terms) {
-    const size_t one = (size_t)kNs * 2 * kFeed * 2;              // 256 rows x 512 K x FP16
+    const size_t one = (size_t)kNs * 2 * kFeed * 2;              // 256 rows x (C, S) x 256 feeds x FP16
     return terms == 3 ? 2 * one : one;
 }
 
-int tc_chunk_k(int terms) { return terms == 3 ? TcCfg<3>::KC : terms == 2 ? TcCfg<2>::KC : TcCfg<1>::KC; }
+size_t tc_a_offset(int m, int n, int part) {
+    // chunk, CTA of the pair, C or S block; 8-row x 16-byte core matrices
+    const size_t block = (((size_t)(n / kTFeeds) * 2 + m / 128) * 2 + part) * kTTw;
+    const int r = m % 128, k = n % kTFeeds;
+    return block + (size_t)(r / 8) * kTASbo + (k / 8) * kTALbo + (r % 8) * 16 + (k % 8) * 2;
+}
 
-cudaError_t fused_tc_launch(const Batch& b, int terms, int mode, int grid, cudaStream_t s) {
+cudaError_t fused_tc_launch(const Batch& b, int terms, int mode, int pairs, cudaStream_t s) {
     switch (terms * 10 + mode) {
-        case 10: return launch_tc<1, 0>(b, grid, s);
-        case 11: return launch_tc<1, 1>(b, grid, s);
-        case 12: return launch_tc<1, 2>(b, grid, s);
-        case 13: return launch_tc<1, 3>(b, grid, s);
-        case 20: return launch_tc<2, 0>(b, grid, s);
-        case 21: return launch_tc<2, 1>(b, grid, s);
-        case 22: return launch_tc<2, 2>(b, grid, s);
-        case 30: return launch_tc<3, 0>(b, grid, s);
-        case 31: return launch_tc<3, 1>(b, grid, s);
-        case 32: return launch_tc<3, 2>(b, grid, s);
+        case 10: return launch_tc<1, 0>(b, pairs, s);
+        case 11: return launch_tc<1, 1>(b, pairs, s);
+        case 12: return launch_tc<1, 2>(b, pairs, s);
+        case 13: return launch_tc<1, 3>(b, pairs, s);
+        case 20: return launch_tc<2, 0>(b, pairs, s);
+        case 21: return launch_tc<2, 1>(b, pairs, s);
+        case 22: return launch_tc<2, 2>(b, pairs, s);
+        case 30: return launch_tc<3, 0>(b, pairs, s);
+        case 31: return launch_tc<3, 1>(b, pairs, s);
+        case 32: return launch_tc<3, 2>(b, pairs, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -135,17 +135,14 @@ struct bf_plan_s {
     std::vector<uint64_t> slot_used;          // LRU clock of the slot's last lookup
     uint64_t lru_clock = 0;
     int terms = 0;                            // tensor-core GEMM terms (0: FP32 FFT form)
-    bool dft512 = false;                      // BF_TC_DFT512: all 512 rows, the clamp at the output
-    int16_t* d_inv = nullptr;                 // 512-row form: [table_cap][kInvLen] bin -> beams lists
-    unsigned char* d_a512 = nullptr;          // 512-row form: the one FP16 image of the 512 x 512 DFT matrix
+    bool dft512 = false;                      // BF_TC_DFT512: the 1-term kernel, no stage dumps
     std::vector<unsigned char*> atc_blocks;   // [kTcBlock][tc_a_bytes(terms)] FP16 twiddle images each
     int* h_status = nullptr;                  // mapped status word written by kernels
     int* d_delays = nullptr;                  // dedispersion delay table (grown on demand)
     size_t delays_cap = 0;
     int* d_status = nullptr;
-    float* d_part = nullptr;                  // FP32 form: halves of split items (see Batch::part)
+    float* d_part = nullptr;                  // sums of split items (see Batch::part)
     unsigned long long* d_part_tok = nullptr;
-    float* d_park = nullptr;                  // tensor-core form: per-CTA first halves (see Batch::park)
     unsigned long long launches = 0;          // launch epochs handed to the kernels
 
     std::mutex mu;
@@ -234,42 +231,33 @@ int track_alloc(bf_plan_s* p, size_t bytes, TrackBuf* out) {
     return BF_OK;
 }
 
-// Tensor-core twiddle image of `rows` rows: A[m][2n] = cos, A[m][2n+1] = sin
-// of 2 pi n L(m) / 512 (the clamped rows of the zero-padded DFT, Eq. 1, with
-// the clamp table as L; all 512 rows of the DFT matrix with L(m) = m), FP16
-// hi (and lo = A - hi), laid out chunk by chunk exactly as the kernel's shared
-// memory operand: 8-row x 16-byte core matrices, k-groups 128 B apart, row
-// groups KC/8 * 128 B apart.
-void tc_image(int terms, const int32_t* lut, int rows, std::vector<__half>& img) {
-    const int KC = tc_chunk_k(terms);
-    const size_t oper = (size_t)rows * KC;                // halves per chunk
-    const size_t nch = 2 * kFeed / KC;
-    const size_t one = oper * nch;
-    img.assign(terms == 3 ? 2 * one : one, __float2half(0.f));
-    for (int m = 0; m < rows; ++m)
+// Tensor-core twiddle image of one table: C[m][n] = cos and S[m][n] = sin of 2 pi n L(m) / 512 (the
+// clamped rows of the zero-padded DFT, Eq. 1), FP16 hi (for three terms also lo = the rest), laid out
+// as the kernel's shared memory operand.  Only 512 angles occur.
+void tc_image(int terms, const int32_t* lut, std::vector<unsigned char>& img) {
+    struct Entry {
+        __half hi[2], lo[2];
+    };
+    std::vector<Entry> tab(kBins);
+    for (int e = 0; e < kBins; ++e) {
+        const double th = 2.0 * kPi * (double)e / kBins;
+        const double v[2] = {std::cos(th), std::sin(th)};
+        for (int c = 0; c < 2; ++c) {
+            tab[e].hi[c] = __double2half(v[c]);
+            tab[e].lo[c] = __double2half(v[c] - (double)__half2float(tab[e].hi[c]));
+        }
+    }
+    const size_t one = tc_a_bytes(1);
+    img.assign(tc_a_bytes(terms), 0);
+    for (int m = 0; m < kNs; ++m)
         for (int n = 0; n < kFeed; ++n) {
-            const long long e = ((long long)n * lut[m]) % kBins;
-            const double th = 2.0 * kPi * (double)e / kBins;
-            const double v[2] = {std::cos(th), std::sin(th)};
+            const Entry& e = tab[((long long)n * lut[m]) % kBins];
             for (int c = 0; c < 2; ++c) {
-                const int kg = 2 * n + c;
-                const size_t kc = kg / KC, k = kg % KC;
-                const size_t off = kc * oper + ((size_t)(m >> 3) * (KC / 8) + (k >> 3)) * 64 + (m & 7) * 8 + (k & 7);
-                const __half hi = __double2half(v[c]);
-                img[off] = hi;
-                if (terms == 3) img[one + off] = __double2half(v[c] - (double)__half2float(hi));
+                const size_t off = tc_a_offset(m, n, c);
+                std::memcpy(&img[off], &e.hi[c], sizeof e.hi[c]);
+                if (terms == 3) std::memcpy(&img[one + off], &e.lo[c], sizeof e.lo[c]);
             }
         }
-}
-
-// The clamp (Eq. 1) read backwards for the 512-row form: inv[k] = the first beam m with
-// L(m) = k and inv[512 + m] = the next beam after m with the same bin (-1 ends a list).
-void inverse_clamp(const int32_t* lut, int16_t* inv) {
-    for (int i = 0; i < kInvLen; ++i) inv[i] = -1;
-    for (int m = kNs - 1; m >= 0; --m) {
-        inv[kBins + m] = inv[lut[m]];
-        inv[lut[m]] = (int16_t)m;
-    }
 }
 
 uint64_t freq_key(double f) {
@@ -385,7 +373,6 @@ void gather_order(const int32_t* lut, int16_t* order) {
 
 const unsigned char* tc_image(const bf_plan_s* p, int slot) {
     if (!p->terms) return nullptr;
-    if (p->dft512) return p->d_a512;
     return p->atc_blocks[slot / kTcBlock] + (size_t)(slot % kTcBlock) * tc_a_bytes(p->terms);
 }
 
@@ -418,7 +405,7 @@ int table_for(bf_plan_s* p, double f, int* idx) {
     ew_table(p, f, ew);
     int16_t order[kNs];
     gather_order(lut, order);
-    if (p->terms && !p->dft512) {
+    if (p->terms) {
         const int blk = n / kTcBlock;
         if (!p->atc_blocks[blk]) CK(cudaMalloc(&p->atc_blocks[blk], (size_t)kTcBlock * tc_a_bytes(p->terms)));
     }
@@ -427,15 +414,10 @@ int table_for(bf_plan_s* p, double f, int* idx) {
     CK(cudaMemcpy(p->d_lut + (size_t)n * kNs, lut16, sizeof lut16, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(p->d_order + (size_t)n * kNs, order, sizeof order, cudaMemcpyHostToDevice));
     CK(cudaMemcpy(p->d_ew + (size_t)n * kEw * kCyl, ew, sizeof ew, cudaMemcpyHostToDevice));
-    if (p->dft512) {
-        int16_t inv[kInvLen];
-        inverse_clamp(lut, inv);
-        CK(cudaMemcpy(p->d_inv + (size_t)n * kInvLen, inv, sizeof inv, cudaMemcpyHostToDevice));
-    } else if (p->terms) {
-        std::vector<__half> img;
-        tc_image(p->terms, lut, kNs, img);
-        CK(cudaMemcpy(const_cast<unsigned char*>(tc_image(p, n)), img.data(), img.size() * sizeof(__half),
-                      cudaMemcpyHostToDevice));
+    if (p->terms) {
+        std::vector<unsigned char> img;
+        tc_image(p->terms, lut, img);
+        CK(cudaMemcpy(const_cast<unsigned char*>(tc_image(p, n)), img.data(), img.size(), cudaMemcpyHostToDevice));
     }
     if (n == p->n_slots) ++p->n_slots;
     p->slot_key[n] = key;
@@ -476,7 +458,6 @@ Batch make_batch(const bf_plan_s* p) {
     Batch b;
     std::memset(&b, 0, sizeof b);
     b.lut = p->d_lut;
-    b.inv = p->d_inv;
     b.order = p->d_order;
     b.ew = p->d_ew;
     b.twl = p->d_twl;
@@ -484,7 +465,6 @@ Batch make_batch(const bf_plan_s* p) {
     b.status = p->d_status;
     b.part = p->d_part;
     b.part_tok = p->d_part_tok;
-    b.park = p->d_park;
     return b;
 }
 
@@ -655,18 +635,14 @@ int launch_jobs(bf_plan_s* p, std::vector<Job>& jobs, size_t bytes) {
     CK(cudaEventRecord(ev_start.ev, p->stream));
     for (auto& bb : batches) {
         bb.epoch = ++p->launches;
-        // a launch of at most half a grid of items runs every item as two halves on two CTAs
-        // (the 2-term tensor-core form never splits)
         cudaError_t e;
-        if (p->dft512) {
-            e = fused_tc_dft512_launch(bb, p->stream);
-        } else if (p->terms == 1) {
-            // the 1-term form runs on CTA pairs, one item per pair at a time
-            e = fused_tc_pair_launch(bb, 2 * std::min(p->grid / 2, bb.n_items), p->stream);
+        if (p->terms) {
+            bb.units = pass_units(bb.n_items, p->grid / 2, bb.part != nullptr);
+            e = fused_tc_launch(bb, p->terms, 0, std::min(p->grid / 2, bb.units.n_units), p->stream);
         } else {
-            int grid = std::min(p->grid, bb.n_items);
-            if (p->terms != 2 && 2 * bb.n_items <= p->grid) grid = 2 * bb.n_items;
-            e = p->terms ? fused_tc_launch(bb, p->terms, 0, grid, p->stream) : fused_fp32_launch(bb, grid, p->stream);
+            // a launch of at most half a grid of items runs every item as two halves on two CTAs
+            const int grid = 2 * bb.n_items <= p->grid ? 2 * bb.n_items : std::min(p->grid, bb.n_items);
+            e = fused_fp32_launch(bb, grid, p->stream);
         }
         if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
     }
@@ -900,15 +876,6 @@ int bf_plan(const bf_config* cfg, bf_plan_t* out) {
     CK(cudaMalloc(&p->d_ew, (size_t)p->table_cap * kEw * kCyl * sizeof(float2)));
     CK(cudaMalloc(&p->d_twl, kLaneTwLen * sizeof(float2)));
     CK(cudaMalloc(&p->d_tw128, kUp * sizeof(float2)));
-    if (p->dft512) {
-        CK(cudaMalloc(&p->d_inv, (size_t)p->table_cap * kInvLen * sizeof(int16_t)));
-        int32_t all[kBins];
-        for (int k = 0; k < kBins; ++k) all[k] = k;
-        std::vector<__half> img;
-        tc_image(1, all, kBins, img);
-        CK(cudaMalloc(&p->d_a512, img.size() * sizeof(__half)));
-        CK(cudaMemcpy(p->d_a512, img.data(), img.size() * sizeof(__half), cudaMemcpyHostToDevice));
-    }
     std::vector<float2> tw(kLaneTwLen);
     for (int n = 0; n < 16; ++n)
         for (int k = 0; k < 32; ++k)
@@ -923,13 +890,12 @@ int bf_plan(const bf_config* cfg, bf_plan_t* out) {
     *p->h_status = 0;
     CK(cudaHostGetDevicePointer(&p->d_status, p->h_status, 0));
     if (p->grid <= 2 * kMaxSplit) {
-        // a launch splits at most grid / 2 items: two halves of 16 x 256 floats each, and
-        // one token per bin; the tensor-core form also parks each CTA's first half
-        const size_t slots = (size_t)p->grid / 2 + 1;
-        CK(cudaMalloc(&p->d_part, slots * 2 * kSub * kNs * sizeof(float)));
+        // a launch splits fewer items than it has CTAs (or CTA pairs): six passes of 16 x 256 floats
+        // each, and one token per bin
+        const size_t slots = (size_t)p->grid;
+        CK(cudaMalloc(&p->d_part, slots * kTds * kPol * kSub * kNs * sizeof(float)));
         CK(cudaMalloc(&p->d_part_tok, slots * kNs * sizeof(unsigned long long)));
         CK(cudaMemset(p->d_part_tok, 0, slots * kNs * sizeof(unsigned long long)));
-        if (p->terms) CK(cudaMalloc(&p->d_park, (size_t)p->grid * kSub * kNs * sizeof(float)));
     }
 
     if (p->cfg.mode == BF_MODE_SERVING) {
@@ -1097,9 +1063,6 @@ int bf_destroy(bf_plan_t p) {
     cudaFree(p->d_tw128);
     cudaFree(p->d_part);
     cudaFree(p->d_part_tok);
-    cudaFree(p->d_park);
-    cudaFree(p->d_inv);
-    cudaFree(p->d_a512);
     for (unsigned char* blk : p->atc_blocks)
         if (blk) cudaFree(blk);
     if (p->d_delays) cudaFree(p->d_delays);
@@ -1281,11 +1244,12 @@ static int debug_fused(bf_plan_t p, double freq_hz, const uint8_t* d_vin, int64_
     b.segs[0].vin = d_vin;
     b.segs[0].n_frames = nf;
     b.dump = reinterpret_cast<float2*>(d_out);
-    const int grid = std::min(p->grid, std::max(b.n_items, 1));
     if (p->terms) {
-        CK(fused_tc_launch(b, p->terms, mode, grid, p->stream));
+        const int pairs = p->grid / 2;
+        b.units = pass_units(b.n_items, pairs, false);
+        CK(fused_tc_launch(b, p->terms, mode, std::min(pairs, std::max(b.n_items, 1)), p->stream));
     } else {
-        CK(fused_fp32_dump_launch(b, grid, p->stream));
+        CK(fused_fp32_dump_launch(b, std::min(p->grid, std::max(b.n_items, 1)), p->stream));
     }
     CK(cudaStreamSynchronize(p->stream));
     if (p->h_status && *(volatile int*)p->h_status) {
@@ -1318,12 +1282,8 @@ int bf_debug_stall(bf_plan_t p, const uint8_t* d_vin, int64_t wait_ns) {
     b.segs[0].vin = d_vin;
     b.segs[0].n_frames = 1;
     b.wait_ns = (unsigned long long)wait_ns;
-    if (p->dft512 || p->terms == 1) {
-        // the form's own kernel: clusters of four (512 rows) or two (256 rows, 1 term)
-        CK(fused_tc_pair_stall_launch(b, p->dft512 ? 4 : 2, p->stream));
-    } else {
-        CK(fused_tc_launch(b, 1, 3, std::min(p->grid, kEw), p->stream));
-    }
+    b.units = pass_units(b.n_items, 1, false);
+    CK(fused_tc_launch(b, 1, 3, 1, p->stream));
     CK(cudaStreamSynchronize(p->stream));
     if (p->h_status && *(volatile int*)p->h_status) {
         *(volatile int*)p->h_status = 0;
