@@ -43,92 +43,149 @@ __global__ void __launch_bounds__(kMapThreads) skymap_kernel(const float* __rest
     }
 }
 
-// One thread per (beam, sub-channel) row: mean and population standard
+// 8-bit codes of (beam, sub-channel) rows: mean and population standard
 // deviation over the row's frames, then code = clip(floor(64 + 16 (x - mean) /
 // std + 1/2), 0, 255), a constant row giving 64.  FP32: the sums run over x -
 // x0 (x0 = the row's first frame), which keeps a constant row exactly constant
 // (mean = x0, std = 0) and makes the rounding error of the mean scale with the
 // row's spread instead of its level.  Valid for |x - mean| below ~1e18 (the
-// squares stay finite).  A CTA stages its 32 rows through shared
-// memory with coalesced loads; when the row length is a multiple of 4 (and the
-// code array 4-byte aligned) the codes
-// go back through shared memory as 32-bit words (rows padded by one word, no
-// bank conflicts) and leave with coalesced stores, row by row.  Rows longer
-// than the stage are read and written directly.
+// squares stay finite).  The sums run frame by frame, so a thread's two chains of
+// adds set the time of its row and rows in flight hide it: a CTA of four warps
+// stages 32 rows in shared memory of just their size (13 CTAs per SM at 128
+// frames), loads and reads 16 bytes at a time (rows padded to an odd number of
+// 16-byte words); one warp runs the sums, a thread per row, and all four write the
+// codes, a lane per four frames, straight to memory.  Rows longer than kU8Whole are
+// staged in chunks, once per sweep (sum, squares, codes), since whole rows would
+// leave too few CTAs.  65536 rows of 128 frames: 14.7 us (one warp per CTA, five CTAs
+// per SM, scalar accesses: 55 us); 42 MB, 6 us of HBM.
 constexpr int kU8Rows = 32;
-constexpr int kU8Stage = 256;          // frames staged per row
-constexpr int kU8Words = kU8Stage / 4 + 1;
+constexpr int kU8Threads = 128;
+constexpr int kU8Whole = 512;          // longest row staged whole
+constexpr int kU8Chunk = 256;          // frames per chunk of longer rows
 
-__global__ void __launch_bounds__(kU8Rows) rescale_u8_kernel(const float* __restrict__ in, long long rows,
-                                                               long long nf, uint8_t* __restrict__ codes,
-                                                               float* __restrict__ stats) {
-    __shared__ float st[kU8Rows][kU8Stage + 1];
-    __shared__ uint32_t cw[kU8Rows][kU8Words];
+// floats between staged rows of up to n frames: a multiple of 4 whose quarter is odd
+__host__ __device__ constexpr int u8_stride(int n) { return 4 * (((n + 3) / 4) | 1); }
+
+// kVec: rows are a multiple of 4 frames and start on 16 bytes (codes: 4 bytes).
+template <bool kVec>
+__global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __restrict__ in, long long rows, int nf,
+                                                                  int chunk, uint8_t* __restrict__ codes,
+                                                                  float* __restrict__ stats) {
+    extern __shared__ __align__(16) float st[];
+    __shared__ float mean_s[kU8Rows], sd_s[kU8Rows];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long r0 = (long long)blockIdx.x * kU8Rows;
-    const long long r = r0 + threadIdx.x;
-    const bool staged = nf <= kU8Stage;
-    const bool words = staged && (nf & 3) == 0 && (reinterpret_cast<uintptr_t>(codes) & 3) == 0;
     const int nr = (int)min((long long)kU8Rows, rows - r0);
-    if (staged) {
-        // the CTA's rows are contiguous: walk the block with 32 consecutive floats per load
-        // instruction, many loads in flight (the row and column advance without a division)
-        const float* src = in + r0 * nf;
-        const long long n = (long long)nr * nf;
-        int rr = (int)(threadIdx.x / nf);
-        long long f = threadIdx.x - rr * nf;
-        const long long step_r = kU8Rows / nf, step_f = kU8Rows % nf;
-#pragma unroll 16
-        for (long long i = threadIdx.x; i < n; i += kU8Rows) {
-            st[rr][f] = __ldg(src + i);
-            rr += (int)step_r;
-            f += step_f;
-            if (f >= nf) {
-                f -= nf;
-                ++rr;
+    const int S = u8_stride(chunk);
+    const float* src = in + r0 * nf;
+    constexpr int V = kVec ? 4 : 1;                       // frames per access
+
+    // n frames from f0 of the CTA's rows; whole rows are one contiguous block, walked without divisions
+    auto stage = [&](int f0, int n) {
+        __syncthreads();
+        if (n == nf) {
+            const int per = nf / V, total = nr * per, dr = kU8Threads / per, dc = kU8Threads % per;
+            int r = tid / per, c = tid % per;
+#pragma unroll 8
+            for (int i = tid; i < total; i += kU8Threads) {
+                if constexpr (kVec)
+                    *reinterpret_cast<float4*>(st + r * S + 4 * c) = __ldg(reinterpret_cast<const float4*>(src) + i);
+                else
+                    st[r * S + c] = __ldg(src + i);
+                r += dr;
+                c += dc;
+                if (c >= per) {
+                    c -= per;
+                    ++r;
+                }
             }
-        }
-        __syncthreads();
-    }
-    if (r < rows) {
-        const float* x = in + r * nf;
-        auto val = [&](long long f) -> float { return staged ? st[threadIdx.x][f] : __ldg(x + f); };
-        const float x0 = val(0);
-        float s = 0.f;
-        for (long long f = 1; f < nf; ++f) s += val(f) - x0;
-        const float mean = x0 + s / (float)nf;
-        float q = 0.f;
-        for (long long f = 0; f < nf; ++f) {
-            const float d = val(f) - mean;
-            q = fmaf(d, d, q);
-        }
-        const float sd = sqrtf(q / (float)nf);
-        if (stats) {
-            stats[2 * r] = mean;
-            stats[2 * r + 1] = sd;
-        }
-        const float scale = sd > 0.f ? 16.f / sd : 0.f;
-        auto code = [&](long long f) -> uint32_t {
-            float v = 64.f;
-            if (sd > 0.f) v = floorf(fmaf(val(f) - mean, scale, 64.5f));
-            v = v < 0.f ? 0.f : (v > 255.f ? 255.f : v);
-            return (uint32_t)v;
-        };
-        if (words) {
-            for (int w = 0; w < (int)(nf >> 2); ++w)
-                cw[threadIdx.x][w] = code(4 * w) | code(4 * w + 1) << 8 | code(4 * w + 2) << 16 |
-                                     code(4 * w + 3) << 24;
         } else {
-            uint8_t* c = codes + r * nf;
-            for (long long f = 0; f < nf; ++f) c[f] = (uint8_t)code(f);
+#pragma unroll 4
+            for (int r = warp; r < nr; r += kU8Threads / 32)
+                for (int i = lane; i < n / V; i += 32) {
+                    const float* p = src + (long long)r * nf + f0 + V * i;
+                    if constexpr (kVec)
+                        *reinterpret_cast<float4*>(st + r * S + 4 * i) = __ldg(reinterpret_cast<const float4*>(p));
+                    else
+                        st[r * S + i] = __ldg(p);
+                }
+        }
+        __syncthreads();
+    };
+    // f(frame, value) over the n staged frames of row `lane` in order
+    const float* row = st + lane * S;
+    auto each = [&](int n, auto f) {
+        if constexpr (kVec) {
+#pragma unroll 4
+            for (int k = 0; k < n; k += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(row + k);
+                f(k, v.x);
+                f(k + 1, v.y);
+                f(k + 2, v.z);
+                f(k + 3, v.w);
+            }
+        } else {
+#pragma unroll 8
+            for (int k = 0; k < n; ++k) f(k, row[k]);
+        }
+    };
+    const bool sums = warp == 0 && lane < nr, single = chunk >= nf;
+    float x0 = 0.f, s = 0.f, q = 0.f;
+    for (int f0 = 0; f0 < nf; f0 += chunk) {
+        const int n = min(chunk, nf - f0);
+        stage(f0, n);
+        if (!sums) continue;
+        if (f0 == 0) {
+            x0 = row[0];
+            each(n, [&](int k, float v) {
+                if (k) s += v - x0;
+            });
+        } else {
+            each(n, [&](int, float v) { s += v - x0; });
         }
     }
-    if (words) {
-        __syncthreads();
-        // row r0 + rr starts at a 4-byte boundary of `codes` (nf is a multiple of 4)
-        const int nw = (int)(nf >> 2);
-        for (int rr = 0; rr < nr; ++rr) {
-            uint32_t* dst = reinterpret_cast<uint32_t*>(codes + (r0 + rr) * nf);
-            for (int w = threadIdx.x; w < nw; w += kU8Rows) dst[w] = cw[rr][w];
+    const float mean = x0 + s / (float)nf;
+    for (int f0 = 0; f0 < nf; f0 += chunk) {
+        const int n = min(chunk, nf - f0);
+        if (!single) stage(f0, n);
+        if (!sums) continue;
+        each(n, [&](int, float v) {
+            const float d = v - mean;
+            q = fmaf(d, d, q);
+        });
+    }
+    if (sums) {
+        const float sd = sqrtf(q / (float)nf);
+        mean_s[lane] = mean;
+        sd_s[lane] = sd;
+        if (stats) {
+            stats[2 * (r0 + lane)] = mean;
+            stats[2 * (r0 + lane) + 1] = sd;
+        }
+    }
+    __syncthreads();
+    for (int f0 = 0; f0 < nf; f0 += chunk) {
+        const int n = min(chunk, nf - f0);
+        if (!single) stage(f0, n);
+#pragma unroll 2
+        for (int r = warp; r < nr; r += kU8Threads / 32) {
+            const float m = mean_s[r], sd = sd_s[r];
+            const float scale = sd > 0.f ? 16.f / sd : 0.f;
+            auto code = [&](float x) -> uint32_t {
+                float v = 64.f;
+                if (sd > 0.f) v = floorf(fmaf(x - m, scale, 64.5f));
+                v = v < 0.f ? 0.f : (v > 255.f ? 255.f : v);
+                return (uint32_t)v;
+            };
+            uint8_t* dst = codes + (r0 + r) * nf + f0;
+            for (int i = lane; i < n / V; i += 32) {
+                if constexpr (kVec) {
+                    const float4 v = *reinterpret_cast<const float4*>(st + r * S + 4 * i);
+                    reinterpret_cast<uint32_t*>(dst)[i] = code(v.x) | code(v.y) << 8 | code(v.z) << 16 | code(v.w) << 24;
+                } else {
+                    dst[i] = (uint8_t)code(st[r * S + i]);
+                }
+            }
         }
     }
 }
@@ -235,7 +292,27 @@ cudaError_t fma_probe_launch(bool paired, long long iters, float* sink, long lon
 cudaError_t rescale_u8_launch(const float* in, long long rows, long long nf, uint8_t* codes, float* stats,
                               cudaStream_t s) {
     if (rows <= 0 || nf <= 0) return cudaSuccess;
-    rescale_u8_kernel<<<(unsigned)((rows + kU8Rows - 1) / kU8Rows), kU8Rows, 0, s>>>(in, rows, nf, codes, stats);
+    const long long ctas = (rows + kU8Rows - 1) / kU8Rows;
+    if (nf > 0x7fffff00LL || ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const bool vec = (nf & 3) == 0 && (reinterpret_cast<uintptr_t>(in) & 15) == 0 && (reinterpret_cast<uintptr_t>(codes) & 3) == 0;
+    const int chunk = nf <= kU8Whole ? (int)nf : kU8Chunk;
+    const size_t smem = (size_t)kU8Rows * u8_stride(chunk) * sizeof(float);
+    auto kernel = vec ? rescale_u8_kernel<true> : rescale_u8_kernel<false>;
+    // more shared memory than a launch gets by default, once per device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    static std::once_flag once[kMaxDevices];
+    static cudaError_t result[kMaxDevices];
+    std::call_once(once[dev], [&] {
+        const int most = (int)(kU8Rows * u8_stride(kU8Whole) * sizeof(float));
+        result[dev] = cudaFuncSetAttribute(rescale_u8_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (result[dev] == cudaSuccess)
+            result[dev] = cudaFuncSetAttribute(rescale_u8_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    });
+    if (result[dev] != cudaSuccess) return result[dev];
+    kernel<<<(unsigned)ctas, kU8Threads, smem, s>>>(in, rows, (int)nf, chunk, codes, stats);
     return cudaGetLastError();
 }
 
