@@ -25,8 +25,6 @@ constexpr int kLaneTwLen = 32 * 16;     // twiddles between the FP32 form's two 
 
 // Segments per launch (kernel-parameter space holds the descriptors).
 constexpr int kMaxSegs = 160;
-// Items of one launch that the FP32 kernel may split in two (at most half its grid).
-constexpr int kMaxSplit = 512;
 
 // One (request, channel): a frame stream made of `carry_rows` leftover rows
 // followed by the request's new rows.
@@ -46,22 +44,22 @@ struct Seg {
 };
 
 // Work units of a launch whose items (six passes each) go to `slots` CTAs or CTA pairs in turn: whole
-// items, and the items of a last round that would not fill the slots in parts of g passes, g chosen
-// for the fewest passes of any slot (of equals the largest).  Every output adds the six passes' sums in
-// one fixed order, whether or not its item was split, so the result does not depend on how a request
-// was batched.
+// items, and the items of a last round that would not fill the slots in parts of g passes, g of the
+// allowed ones chosen for the fewest passes of any slot (of equals the largest).  Every output adds the
+// six passes' sums in one fixed order, whether or not its item was split, so the result does not depend
+// on how a request was batched.
 struct PassUnits {
     int n_full;     // items run whole: 0 .. n_full - 1
     int g;          // passes of a part of the others (1, 2, 3; 6: none is split)
     int n_units;    // n_full + (6 / g) x (split items)
 };
-inline PassUnits pass_units(int n_items, int slots, bool split) {
+inline PassUnits pass_units(int n_items, int slots, int least_g) {
     constexpr int kPasses = kTds * kPol;
     PassUnits u{n_items, kPasses, n_items};
     const int rem = n_items % slots;
-    if (!split || rem == 0) return u;
+    if (rem == 0) return u;
     int best = kPasses;
-    for (int g = 3; g >= 1; --g) {
+    for (int g = 3; g >= least_g; --g) {
         const int cost = (rem * (kPasses / g) + slots - 1) / slots * g;
         if (cost < best) {
             best = cost;
@@ -82,9 +80,9 @@ struct Batch {
     float2* dump;            // debug: up-channelised voltages instead of detection
     int* status;                 // set non-zero by a kernel whose bounded wait expired
     unsigned long long wait_ns;  // bound on each device-side wait (0: the default, 2 s)
-    PassUnits units;             // tensor-core form: work units of the launch
-    float* part;                 // sums of split items' passes [grid][6][16][256] (null: no split)
-    unsigned long long* part_tok;    // [grid][256] handshake tokens
+    PassUnits units;             // work units of the launch
+    float* part;                 // sums of split items' passes [CTAs][6][16][256]
+    unsigned long long* part_tok;    // [CTAs][256] passes published (see add_passes)
     unsigned long long epoch;        // this launch's number within the plan (from 1)
     Seg segs[kMaxSegs];
 };

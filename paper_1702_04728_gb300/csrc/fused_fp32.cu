@@ -53,7 +53,7 @@ constexpr int kFullThreads = 32 * (kTeam + kCons);
 // Register split (setmaxnreg): the launch gives every warp kRegLaunch registers per
 // thread; the producer warpgroups (warps 0-7) raise theirs to kRegProd and the
 // consumer warpgroup (warps 8-11) lowers its to kRegCons, within the same total.
-constexpr int kRegLaunch = 168, kRegProd = 184, kRegCons = 136;
+constexpr int kRegLaunch = 168, kRegProd = 176, kRegCons = 152;
 static_assert(kWarps * kRegProd + kCons * kRegCons <= (kWarps + kCons) * kRegLaunch,
               "the register split must fit in the launch's register file share");
 
@@ -121,7 +121,7 @@ __device__ __forceinline__ constexpr uint32_t tslot(int n2, int R) {
 // `before_tb` before the bin rows are first written.
 //
 // Bound: the FMA pipe with the register reads of its operands, 530 packed operations per row pair
-// here and 178 in the consumers.  Two warps per scheduler at 184 registers; one row pair per warp
+// here and 178 in the consumers.  Two warps per scheduler at 176 registers; one row pair per warp
 // and three warps at 128 registers (lane-dependent twiddles in both transforms) took 1.67 ms against
 // 1.57 ms here for 4 channels x 49152 samples.  The unpack straight from the transposing loads
 // replaced a store and two loads of the phased feeds per row pair and the odd half's divergent
@@ -220,7 +220,12 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 // of the slowest consumer, so no barrier phase ever mixes iterations.  The EMPTY
 // waits are bounded; on expiry the kernel carries on (keeping every barrier
 // matched) and reports through the status word.
-template <bool kDump>
+//
+// kMode: items = whole items and halves (units of 6 and 3 passes), parts = every item in parts of
+// 1 or 2 passes (a launch of few items), dump = up-channelised voltages instead of detection.  An
+// output is H0 + H1, H0 = (P0 + P1) + P2 and H1 = (P3 + P4) + P5 of its item's passes, in every mode.
+constexpr int kItems = 0, kParts = 1, kDump = 2;
+template <int kMode>
 __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_constant__ Batch bt) {
     extern __shared__ __align__(256) unsigned char smem[];   // the swizzles XOR address bits 4-7
     float4* bins_all = reinterpret_cast<float4*>(smem);
@@ -261,8 +266,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
     constexpr int kPasses = kTds * kPol;
     const unsigned long long wlim = bt.wait_ns ? bt.wait_ns : kWaitNs;
 
-    const Units units = make_units(bt.n_items, (int)gridDim.x, !kDump && bt.part != nullptr);
-    static_assert(kTds * kPol == 6, "an item is two halves of three passes");
+    const PassUnits units = bt.units;
+    static_assert(kPasses == 6, "an item is two halves of three passes");
 
     if (warp < kWarps) {
         // ---------------------------------- producers ----------------------------------
@@ -275,8 +280,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
         const uint32_t twl = smem_sa(twl_s) + 16u * lane;
         uint32_t g = 0;                                   // this team's iterations so far
         for (int un = blockIdx.x; un < units.n_units; un += gridDim.x) {
-            int item, ps0, ps1, half;
-            unit_of(units, un, item, ps0, ps1, half);
+            int item, ps0, ps1;
+            pass_unit(units, un, item, ps0, ps1);
             int sgi = 0;
             while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
             const Seg& sg = bt.segs[sgi];
@@ -332,8 +337,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
         const int m0 = 32 * cq + lane;                   // consumer slots m0 (half 0) and m0 + 128 (half 1)
         uint32_t g = 0;
         for (int un = blockIdx.x; un < units.n_units; un += gridDim.x) {
-            int item, ps0, ps1, half;
-            unit_of(units, un, item, ps0, ps1, half);
+            int item, ps0, ps1;
+            pass_unit(units, un, item, ps0, ps1);
             int sgi = 0;
             while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
             const Seg& sg = bt.segs[sgi];
@@ -347,10 +352,12 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
                 lut_s[i] = bt.lut[sg.table * kNs + bm];
             }
             bar_sync_n(kBarCons, 32 * kCons);
+            const bool whole = ps1 - ps0 == kPasses;
             const int Lsw0 = bsw(lut_s[m0]), Lsw1 = bsw(lut_s[m0 + 128]);
             // the slots' beams (gather order); output addresses are formed where they are used
             auto out0 = [&] { return sg.out + (long long)(kNs * j + beam_s[m0]) * sg.beam_stride + F; };
             auto out1 = [&] { return sg.out + (long long)(kNs * j + beam_s[m0 + 128]) * sg.beam_stride + F; };
+            // sums of the passes of the current half item (passes 0-2 or 3-5)
             float acc0[kSub], acc1[kSub];
 #pragma unroll
             for (int s2 = 0; s2 < kSub; ++s2) {
@@ -389,12 +396,45 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
                 tmem_wait_st();
                 // second pass: 16-point DFT over b for fine channels q = c + 8 d (this warp's lanes only)
                 const long long dbase = ((((long long)(F * kTds + blk) * kPol + pol) * kEw + j) * kNs) * kUp;
-                upchan_pass2(tlane, 0, acc0, kDump ? bt.dump + dbase + (long long)beam_s[m0] * kUp : nullptr);
-                upchan_pass2(tlane, 1, acc1, kDump ? bt.dump + dbase + (long long)beam_s[m0 + 128] * kUp : nullptr);
+                auto pass2 = [&](int hh, float (&acc)[kSub]) {
+                    float p[kSub];                            // this pass's sums
+#pragma unroll
+                    for (int s2 = 0; s2 < kSub; ++s2) p[s2] = 0.f;
+                    upchan_pass2(tlane, hh, p, kMode == kDump ? bt.dump + dbase + (long long)beam_s[m0 + 128 * hh] * kUp : nullptr);
+                    if constexpr (kMode == kParts) {
+                        float* mine = bt.part + ((size_t)(item - units.n_full) * kPasses + ps) * (kSub * kNs) + m0 + 128 * hh;
+#pragma unroll
+                        for (int s2 = 0; s2 < kSub; ++s2) mine[s2 * kNs] = p[s2];
+                    } else {
+#pragma unroll
+                        for (int s2 = 0; s2 < kSub; ++s2) acc[s2] += p[s2];
+                    }
+                };
+                pass2(0, acc0);
+                pass2(1, acc1);
                 // the next pass's gathers overwrite these TMEM columns in this warp's program order
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if constexpr (!kDump) {
-                    if (half < 0 && ps == kTds * kPol / 2 - 1) {
+                if constexpr (kMode == kParts) {
+                    // the thread that completes the item's six passes adds them (slots m0 and m0 + 128)
+                    const int slot = item - units.n_full;
+                    if (add_passes(bt.part_tok + (size_t)slot * kNs + m0, bt.epoch, 1)) {
+                        const float* in = bt.part + (size_t)slot * kPasses * (kSub * kNs) + m0;
+#pragma unroll 1
+                        for (int hh = 0; hh < 2; ++hh) {
+                            float* o = hh ? out1() : out0();
+#pragma unroll 4
+                            for (int s2 = 0; s2 < kSub; ++s2) {
+                                float v[kPasses];
+#pragma unroll
+                                for (int k = 0; k < kPasses; ++k)
+                                    v[k] = __ldcg(in + (size_t)k * (kSub * kNs) + s2 * kNs + 128 * hh);
+                                o[(long long)s2 * sg.sub_stride] = ((v[0] + v[1]) + v[2]) + ((v[3] + v[4]) + v[5]);
+                            }
+                        }
+                    }
+                }
+                if constexpr (kMode == kItems) {
+                    if (whole && ps == kPasses / 2 - 1) {
                         // whole item: H0 (passes 0-2) parks in shared memory until H1 is done
                         // (each thread reads back only its own words)
                         float* pk = park_s;
@@ -408,8 +448,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
                     }
                 }
             }
-            if constexpr (!kDump) {
-                if (half < 0) {
+            if constexpr (kMode == kItems) {
+                if (whole) {
                     // all loads before the first store: the stores could alias them as far as
                     // the compiler knows, and would otherwise serialise the loads
                     const float* pk = park_s;
@@ -427,14 +467,14 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
                 } else {
                     // half unit: publish this half; the second of the two halves to finish
                     // adds them (per thread: slots m0 and m0 + 128)
-                    const int slot = item - units.n_full;
+                    const int slot = item - units.n_full, half = ps0 ? 1 : 0;
                     float* mine = bt.part + ((size_t)slot * 2 + half) * (kSub * kNs);
 #pragma unroll
                     for (int s2 = 0; s2 < kSub; ++s2) {
                         mine[s2 * kNs + m0] = acc0[s2];
                         mine[s2 * kNs + m0 + 128] = acc1[s2];
                     }
-                    if (second_half(bt.part_tok + (size_t)slot * kNs + m0, bt.epoch, half)) {
+                    if (add_passes(bt.part_tok + (size_t)slot * kNs + m0, bt.epoch, kPasses / 2)) {
                         // H0 + H1 in either order: one addition of two terms is exact-commutative
                         const float* other = bt.part + ((size_t)slot * 2 + (half ^ 1)) * (kSub * kNs);
                         float h[kSub];
@@ -511,7 +551,7 @@ __global__ void debug_unpack_kernel(const uint8_t* __restrict__ in, float2* __re
 // increase could not be granted, so such a build is refused instead of launched.
 // Done once per device (the outcome is kept and returned on every launch); the flags
 // have internal linkage, so two copies of the library in one process keep their own.
-template <bool kDump>
+template <int kMode>
 cudaError_t prepare_fp32() {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -521,10 +561,10 @@ cudaError_t prepare_fp32() {
     static cudaError_t result[kMaxDevices];
     std::call_once(once[dev], [&] {
         cudaFuncAttributes fa;
-        cudaError_t r = cudaFuncGetAttributes(&fa, fused_fp32_kernel<kDump>);
+        cudaError_t r = cudaFuncGetAttributes(&fa, fused_fp32_kernel<kMode>);
         if (r == cudaSuccess && fa.numRegs < kRegLaunch) r = cudaErrorInvalidConfiguration;
         if (r == cudaSuccess)
-            r = cudaFuncSetAttribute(fused_fp32_kernel<kDump>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            r = cudaFuncSetAttribute(fused_fp32_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kSmemTotal);
         result[dev] = r;
     });
@@ -533,22 +573,23 @@ cudaError_t prepare_fp32() {
 
 }  // namespace
 
-cudaError_t fused_fp32_launch(const Batch& b, int grid, cudaStream_t s) {
+namespace {
+template <int kMode>
+cudaError_t launch_fp32(const Batch& b, int grid, cudaStream_t s) {
     if (b.n_items <= 0) return cudaSuccess;
-    if (b.part && grid > 2 * kMaxSplit) return cudaErrorInvalidValue;
-    cudaError_t e = prepare_fp32<false>();
+    if (b.units.g < kTds * kPol && (!b.part || !b.part_tok)) return cudaErrorInvalidValue;
+    cudaError_t e = prepare_fp32<kMode>();
     if (e != cudaSuccess) return e;
-    fused_fp32_kernel<false><<<grid, kThreads, kSmemTotal, s>>>(b);
+    fused_fp32_kernel<kMode><<<grid, kThreads, kSmemTotal, s>>>(b);
     return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t fused_fp32_launch(const Batch& b, int grid, cudaStream_t s) {
+    return b.units.g < kTds * kPol / 2 ? launch_fp32<kParts>(b, grid, s) : launch_fp32<kItems>(b, grid, s);
 }
 
-cudaError_t fused_fp32_dump_launch(const Batch& b, int grid, cudaStream_t s) {
-    if (b.n_items <= 0) return cudaSuccess;
-    cudaError_t e = prepare_fp32<true>();
-    if (e != cudaSuccess) return e;
-    fused_fp32_kernel<true><<<grid, kThreads, kSmemTotal, s>>>(b);
-    return cudaGetLastError();
-}
+cudaError_t fused_fp32_dump_launch(const Batch& b, int grid, cudaStream_t s) { return launch_fp32<kDump>(b, grid, s); }
 
 int fused_fp32_max_grid(int device) {
     int sms = 0;

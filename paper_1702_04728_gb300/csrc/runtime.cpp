@@ -635,15 +635,13 @@ int launch_jobs(bf_plan_s* p, std::vector<Job>& jobs, size_t bytes) {
     CK(cudaEventRecord(ev_start.ev, p->stream));
     for (auto& bb : batches) {
         bb.epoch = ++p->launches;
-        cudaError_t e;
-        if (p->terms) {
-            bb.units = pass_units(bb.n_items, p->grid / 2, bb.part != nullptr);
-            e = fused_tc_launch(bb, p->terms, 0, std::min(p->grid / 2, bb.units.n_units), p->stream);
-        } else {
-            // a launch of at most half a grid of items runs every item as two halves on two CTAs
-            const int grid = 2 * bb.n_items <= p->grid ? 2 * bb.n_items : std::min(p->grid, bb.n_items);
-            e = fused_fp32_launch(bb, grid, p->stream);
-        }
+        // One CTA (FP32 form) or CTA pair (tensor-core forms) per work unit at a time.  The FP32 form's
+        // parts of fewer than three passes have a kernel of their own, without whole items: the
+        // code that publishes single passes costs the other 3 %.
+        const int slots = p->terms ? p->grid / 2 : p->grid;
+        bb.units = pass_units(bb.n_items, slots, p->terms || bb.n_items < slots ? 1 : 3);
+        const int n = std::min(slots, bb.units.n_units);
+        const cudaError_t e = p->terms ? fused_tc_launch(bb, p->terms, 0, n, p->stream) : fused_fp32_launch(bb, n, p->stream);
         if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
     }
     for (auto& c : carries) {
@@ -889,14 +887,12 @@ int bf_plan(const bf_config* cfg, bf_plan_t* out) {
     CK(cudaHostAlloc(&p->h_status, sizeof(int), cudaHostAllocMapped));
     *p->h_status = 0;
     CK(cudaHostGetDevicePointer(&p->d_status, p->h_status, 0));
-    if (p->grid <= 2 * kMaxSplit) {
-        // a launch splits fewer items than it has CTAs (or CTA pairs): six passes of 16 x 256 floats
-        // each, and one token per bin
-        const size_t slots = (size_t)p->grid;
-        CK(cudaMalloc(&p->d_part, slots * kTds * kPol * kSub * kNs * sizeof(float)));
-        CK(cudaMalloc(&p->d_part_tok, slots * kNs * sizeof(unsigned long long)));
-        CK(cudaMemset(p->d_part_tok, 0, slots * kNs * sizeof(unsigned long long)));
-    }
+    // a launch splits fewer items than it has CTAs: six passes of 16 x 256 floats each, and one token
+    // per bin
+    const size_t slots = (size_t)p->grid;
+    CK(cudaMalloc(&p->d_part, slots * kTds * kPol * kSub * kNs * sizeof(float)));
+    CK(cudaMalloc(&p->d_part_tok, slots * kNs * sizeof(unsigned long long)));
+    CK(cudaMemset(p->d_part_tok, 0, slots * kNs * sizeof(unsigned long long)));
 
     if (p->cfg.mode == BF_MODE_SERVING) {
         bf_plan_s* raw = p.get();
@@ -1244,12 +1240,13 @@ static int debug_fused(bf_plan_t p, double freq_hz, const uint8_t* d_vin, int64_
     b.segs[0].vin = d_vin;
     b.segs[0].n_frames = nf;
     b.dump = reinterpret_cast<float2*>(d_out);
+    const int slots = p->terms ? p->grid / 2 : p->grid;
+    b.units = pass_units(b.n_items, slots, 6);
+    const int n = std::min(slots, std::max(b.n_items, 1));
     if (p->terms) {
-        const int pairs = p->grid / 2;
-        b.units = pass_units(b.n_items, pairs, false);
-        CK(fused_tc_launch(b, p->terms, mode, std::min(pairs, std::max(b.n_items, 1)), p->stream));
+        CK(fused_tc_launch(b, p->terms, mode, n, p->stream));
     } else {
-        CK(fused_fp32_dump_launch(b, std::min(p->grid, std::max(b.n_items, 1)), p->stream));
+        CK(fused_fp32_dump_launch(b, n, p->stream));
     }
     CK(cudaStreamSynchronize(p->stream));
     if (p->h_status && *(volatile int*)p->h_status) {
@@ -1282,7 +1279,7 @@ int bf_debug_stall(bf_plan_t p, const uint8_t* d_vin, int64_t wait_ns) {
     b.segs[0].vin = d_vin;
     b.segs[0].n_frames = 1;
     b.wait_ns = (unsigned long long)wait_ns;
-    b.units = pass_units(b.n_items, 1, false);
+    b.units = pass_units(b.n_items, 1, 6);
     CK(fused_tc_launch(b, 1, 3, 1, p->stream));
     CK(cudaStreamSynchronize(p->stream));
     if (p->h_status && *(volatile int*)p->h_status) {

@@ -180,3 +180,21 @@ def test_dedispersion_recovers_a_burst(built_lib):
 
     assert snr(ser[beam]) > 1.5 * snr(ser0[beam][: ser.shape[1]])
     assert int(np.argmax(ser.max(axis=1))) == beam
+
+
+@pytest.mark.parametrize("rows,nf,offset", [(31, 2, 0), (64, 3, 0), (45, 4, 0), (97, 31, 0), (64, 36, 1),
+                                            (40, 128, 3), (65, 511, 0), (33, 512, 0), (33, 513, 0), (34, 516, 0),
+                                            (50, 516, 2)])
+def test_rescale_u8_staging(built_lib, rows, nf, offset):
+    """Row lengths around the staged sizes (whole rows up to 512 frames, chunks of 256 and a short
+    last one beyond), a last group of fewer than 32 rows, and code arrays off a 4-byte boundary."""
+    rng = np.random.default_rng(rows + nf)
+    xh = intensity_rows(rng, rows, nf)
+    buf = torch.zeros(rows * nf + 8, dtype=torch.uint8, device="cuda")
+    codes = buf[offset:offset + rows * nf]
+    stats = torch.empty(rows, 2, dtype=torch.float32, device="cuda")
+    with B.Plan() as p:
+        B.bf_rescale_u8(p.handle, torch.from_numpy(xh).cuda(), rows, nf, codes, stats)
+        torch.cuda.synchronize()
+    check_rescale(xh, codes.cpu().numpy(), stats.cpu().numpy())
+    assert buf[:offset].sum().item() == 0 and buf[offset + rows * nf:].sum().item() == 0
