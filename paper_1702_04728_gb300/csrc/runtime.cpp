@@ -37,6 +37,7 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr int kTableCap = 4096;        // default and largest number of per-frequency table slots
 constexpr int kTcBlock = 64;           // tensor-core twiddle images are allocated 64 slots at a time
 constexpr int kMaxInflight = 4;
+constexpr int kPollSpinUs = 3000;      // bf_poll on a direct plan: time polled without sleeping
 
 thread_local std::string g_err;
 
@@ -1008,8 +1009,16 @@ static int poll_ticket(bf_plan_t p, uint64_t ticket, int64_t timeout_us, int64_t
         }
         const auto el = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
         if (timeout_us >= 0 && el >= timeout_us) return BF_PENDING;
-        // inflight: poll the event; queued: wait for the worker
-        p->cv.wait_for(lk, std::chrono::microseconds(it->second.state == T_INFLIGHT ? 10 : 200));
+        // inflight: poll the event; queued: wait for the worker.  A timed sleep lasts some 60 us (10 us
+        // and the timer slack), as long as the kernel of a short request, so on a direct plan
+        // the first milliseconds are polled without sleeping, with the lock open in between.
+        if (it->second.state == T_INFLIGHT && p->cfg.mode == BF_MODE_DIRECT && el < kPollSpinUs) {
+            lk.unlock();
+            std::this_thread::yield();
+            lk.lock();
+        } else {
+            p->cv.wait_for(lk, std::chrono::microseconds(it->second.state == T_INFLIGHT ? 10 : 200));
+        }
     }
 }
 
