@@ -265,18 +265,26 @@ __device__ __forceinline__ unsigned long long globaltimer() {
     return t;
 }
 
+__device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
+    return ok != 0;
+}
+
 // Wait for the completion of phase `parity` of an mbarrier: false once `limit`
-// ns have passed without it.
+// ns have passed without it.  The timer is read only after a first test has failed, and then once in a
+// number of tests: a read costs some hundred cycles, and the waits are on the path of every hand-off.
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, unsigned long long limit) {
+    if (mbar_try(mbar, parity)) return true;
     const unsigned long long t0 = globaltimer();
     for (;;) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
-        if (ok) return true;
+#pragma unroll 1
+        for (int i = 0; i < 16; ++i)
+            if (mbar_try(mbar, parity)) return true;
         if (globaltimer() - t0 > limit) return false;
     }
 }

@@ -36,7 +36,7 @@
 //
 // Bound: the builders' unpack and E-W arithmetic (FP32 pipe) and the latency of two builder warps per
 // scheduler; the tensor pipe needs 512 x terms cycles of a chunk (3 terms: it and the shared-memory
-// reads of its operands).  Per 4 x 49152-sample request on 152 SMs: 1.02 / 1.36 / 1.75 ms for 1 / 2 / 3
+// reads of its operands).  Per 4 x 49152-sample request on 152 SMs: 0.98 / 1.34 / 1.70 ms for 1 / 2 / 3
 // terms, where one CTA with streamed twiddles took 1.89 (2) and 2.55 (3) and CTAs that copied the data
 // tile to each other 1.36 (1).
 #include "device_common.cuh"
@@ -90,25 +90,36 @@ struct TcCfg {
 constexpr uint32_t kTIdesc = (1u << 4) | ((128u >> 3) << 17) | ((256u >> 4) << 24);
 constexpr uint32_t kTIdescNeg = kTIdesc | (1u << 13);
 
-// shared-memory matrix descriptor (no swizzle, version 1)
-__device__ __forceinline__ uint64_t tdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
+// Shared-memory matrix descriptor (no swizzle, version 1): the address field is the low bits of the low
+// word, so an operand x bytes on has the low word + x / 16 (shared memory stays below 2^18 bytes).
+struct Desc {
+    uint32_t lo, hi;
+};
+__device__ __forceinline__ Desc tdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+    return {(saddr >> 4) | (lbo >> 4) << 16, (sbo >> 4) | 1u << 14};
 }
-__device__ __forceinline__ uint64_t adesc(uint32_t saddr) { return tdesc(saddr, kTALbo, kTASbo); }
 
-__device__ __forceinline__ void tmma(uint32_t dtmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
+// One MMA of the pair, issued by the lane with `leader` set; the whole warp runs the code around it, so
+// that descriptors stay in uniform registers.
+__device__ __forceinline__ void tmma(uint32_t leader, uint32_t dtmem, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                     uint32_t bhi, uint32_t idesc, uint32_t accum) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        :: "r"(dtmem), "l"(a), "l"(b), "r"(idesc), "r"(accum)
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %7, 0;\n\t"
+        "setp.ne.b32 q, %0, 0;\n\t"
+        "mov.b64 a, {%2, %3};\n\t"
+        "mov.b64 b, {%4, %5};\n\t"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%1], a, b, %6, p;\n\t}"
+        :: "r"(leader), "r"(dtmem), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accum)
         : "memory");
 }
 
-// commit of this thread's outstanding MMAs to the same mbarrier in both CTAs
-__device__ __forceinline__ void tcommit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 :: "r"(mbar), "h"((uint16_t)3) : "memory");
+// commit of the leader's outstanding MMAs to the same mbarrier in both CTAs
+__device__ __forceinline__ void tcommit(uint32_t leader, uint32_t mbar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %0, 0;\n\t"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%1], %2;\n\t}"
+        :: "r"(leader), "r"(mbar), "h"((uint16_t)3) : "memory");
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {
@@ -269,11 +280,20 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
 
     if (warp == kTMma) {
         // ------------------------------ twiddle loads and MMAs ------------------------------
-        if (lane == 0 && MODE != 3) {
+        // The whole warp runs this and the leader lane issues: in a branch of one lane every descriptor
+        // would be computed in vector registers and moved over (3 % of the 1- and 2-term forms).
+        if (MODE != 3) {
+            const uint32_t leader = lane == 0;
             uint32_t p_bfull = 0, p_tfree = 0, p_a = 0, p_lo = 0;
             const unsigned char* a_cur = nullptr;
             uint32_t s = 0, pass = 0;
             bool ok = true;
+            // a wait of the whole warp
+            auto wait = [&](uint32_t bar, uint32_t parity) {
+                ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, wlim)) && ok;
+            };
+            const Desc da = tdesc(smem0, kTALbo, kTASbo), db = tdesc(smem0 + (uint32_t)C::SM_A, C::B_LBO, C::B_SBO);
+            const Desc dl = tdesc(smem0 + (uint32_t)C::SM_A + C::B_STAGE, kTALbo, kTASbo);    // lo twiddles
             int seg_cursor = 0;
             for (int un = pair; un < units.n_units && ok; un += npairs) {
                 int item, ps0, ps1;
@@ -283,20 +303,24 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                 if (a_img != a_cur) {
                     if (a_cur) {
                         // the MMAs that read the old twiddles are complete before they are replaced
-                        if (rank == 0) tcommit(adone);
-                        ok = mbar_wait(adone, (p_a >> 1) & 1u, wlim) && ok;
+                        if (rank == 0) tcommit(leader, adone);
+                        wait(adone, (p_a >> 1) & 1u);
                         p_a ^= 2u;
                     }
-                    expect_tx(afull, (uint32_t)C::SM_A);
+                    if (leader) {
+                        expect_tx(afull, (uint32_t)C::SM_A);
 #pragma unroll 1
-                    for (int kc = 0; kc < kTNch; ++kc)
-                        bulk_g2s(smem0 + (uint32_t)(kc * 2 * kTTw), a_img + (size_t)(kc * 2 + (int)rank) * (2 * kTTw),
-                                 2 * kTTw, afull);
-                    ok = mbar_wait(afull, p_a & 1u, wlim) && ok;
+                        for (int kc = 0; kc < kTNch; ++kc)
+                            bulk_g2s(smem0 + (uint32_t)(kc * 2 * kTTw), a_img + (size_t)(kc * 2 + (int)rank) * (2 * kTTw),
+                                     2 * kTTw, afull);
+                    }
+                    __syncwarp();
+                    wait(afull, p_a & 1u);
                     if (rank == 1) {
-                        arrive_cluster(cta_addr(aother, 0));
+                        if (leader) arrive_cluster(cta_addr(aother, 0));
+                        __syncwarp();
                     } else {
-                        ok = mbar_wait(aother, p_a & 1u, wlim) && ok;
+                        wait(aother, p_a & 1u);
                     }
                     p_a ^= 1u;
                     a_cur = a_img;
@@ -306,64 +330,62 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                     const uint32_t buf = pass & 1u;
                     if (rank == 0 && pass >= 2) {
                         // the up-channel warps of both CTAs have read this accumulator half (pass - 2)
-                        ok = mbar_wait(tfree((int)buf), (p_tfree >> buf) & 1u, wlim) && ok;
+                        wait(tfree((int)buf), (p_tfree >> buf) & 1u);
                         p_tfree ^= 1u << buf;
                     }
+                    const uint32_t re = tmem + 256u * buf, im = re + 128u;
+#pragma unroll 1
                     for (int kc = 0; kc < kTNch && ok; ++kc) {
                         if (rank == 1) {
                             // 3 terms: this CTA's lo twiddles of the stage have landed
-                            ok = mbar_wait(lofull((int)s), (p_lo >> s) & 1u, wlim);
+                            wait(lofull((int)s), (p_lo >> s) & 1u);
                             p_lo ^= 1u << s;
-                            if (ok) arrive_cluster(cta_addr(bfull((int)s), 0));
+                            if (ok && leader) arrive_cluster(cta_addr(bfull((int)s), 0));
+                            __syncwarp();
                         } else {
-                            ok = mbar_wait(bfull((int)s), (p_bfull >> s) & 1u, wlim) && ok;
+                            wait(bfull((int)s), (p_bfull >> s) & 1u);
                             p_bfull ^= 1u << s;
                             if (!ok) break;
                             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                            const uint32_t a0 = smem0 + (uint32_t)(kc * 2 * kTTw);
-                            const uint32_t b0 = smem0 + (uint32_t)C::SM_A + s * (uint32_t)C::STAGE;
-                            const uint32_t re = tmem + 256u * buf, im = re + 128u;
-                            auto bdesc = [](uint32_t saddr) { return tdesc(saddr, C::B_LBO, C::B_SBO); };
+                            const uint32_t a0 = da.lo + (uint32_t)kc * (2 * kTTw / 16), b0 = db.lo + s * (C::STAGE / 16u);
+                            const uint32_t l0 = dl.lo + s * (C::STAGE / 16u);
 #pragma unroll
                             for (int ks = 0; ks < kTFeeds / 16; ++ks) {
-                                const uint64_t c = adesc(a0 + ks * 2 * kTALbo), sn = adesc(a0 + kTTw + ks * 2 * kTALbo);
-                                const uint32_t bk = b0 + ks * 2 * C::B_LBO;
-                                const uint64_t yr = bdesc(bk), yi = bdesc(bk + 128);
+                                const uint32_t c = a0 + ks * (2 * kTALbo / 16), sn = c + kTTw / 16;
+                                const uint32_t yr = b0 + ks * (2 * C::B_LBO / 16), yi = yr + 128 / 16;
                                 const uint32_t more = (kc | ks) ? 1u : 0u;
-                                tmma(re, c, yr, kTIdesc, more);
-                                tmma(im, c, yi, kTIdesc, more);
-                                tmma(re, sn, yi, kTIdesc, 1u);
-                                tmma(im, sn, yr, kTIdescNeg, 1u);
+                                tmma(leader, re, c, da.hi, yr, db.hi, kTIdesc, more);
+                                tmma(leader, im, c, da.hi, yi, db.hi, kTIdesc, more);
+                                tmma(leader, re, sn, da.hi, yi, db.hi, kTIdesc, 1u);
+                                tmma(leader, im, sn, da.hi, yr, db.hi, kTIdescNeg, 1u);
                                 if constexpr (C::B_LO) {
-                                    const uint64_t zr = bdesc(bk + 256), zi = bdesc(bk + 384);
-                                    tmma(re, c, zr, kTIdesc, 1u);
-                                    tmma(im, c, zi, kTIdesc, 1u);
-                                    tmma(re, sn, zi, kTIdesc, 1u);
-                                    tmma(im, sn, zr, kTIdescNeg, 1u);
+                                    const uint32_t zr = yr + 256 / 16, zi = yr + 384 / 16;
+                                    tmma(leader, re, c, da.hi, zr, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, c, da.hi, zi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, re, sn, da.hi, zi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, sn, da.hi, zr, db.hi, kTIdescNeg, 1u);
                                 }
                                 if constexpr (C::A_LO) {
-                                    const uint32_t l0 = b0 + (uint32_t)C::B_STAGE;
-                                    const uint64_t cl = adesc(l0 + ks * 2 * kTALbo), sl = adesc(l0 + kTTw + ks * 2 * kTALbo);
-                                    tmma(re, cl, yr, kTIdesc, 1u);
-                                    tmma(im, cl, yi, kTIdesc, 1u);
-                                    tmma(re, sl, yi, kTIdesc, 1u);
-                                    tmma(im, sl, yr, kTIdescNeg, 1u);
+                                    const uint32_t cl = l0 + ks * (2 * kTALbo / 16), sl = cl + kTTw / 16;
+                                    tmma(leader, re, cl, da.hi, yr, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, cl, da.hi, yi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, re, sl, da.hi, yi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, sl, da.hi, yr, db.hi, kTIdescNeg, 1u);
                                 }
                             }
-                            tcommit(bempty((int)s));
-                            if (kc == kTNch - 1) tcommit(accfull((int)buf));
+                            tcommit(leader, bempty((int)s));
+                            if (kc == kTNch - 1) tcommit(leader, accfull((int)buf));
                         }
                         if (++s == (uint32_t)NB) s = 0;
                     }
-                    if (*(volatile int*)&abort_s) ok = false;
+                    if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;
                 }
             }
             // every issued MMA is complete before shared and tensor memory are released
-            if (rank == 0) tcommit(adone);
-            if (!mbar_wait(adone, (p_a >> 1) & 1u, wlim)) ok = false;
+            if (rank == 0) tcommit(leader, adone);
+            wait(adone, (p_a >> 1) & 1u);
             if (!ok) abort_s = 1;
         }
-        __syncwarp();
     } else if (warp < kTBuild) {
         // ------------------------------ builders ------------------------------
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kTRegBuild) : "memory");
@@ -377,9 +399,22 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
         auto row_of = [&](const Seg& sg, int F, int ps) {
             return frame_row(sg, (long long)F * kFrame + (ps >> 1) * kUp + t) + 16 * oct;
         };
+        // ... of the first pass of unit un (at or after the segment `from`)
+        auto row_of_unit = [&](int un, int from) {
+            int item, ps0, ps1;
+            pass_unit(units, un, item, ps0, ps1);
+            while (from + 1 < bt.n_segs && bt.segs[from + 1].item_begin <= item) ++from;
+            return row_of(bt.segs[from], (item - bt.segs[from].item_begin) >> 2, ps0);
+        };
         uint32_t p_bempty = 0, s = 0;
         bool wrapped = false, ok = true;
         int sgi = 0;
+        const uint8_t *p = nullptr, *next = nullptr;                   // the current and the next block's row
+        RawT raw;
+        if (pair < units.n_units) {
+            p = row_of_unit(pair, 0);
+            load_raw(p, 0, raw);
+        }
         for (int un = pair; un < units.n_units && ok; un += npairs) {
             int item, ps0, ps1;
             pass_unit(units, un, item, ps0, ps1);
@@ -389,13 +424,15 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
             const int F = local >> 2, j = local & 3;
             EwW w;
             load_ew_frame(sg, bt.ew, F, j, w);
-            const uint8_t* p = row_of(sg, F, ps0);
-            RawT raw;
-            load_raw(p, 0, raw);
             for (int ps = ps0; ps < ps1 && ok; ++ps) {
+                if (ps == ps0 || !(ps & 1)) {
+                    // the rows after this block's: the item's next block or the next unit's first
+                    next = (ps | 1) + 1 < ps1 ? row_of(sg, F, ps + 2)
+                           : un + npairs < units.n_units ? row_of_unit(un + npairs, sgi) : nullptr;
+                }
                 const PolSel sel = pol_sel(ps & 1);
                 // four chunks per loop body: the raw rows alternate between registers without copies
-                // (1.16 ms with a copy per chunk, 1.02 ms without)
+                // (1.16 ms with a copy per chunk, 1.02 ms without, when this was taken)
 #pragma unroll 4
                 for (int kc = 0; kc < kTNch; ++kc) {
                     if (wrapped) {
@@ -420,9 +457,9 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                     const RawT cur = raw;
                     if (kc + 1 < kTNch) {
                         load_raw(p, kc + 1, raw);
-                    } else if (ps + 1 < ps1) {
-                        p = row_of(sg, F, ps + 1);
-                        load_raw(p, 0, raw);
+                    } else {
+                        if ((ps & 1) || ps + 1 == ps1) p = next;
+                        if (p) load_raw(p, 0, raw);
                     }
                     build<TERMS>(cur, sel, w, dst0 + s * (uint32_t)C::STAGE);
                     // the generic-proxy stores are visible to the tensor cores
