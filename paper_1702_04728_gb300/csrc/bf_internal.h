@@ -76,7 +76,6 @@ struct Batch {
     const int16_t* order;    // [n_tables][256]   FP32 form: beam taken by consumer slot (TMEM lane + 128 x half)
     const float2* ew;        // [n_tables][4 ew][4 cyl] E-W phases
     const float2* twl;       // FP32 form: exp(-2 pi i n k / 512) at [n / 2][k][n & 1], n < 16, k < 32
-    const float2* tw128;     // [128] exp(-2 pi i e / 128)
     float2* dump;            // debug: up-channelised voltages instead of detection
     int* status;                 // set non-zero by a kernel whose bounded wait expired
     unsigned long long wait_ns;  // bound on each device-side wait (0: the default, 2 s)
@@ -100,9 +99,19 @@ int fused_fp32_max_grid(int device);   // CTAs that fit at once (1 per SM)
 // (1 term only): the MMA thread stays idle, so the other waits run out and the kernel reports through
 // `status`.
 cudaError_t fused_tc_launch(const Batch& b, int terms, int mode, int pairs, cudaStream_t s);
-size_t tc_a_bytes(int terms);    // bytes of one table's twiddle image(s)
-// byte offset in an image of cos (part 0) or sin (part 1) of 2 pi n L(m) / 512, FP16; the lo image follows
-size_t tc_a_offset(int m, int n, int part);
+// Tensor-core form: a table's twiddle image, C (part 0) and S (part 1) = cos and sin of 2 pi n L(m) / 512
+// in FP16, in the order of the kernel's shared memory operand: chunks of kTFeeds feeds, the CTAs of a
+// pair (128 bins each), C and S blocks of 8-row x 16-byte core matrices.  For three terms the image of
+// the rest (lo) follows.
+constexpr int kTFeeds = 32;                       // feeds per chunk
+constexpr int kTTw = 128 * kTFeeds * 2;           // 8 KB: C or S of 128 bins for one chunk
+// operand blocks: k-groups (8 feeds) kTALbo and 8-row groups kTASbo bytes apart
+constexpr int kTALbo = 128, kTASbo = kTFeeds / 8 * kTALbo;
+constexpr size_t tc_a_bytes(int terms) { return (size_t)kNs * 2 * kFeed * 2 * (terms == 3 ? 2 : 1); }
+constexpr size_t tc_a_offset(int m, int n, int part) {
+    return (((size_t)(n / kTFeeds) * 2 + m / 128) * 2 + part) * kTTw + (size_t)(m % 128 / 8) * kTASbo +
+           (n % kTFeeds / 8) * kTALbo + (m % 8) * 16 + (n % 8) * 2;
+}
 cudaError_t skymap_launch(const float* in, int n_beams, long long per_beam, float* map, cudaStream_t s);
 cudaError_t dedisperse_launch(const float* in, const int* delays, int n_sub, long long nf, long long n_out,
                               float* out, cudaStream_t s);

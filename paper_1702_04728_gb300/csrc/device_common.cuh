@@ -166,16 +166,21 @@ __device__ __forceinline__ void dft16(cp (&x)[16]) {
 // in the mantissa of 2^23; one FFMA2 scales it back by 2^-q and removes 2^23 and the +8 offset --
 // exact throughout.
 // ---------------------------------------------------------------------------
+// The same bits in a uniform register (every lane holds x): an operand that costs no register read.
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __reduce_or_sync(0xffffffffu, x); }
+__device__ __forceinline__ float uniform(float x) { return __uint_as_float(uniform(__float_as_uint(x))); }
+
 // The nibbles of one polarisation in a byte pair (low byte polarisation 0): masks and the
 // constants of the exact rescaling.
 struct PolSel {
     uint32_t mi, mr;
     float si, bi, sr, br;
 };
+// (called by whole warps; in uniform registers: 1.55 -> 1.49 ms per 4 x 49152 samples in the FP32 form)
 __device__ __forceinline__ PolSel pol_sel(int pol) {
     const float s = pol ? 1.f / 256.f : 1.f;
-    return {pol ? 0xF00u : 0xFu, pol ? 0xF000u : 0xF0u, s, -(8388608.f * s + 8.f), s * 0.0625f,
-            -(524288.f * s + 8.f)};
+    return {uniform(pol ? 0xF00u : 0xFu), uniform(pol ? 0xF000u : 0xF0u), uniform(s),
+            uniform(-(8388608.f * s + 8.f)), uniform(s * 0.0625f), uniform(-(524288.f * s + 8.f))};
 }
 __device__ __forceinline__ float2 nibm(uint32_t g0, uint32_t g1, uint32_t m, float s, float b) {
     return fma2(make_float2(__uint_as_float((g0 & m) | 0x4B000000u), __uint_as_float((g1 & m) | 0x4B000000u)),
@@ -190,18 +195,13 @@ struct EwW {
     float2 R[3], I[3], NI[3];
 };
 
-// The same bits in a uniform register (every lane holds x): an operand that costs no register read.
-__device__ __forceinline__ float uniform(float x) {
-    return __uint_as_float(__reduce_or_sync(0xffffffffu, __float_as_uint(x)));
-}
-
 __device__ __forceinline__ void load_ew(const float2* __restrict__ ew, int table, int j, EwW& w) {
 #pragma unroll
     for (int c = 1; c < kCyl; ++c) {
         const float2 v = ew[(table * kEw + j) * kCyl + c];
-        w.R[c - 1] = bc(uniform(v.x));
-        w.I[c - 1] = bc(uniform(v.y));
-        w.NI[c - 1] = bc(uniform(-v.y));
+        w.R[c - 1] = bc(v.x);
+        w.I[c - 1] = bc(v.y);
+        w.NI[c - 1] = bc(-v.y);
     }
 }
 
@@ -214,6 +214,42 @@ __device__ __forceinline__ void load_ew_frame(const Seg& sg, const float2* __res
         load_ew(ew, sg.table, j, w);
     }
 }
+
+// Twiddles of the first up-channel pass: [b / 2][c] = (Re, Re', Im, Im') of exp(-2 pi i b c / 128) for b
+// and b + 1.  In constant memory: the FP32 form reads them by a warp-uniform index and so through
+// uniform registers (1.49 -> 1.47 ms per 4 x 49152 samples); the tensor-core forms, whose up-channel
+// warps have a scheduler's slots to themselves less often, from a copy in shared memory (constant reads
+// there: 1.01 -> 1.04 ms).
+struct PairTw {
+    float4 w[kUp / 16][8];
+};
+constexpr double cos128(int e) {                         // cos(2 pi e / 128)
+    constexpr double t[33] = {1.0, 0.99879545620517239271, 0.99518472667219688624, 0.98917650996478097345,
+                              0.98078528040323044913, 0.97003125319454399260, 0.95694033573220886494,
+                              0.94154406518302077841, 0.92387953251128675613, 0.90398929312344333159,
+                              0.88192126434835502971, 0.85772861000027206990, 0.83146961230254523708,
+                              0.80320753148064490981, 0.77301045336273696081, 0.74095112535495909118,
+                              0.70710678118654752440, 0.67155895484701840063, 0.63439328416364549822,
+                              0.59569930449243334347, 0.55557023301960222474, 0.51410274419322172659,
+                              0.47139673682599764856, 0.42755509343028209432, 0.38268343236508977173,
+                              0.33688985339222005069, 0.29028467725446236764, 0.24298017990326388995,
+                              0.19509032201612826785, 0.14673047445536175166, 0.098017140329560601994,
+                              0.049067674327418014255, 0.0};
+    const int k = e & (kUp - 1), h = k > 64 ? 128 - k : k;
+    return h > 32 ? -t[64 - h] : t[h];
+}
+constexpr PairTw make_pair_tw() {
+    PairTw p{};
+    for (int b = 0; b < kUp / 8; b += 2)
+        for (int c = 0; c < 8; ++c) {
+            p.w[b / 2][c].x = (float)cos128(b * c);
+            p.w[b / 2][c].y = (float)cos128((b + 1) * c);
+            p.w[b / 2][c].z = (float)-cos128(b * c - 32);
+            p.w[b / 2][c].w = (float)-cos128((b + 1) * c - 32);
+        }
+    return p;
+}
+__constant__ PairTw kPairTw = make_pair_tw();
 
 // ---------------------------------------------------------------------------
 // tensor-memory access (tcgen05), one warp per 32-lane quarter

@@ -66,10 +66,9 @@ constexpr int kRawB = 4 * kRawRow;                   // per producer warp: its t
 constexpr size_t kSmemBins = 2 * (size_t)kBinsF4 * 16;   // one buffer per team
 constexpr size_t kSmemRaw = (size_t)kWarps * kRawB;      // raw rows (cp.async), one iteration ahead
 constexpr size_t kSmemLut = 2 * kNs * sizeof(int);   // bins and beams in gather order
-constexpr size_t kSmemTw = 8 * 8 * 16;               // pair twiddles of the first up-channel pass
 constexpr size_t kSmemTwl = kLaneTwLen * sizeof(float2);           // exp(-2 pi i n2 k / 512), [8][32 k] x 2 n2
 constexpr size_t kSmemPark = (size_t)kSub * kNs * sizeof(float);   // first half of the current item
-constexpr size_t kSmemTotal = kSmemBins + kSmemRaw + kSmemLut + kSmemTw + kSmemTwl + kSmemPark;
+constexpr size_t kSmemTotal = kSmemBins + kSmemRaw + kSmemLut + kSmemTwl + kSmemPark;
 
 __device__ __forceinline__ uint32_t smem_sa(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -232,9 +231,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
     unsigned char* raw_all = smem + kSmemBins;
     int* lut_s = reinterpret_cast<int*>(smem + kSmemBins + kSmemRaw);
     int* beam_s = lut_s + kNs;
-    float4* tw_s = reinterpret_cast<float4*>(smem + kSmemBins + kSmemRaw + kSmemLut);
-    float4* twl_s = tw_s + kSmemTw / 16;
-    float* park_s = reinterpret_cast<float*>(smem + kSmemBins + kSmemRaw + kSmemLut + kSmemTw + kSmemTwl);
+    float4* twl_s = reinterpret_cast<float4*>(smem + kSmemBins + kSmemRaw + kSmemLut);
+    float* park_s = reinterpret_cast<float*>(smem + kSmemBins + kSmemRaw + kSmemLut + kSmemTwl);
     __shared__ uint32_t tmem_base_s;
     __shared__ __align__(8) uint64_t empty_s[2];
     __shared__ int expired_s;
@@ -246,13 +244,6 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
         const uint32_t dst = static_cast<uint32_t>(__cvta_generic_to_shared(&tmem_base_s));
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" :: "r"(dst) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    // pair twiddles of the first up-channel pass: (b0, b1) = (2 it, 2 it + 1), c = 0..7
-    for (int i = tid; i < 64; i += kThreads) {
-        const int it = i >> 3, c = i & 7;
-        const float2 w0 = bt.tw128[(2 * it * c) & (kUp - 1)];
-        const float2 w1 = bt.tw128[((2 * it + 1) * c) & (kUp - 1)];
-        tw_s[i] = make_float4(w0.x, w1.x, w0.y, w1.y);
     }
     for (int i = tid; i < kLaneTwLen / 2; i += kThreads) twl_s[i] = reinterpret_cast<const float4*>(bt.twl)[i];
     if (tid == 0) {
@@ -383,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
 #pragma unroll
                         for (int c = 0; c < 8; ++c) {
                             if (c) {
-                                const float4 t = tw_s[it * 8 + c];
+                                const float4 t = kPairTw.w[it][c];
                                 z[c] = cmulp(z[c], make_float2(t.x, t.y), make_float2(t.z, t.w));
                             }
                             tmem_st4(tlane + hh * 256 + 2 * (16 * c + b0), z[c].re.x, z[c].im.x, z[c].re.y,
@@ -538,9 +529,9 @@ __global__ void __launch_bounds__(32) debug_beams_kernel(const uint8_t* __restri
 
 __global__ void debug_unpack_kernel(const uint8_t* __restrict__ in, float2* __restrict__ out, long long n) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const PolSel ps = pol_sel(0);                        // by the whole warp
     if (i >= n) return;
     const uint32_t g = in[i];                            // as a polarisation-0 byte
-    const PolSel ps = pol_sel(0);
     const float2 re = nibm(g, g, ps.mr, ps.sr, ps.br), im = nibm(g, g, ps.mi, ps.si, ps.bi);
     out[i] = make_float2(re.x, im.x);
 }

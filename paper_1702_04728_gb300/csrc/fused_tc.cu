@@ -49,12 +49,9 @@
 namespace chimebf {
 namespace {
 
-constexpr int kTFeeds = 32;                       // feeds per chunk
+// Operands are K-major without swizzle (twiddles: bf_internal.h): 8-row x 16-byte core matrices, k-groups
+// (8 feeds) *LBO and 8-row groups *SBO bytes apart.
 constexpr int kTNch = kFeed / kTFeeds;            // 8 chunks per pass
-constexpr int kTTw = 128 * kTFeeds * 2;           // 8 KB: C or S of 128 bins for one chunk
-// Operands are K-major without swizzle: 8-row x 16-byte core matrices, k-groups (8 feeds) *Lbo and
-// 8-row groups *Sbo bytes apart.
-constexpr int kTALbo = 128, kTASbo = kTFeeds / 8 * kTALbo;
 constexpr int kTBuild = 8;                        // builder warps
 constexpr int kTUp = 4;                           // up-channel warps
 constexpr int kTMma = kTBuild + kTUp;             // the MMA / twiddle warp
@@ -80,7 +77,7 @@ struct TcCfg {
     static constexpr int BARS = 3 * NB + 7;
     static constexpr size_t SM_A = (size_t)kTNch * 2 * kTTw;           // 128 KB
     static constexpr size_t SM_RING = (size_t)NB * STAGE;
-    static constexpr size_t SM_TW = 8 * 8 * 16;
+    static constexpr size_t SM_TW = sizeof(PairTw);
     static constexpr size_t SMEM = SM_A + SM_RING + SM_TW + 8 * BARS;
     static_assert(SMEM + 128 <= 227 * 1024, "dynamic and static shared memory");
 };
@@ -263,12 +260,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         abort_s = 0;
     }
-    for (int i = tid; i < 64; i += kTThreads) {
-        const int it = i >> 3, c = i & 7;
-        const float2 w0 = bt.tw128[(2 * it * c) & (kUp - 1)];
-        const float2 w1 = bt.tw128[((2 * it + 1) * c) & (kUp - 1)];
-        tw_s[i] = make_float4(w0.x, w1.x, w0.y, w1.y);
-    }
+    for (int i = tid; i < 64; i += kTThreads) tw_s[i] = kPairTw.w[i >> 3][i & 7];
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     cluster_sync();                        // both CTAs' barriers exist before any remote arrival
@@ -621,18 +613,6 @@ cudaError_t launch_tc(const Batch& b, int pairs, cudaStream_t s) {
 }
 
 }  // namespace
-
-size_t tc_a_bytes(int terms) {
-    const size_t one = (size_t)kNs * 2 * kFeed * 2;              // 256 rows x (C, S) x 256 feeds x FP16
-    return terms == 3 ? 2 * one : one;
-}
-
-size_t tc_a_offset(int m, int n, int part) {
-    // chunk, CTA of the pair, C or S block; 8-row x 16-byte core matrices
-    const size_t block = (((size_t)(n / kTFeeds) * 2 + m / 128) * 2 + part) * kTTw;
-    const int r = m % 128, k = n % kTFeeds;
-    return block + (size_t)(r / 8) * kTASbo + (k / 8) * kTALbo + (r % 8) * 16 + (k % 8) * 2;
-}
 
 cudaError_t fused_tc_launch(const Batch& b, int terms, int mode, int pairs, cudaStream_t s) {
     switch (terms * 10 + mode) {

@@ -123,7 +123,6 @@ struct bf_plan_s {
     int16_t* d_order = nullptr;               // FP32 form: gather order of the beams per table
     float2* d_ew = nullptr;
     float2* d_twl = nullptr;
-    float2* d_tw128 = nullptr;
     // Per-frequency table slots (clamp table, gather order, E-W phases and, for the
     // tensor-core form, the FP16 twiddle image).  A slot is referenced by every open
     // stream that uses its frequency and by every unretired batch that reads it; a
@@ -462,7 +461,6 @@ Batch make_batch(const bf_plan_s* p) {
     b.order = p->d_order;
     b.ew = p->d_ew;
     b.twl = p->d_twl;
-    b.tw128 = p->d_tw128;
     b.status = p->d_status;
     b.part = p->d_part;
     b.part_tok = p->d_part_tok;
@@ -874,17 +872,12 @@ int bf_plan(const bf_config* cfg, bf_plan_t* out) {
     CK(cudaMalloc(&p->d_order, (size_t)p->table_cap * kNs * sizeof(int16_t)));
     CK(cudaMalloc(&p->d_ew, (size_t)p->table_cap * kEw * kCyl * sizeof(float2)));
     CK(cudaMalloc(&p->d_twl, kLaneTwLen * sizeof(float2)));
-    CK(cudaMalloc(&p->d_tw128, kUp * sizeof(float2)));
     std::vector<float2> tw(kLaneTwLen);
     for (int n = 0; n < 16; ++n)
         for (int k = 0; k < 32; ++k)
             tw[((n >> 1) * 32 + k) * 2 + (n & 1)] = make_float2((float)std::cos(-2.0 * kPi * (n * k) / kBins),
                                                                 (float)std::sin(-2.0 * kPi * (n * k) / kBins));
     CK(cudaMemcpy(p->d_twl, tw.data(), kLaneTwLen * sizeof(float2), cudaMemcpyHostToDevice));
-    tw.resize(kUp);
-    for (int e = 0; e < kUp; ++e)
-        tw[e] = make_float2((float)std::cos(-2.0 * kPi * e / kUp), (float)std::sin(-2.0 * kPi * e / kUp));
-    CK(cudaMemcpy(p->d_tw128, tw.data(), kUp * sizeof(float2), cudaMemcpyHostToDevice));
     CK(cudaHostAlloc(&p->h_status, sizeof(int), cudaHostAllocMapped));
     *p->h_status = 0;
     CK(cudaHostGetDevicePointer(&p->d_status, p->h_status, 0));
@@ -1065,7 +1058,6 @@ int bf_destroy(bf_plan_t p) {
     cudaFree(p->d_order);
     cudaFree(p->d_ew);
     cudaFree(p->d_twl);
-    cudaFree(p->d_tw128);
     cudaFree(p->d_part);
     cudaFree(p->d_part_tok);
     for (unsigned char* blk : p->atc_blocks)
