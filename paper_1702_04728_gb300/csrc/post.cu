@@ -191,17 +191,67 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
 }
 
 // Incoherent dedispersion to one DM: series[beam][t] = sum over sub-channels s
-// (in order) of in[beam][s][t + d_s], t < n_out.  Threads run along t, so each
-// sub-channel row is read with coalesced loads.
-__global__ void dedisperse_kernel(const float* __restrict__ in, const int* __restrict__ delays, int n_sub,
-                                  long long nf, long long n_out, float* __restrict__ out) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// of in[beam][s][t + d_s], t < n_out.  Threads run along t, so each sub-channel row
+// is read with coalesced (unaligned) loads.  A CTA takes up to 1024 frames of a beam, kR of them per
+// thread and wt apart, so that a row is read as one piece; `groups` of wt threads take a contiguous
+// share of the sub-channels each (in order), added in order at the end.  A thread loads dd_unroll rows
+// at a time: eight of long rows keep some 100 KB in flight per SM, of short ones (many groups) two are
+// enough and better (54 us at 64 frames, four 61, eight 66).  1024 sub-channels x 1017 frames to 630:
+// 446 us (5.9 TB/s); 64 frames to 58: 54 us (128 frames per CTA, rows one after the other: 518 and
+// 136 us).
+constexpr int kDdThreads = 512;
+constexpr int dd_unroll(int r) { return r == 1 ? 2 : 8; }
+
+template <int kR>
+__global__ void __launch_bounds__(kDdThreads) dedisperse_kernel(const float* __restrict__ in,
+                                                                  const int* __restrict__ delays, int n_sub, long long nf,
+                                                                  long long n_out, int wt, int groups,
+                                                                  float* __restrict__ out) {
+    __shared__ float part[kR][kDdThreads];
+    const int g = threadIdx.x / wt, c = threadIdx.x - g * wt;     // wt is a multiple of 32
+    const long long t0 = (long long)blockIdx.x * (kR * wt) + c;
     const int beam = blockIdx.y;
-    if (t >= n_out) return;
-    const float* row = in + (long long)beam * n_sub * nf + t;
-    float acc = 0.f;
-    for (int s = 0; s < n_sub; ++s) acc += __ldg(row + (long long)s * nf + delays[s]);
-    out[(long long)beam * n_out + t] = acc;
+    const int s0 = (int)((long long)n_sub * g / groups), s1 = (int)((long long)n_sub * (g + 1) / groups);
+    float acc[kR];
+    bool in_range[kR];
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+        acc[r] = 0.f;
+        in_range[r] = t0 + r * wt < n_out;
+    }
+    constexpr int kDdUnroll = dd_unroll(kR);
+    const float* row = in + ((long long)beam * n_sub + s0) * nf + t0;
+    int s = s0;
+    for (; s + kDdUnroll <= s1; s += kDdUnroll, row += kDdUnroll * nf) {
+        float v[kDdUnroll][kR];
+#pragma unroll
+        for (int k = 0; k < kDdUnroll; ++k) {
+            const float* p = row + k * nf + __ldg(delays + s + k);
+#pragma unroll
+            for (int r = 0; r < kR; ++r) v[k][r] = in_range[r] ? __ldg(p + r * wt) : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < kDdUnroll; ++k)
+#pragma unroll
+            for (int r = 0; r < kR; ++r) acc[r] += v[k][r];
+    }
+    for (; s < s1; ++s, row += nf) {
+        const float* p = row + __ldg(delays + s);
+#pragma unroll
+        for (int r = 0; r < kR; ++r) acc[r] += in_range[r] ? __ldg(p + r * wt) : 0.f;
+    }
+    if (groups > 1) {
+#pragma unroll
+        for (int r = 0; r < kR; ++r) part[r][threadIdx.x] = acc[r];
+        __syncthreads();
+        if (g) return;
+        for (int k = 1; k < groups; ++k)
+#pragma unroll
+            for (int r = 0; r < kR; ++r) acc[r] += part[r][k * wt + c];
+    }
+#pragma unroll
+    for (int r = 0; r < kR; ++r)
+        if (in_range[r]) out[(long long)beam * n_out + t0 + r * wt] = acc[r];
 }
 
 // Delay table of the allocation-free dedispersion entry point: one array per
@@ -265,8 +315,14 @@ cudaError_t dedisperse_static_table(int device, int** table) {
 cudaError_t dedisperse_launch(const float* in, const int* delays, int n_sub, long long nf, long long n_out,
                               float* out, cudaStream_t s) {
     if (n_out <= 0) return cudaSuccess;
-    dim3 grid((unsigned)((n_out + 127) / 128), kBeams);
-    dedisperse_kernel<<<grid, 128, 0, s>>>(in, delays, n_sub, nf, n_out, out);
+    // tiles of equal width up to 1024 frames, up to 256 threads along them; groups: as many as fill the
+    // CTA, each of 32 sub-channels or more
+    const long long tiles = (n_out + 1023) / 1024, width = (n_out + tiles - 1) / tiles;
+    const int r = (int)((width + 255) / 256), wt = (int)(((width + r - 1) / r + 31) / 32 * 32);
+    const int groups = std::max(1, std::min(kDdThreads / wt, n_sub / 32));
+    const dim3 grid((unsigned)((n_out + r * wt - 1) / (r * wt)), kBeams);
+    auto kernel = r == 1 ? dedisperse_kernel<1> : r == 2 ? dedisperse_kernel<2> : r == 3 ? dedisperse_kernel<3> : dedisperse_kernel<4>;
+    kernel<<<grid, wt * groups, 0, s>>>(in, delays, n_sub, nf, n_out, wt, groups, out);
     return cudaGetLastError();
 }
 

@@ -198,3 +198,19 @@ def test_rescale_u8_staging(built_lib, rows, nf, offset):
         torch.cuda.synchronize()
     check_rescale(xh, codes.cpu().numpy(), stats.cpu().numpy())
     assert buf[:offset].sum().item() == 0 and buf[offset + rows * nf:].sum().item() == 0
+
+
+@pytest.mark.parametrize("n_chan,nf,dm", [(2, 1, 0.0), (5, 33, 0.0), (3, 257, 0.2), (2, 513, 0.1), (3, 800, 1.0),
+                                          (2, 1025, 0.4), (9, 2050, 0.05)])
+def test_dedisperse_tiles(built_lib, n_chan, nf, dm):
+    """Series around the tile widths (1 to 4 frames per thread 256 apart, several tiles beyond 1024
+    frames) with few and with many groups of sub-channels: 32-bit sums of up to 144 positive terms,
+    each rounding at most 2^-24 of the sum, so 144 x 2^-24 < 1e-5 relative."""
+    rng = np.random.default_rng(n_chan * nf)
+    freqs = [600e6 + 390625.0 * 40 * k for k in range(n_chan)]
+    x = rng.gamma(48.0, 1e4, size=(1024, 16 * n_chan, nf)).astype(np.float32)
+    ref, d = O.dedisperse(x, freqs, dm)
+    with B.Plan() as p:
+        ser = p.dedisperse(torch.from_numpy(x).cuda(), freqs, dm).cpu().numpy()
+    assert ser.shape == ref.shape and ref.shape[1] > 0
+    assert np.max(np.abs(ser - ref) / ref) <= 1e-5
