@@ -348,7 +348,7 @@ __device__ __forceinline__ void pass_unit(const PassUnits& u, int un, int& item,
 // six (all of them are then visible to it).  The token holds the launch's epoch and the passes
 // counted so far, so a launch that was abandoned leaves nothing to clean up, and nothing waits.
 __device__ __forceinline__ bool add_passes(unsigned long long* tok, unsigned long long epoch, unsigned n) {
-    __threadfence();                                   // the published sums before the token
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");    // the published sums before the token
     unsigned long long seen = *(volatile unsigned long long*)tok, next;
     for (;;) {
         next = ((seen >> 3) == epoch ? seen : epoch << 3) + n;
@@ -357,8 +357,18 @@ __device__ __forceinline__ bool add_passes(unsigned long long* tok, unsigned lon
         seen = was;
     }
     if ((next & 7u) != (unsigned)(kTds * kPol)) return false;
-    __threadfence();                                   // the other parts' sums after their tokens
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");    // the other parts' sums after their tokens
     return true;
+}
+
+// The published sums of an item's six passes for one beam (`in`: its place in pass 0).  All loads come
+// before the caller's first store, which could alias them as far as the compiler knows: with
+// stores in between, the adds of a one-frame request took 16 of its 43 us.
+__device__ __forceinline__ void load_passes(const float* in, float (&v)[kTds * kPol][kSub]) {
+#pragma unroll
+    for (int k = 0; k < kTds * kPol; ++k)
+#pragma unroll
+        for (int q = 0; q < kSub; ++q) v[k][q] = __ldcg(in + (size_t)k * (kSub * kNs) + q * kNs);
 }
 
 // CTA barrier that also orders tensor-memory accesses across it.

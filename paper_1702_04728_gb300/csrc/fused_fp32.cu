@@ -413,14 +413,12 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
 #pragma unroll 1
                         for (int hh = 0; hh < 2; ++hh) {
                             float* o = hh ? out1() : out0();
-#pragma unroll 4
-                            for (int s2 = 0; s2 < kSub; ++s2) {
-                                float v[kPasses];
+                            float v[kPasses][kSub];
+                            load_passes(in + 128 * hh, v);
 #pragma unroll
-                                for (int k = 0; k < kPasses; ++k)
-                                    v[k] = __ldcg(in + (size_t)k * (kSub * kNs) + s2 * kNs + 128 * hh);
-                                o[(long long)s2 * sg.sub_stride] = ((v[0] + v[1]) + v[2]) + ((v[3] + v[4]) + v[5]);
-                            }
+                            for (int s2 = 0; s2 < kSub; ++s2)
+                                o[(long long)s2 * sg.sub_stride] =
+                                    ((v[0][s2] + v[1][s2]) + v[2][s2]) + ((v[3][s2] + v[4][s2]) + v[5][s2]);
                         }
                     }
                 }

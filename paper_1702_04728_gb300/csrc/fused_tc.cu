@@ -536,15 +536,12 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
 #pragma unroll
                         for (int q = 0; q < kSub; ++q) o[q * kNs] = pw[q].x + pw[q].y;
                         if (add_passes(bt.part_tok + (size_t)slot * kNs + m, bt.epoch, 1)) {
-                            const float* in = bt.part + (size_t)slot * (kTds * kPol) * (kSub * kNs) + m;
+                            float v[kTds * kPol][kSub];
+                            load_passes(bt.part + (size_t)slot * (kTds * kPol) * (kSub * kNs) + m, v);
                             float* out = sg.out + (long long)(kNs * j + m) * sg.beam_stride + F;
 #pragma unroll
-                            for (int q = 0; q < kSub; ++q) {
-                                float v[kTds * kPol];
-#pragma unroll
-                                for (int k = 0; k < kTds * kPol; ++k) v[k] = __ldcg(in + (size_t)k * (kSub * kNs) + q * kNs);
-                                out[(long long)q * sg.sub_stride] = ((v[0] + v[2]) + v[4]) + ((v[1] + v[3]) + v[5]);
-                            }
+                            for (int q = 0; q < kSub; ++q)
+                                out[(long long)q * sg.sub_stride] = ((v[0][q] + v[2][q]) + v[4][q]) + ((v[1][q] + v[3][q]) + v[5][q]);
                         }
                     }
                 }
