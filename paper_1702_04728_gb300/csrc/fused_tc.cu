@@ -27,18 +27,21 @@
 //     memory, so passes alternate between the halves and the MMAs of pass p + 1 overlap the
 //     up-channel passes (Sec. 3.2) of pass p.
 //
-// Per CTA: warps 0-7 build (one (time, 8 feeds) task per thread and 32-feed chunk, the next chunk's
-// raw rows prefetched into registers), warps 8-11 (one per tensor-memory lane quarter) run the
-// up-channel passes and detection for one bin per thread, warp 12 loads the twiddles and, in the first
-// CTA, issues the MMAs of the pair.  Hand-offs are mbarriers only; every wait is bounded
-// by %globaltimer, and on expiry the CTA records the failure and leaves its loops (the other CTA's
-// waits then expire too).
+// Per CTA: warps 0-10 build (a task is 8 times of a 32-feed chunk, 8 feeds of one time per thread; the
+// warps take the tasks in turn, with the next one's raw rows prefetched into registers), warp 11 loads
+// the twiddles and, in the first CTA, issues the MMAs of the pair, warps 12-15 (one per tensor-memory
+// lane quarter) run the up-channel passes and detection for one bin per thread.  16 warps is what the
+// register file gives at 128 a thread; with 8 builders, one per group of 8 times, the loads and the
+// arithmetic of two warps left each scheduler idle for half of its cycles: 0.98 / 1.33 / 1.69 ms for 1 /
+// 2 / 3 terms against 0.89 / 1.06 / 1.39 with 11 (4 x 49152 samples, 152 SMs).  Hand-offs are mbarriers
+// only; every wait is bounded by %globaltimer, and on expiry the CTA records the failure and leaves its
+// loops (the other CTA's waits then expire too).
 //
-// Bound: the builders' unpack and E-W arithmetic (FP32 pipe) and the latency of two builder warps per
-// scheduler; the tensor pipe needs 512 x terms cycles of a chunk (3 terms: it and the shared-memory
-// reads of its operands).  Per 4 x 49152-sample request on 152 SMs: 0.98 / 1.34 / 1.70 ms for 1 / 2 / 3
-// terms, where one CTA with streamed twiddles took 1.89 (2) and 2.55 (3) and CTAs that copied the data
-// tile to each other 1.36 (1).
+// Bound: the issue slots and the FP32 pipe that the builders' unpack and E-W arithmetic and the one
+// up-channel warp of a scheduler share (61 % and 54 % of cycles for 1 term); the tensor pipe needs 512 x
+// terms cycles of a chunk (3 terms: it and the shared-memory reads of its operands).  Per 4 x
+// 49152-sample request on 152 SMs: 0.89 / 1.06 / 1.39 ms for 1 / 2 / 3 terms, where one CTA with streamed
+// twiddles took 1.89 (2) and 2.55 (3) and CTAs that copied the data tile to each other 1.36 (1).
 #include "device_common.cuh"
 
 #include <cuda_fp16.h>
@@ -52,14 +55,15 @@ namespace {
 // Operands are K-major without swizzle (twiddles: bf_internal.h): 8-row x 16-byte core matrices, k-groups
 // (8 feeds) *LBO and 8-row groups *SBO bytes apart.
 constexpr int kTNch = kFeed / kTFeeds;            // 8 chunks per pass
-constexpr int kTBuild = 8;                        // builder warps
+constexpr int kTGroups = 8;                       // build tasks of a chunk in a CTA (8 times x 32 feeds each)
+constexpr int kTBuild = 11;                       // builder warps
+constexpr int kTMma = kTBuild;                    // the MMA / twiddle warp
 constexpr int kTUp = 4;                           // up-channel warps
-constexpr int kTMma = kTBuild + kTUp;             // the MMA / twiddle warp
-constexpr int kTThreads = 32 * (kTMma + 1);
-// Register split (setmaxnreg): builders kTRegBuild, up-channel warps kTRegUp, the MMA warp keeps the
-// launch count; the launcher checks that the launch gives enough (with fewer, the up-channel warps'
-// increase could never be granted).
-constexpr int kTRegBuild = 104, kTRegUp = 176;
+constexpr int kTThreads = 32 * (kTBuild + 1 + kTUp);
+// Register split (setmaxnreg, by warpgroup): builders and the MMA warp kTRegBuild, up-channel warps
+// kTRegUp (104 and 200: 0.93 ms for 1 term against 0.89); the launcher checks that the launch gives
+// enough (with fewer, the up-channel warps' increase could never be granted).
+constexpr int kTRegBuild = 112, kTRegUp = 176;
 
 template <int TERMS>
 struct TcCfg {
@@ -68,12 +72,12 @@ struct TcCfg {
     // eight lanes of a 128-bit store (two times, four k-groups, see the builders) in distinct bank
     // groups; for three terms there is room for half of it, a store then takes two passes
     static constexpr int B_LBO = (B_LO ? 512 : 256) + (A_LO ? 16 : 32), B_SBO = kTFeeds / 8 * B_LBO;
-    static constexpr int B_STAGE = 8 * B_SBO;                          // 64 times
+    static constexpr int B_STAGE = kTGroups * B_SBO;                   // 64 times
     static constexpr int STAGE = B_STAGE + (A_LO ? 2 * kTTw : 0);      // and the chunk's lo twiddles
     static constexpr int NB = TERMS == 1 ? 6 : TERMS == 2 ? 5 : 3;     // ring stages
     // arrivals on "stage full" in the first CTA: the builder warps of both CTAs; 3 terms: both
     // CTAs' lo twiddles
-    static constexpr int FULL = 2 * kTBuild + (A_LO ? 2 : 0);
+    static constexpr int FULL = 2 * kTGroups + (A_LO ? 2 : 0);
     static constexpr int BARS = 3 * NB + 7;
     static constexpr size_t SM_A = (size_t)kTNch * 2 * kTTw;           // 128 KB
     static constexpr size_t SM_RING = (size_t)NB * STAGE;
@@ -274,6 +278,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
         // ------------------------------ twiddle loads and MMAs ------------------------------
         // The whole warp runs this and the leader lane issues: in a branch of one lane every descriptor
         // would be computed in vector registers and moved over (3 % of the 1- and 2-term forms).
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kTRegBuild) : "memory");
         if (MODE != 3) {
             const uint32_t leader = lane == 0;
             uint32_t p_bfull = 0, p_tfree = 0, p_a = 0, p_lo = 0;
@@ -381,90 +386,111 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
     } else if (warp < kTBuild) {
         // ------------------------------ builders ------------------------------
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kTRegBuild) : "memory");
-        // lane bits 0-1 take the four feed octets of a chunk, bits 2-4 eight times: a quarter warp loads 64
-        // contiguous bytes of two rows (lanes on eight different lines at one offset instead take a
-        // pass of the L1 data banks each: 1.29 ms per 4 x 49152-sample request against 1.16)
-        const int t = 64 * (int)rank + 8 * warp + (lane >> 2), oct = lane & 3;
-        unsigned char* dst0 = ring + warp * C::B_SBO + oct * C::B_LBO + (lane >> 2) * 16;
+        // The warps take the CTA's tasks (unit, pass, chunk, group of 8 times) in turn.  Lane bits 0-1 take
+        // the four feed octets of a chunk, bits 2-4 eight times: a quarter warp loads 64 contiguous bytes
+        // of two rows (lanes on eight different lines at one offset instead take a pass of the L1 data
+        // banks each: 1.29 ms per 4 x 49152-sample request against 1.16)
+        const int wu = (int)uniform((uint32_t)warp);
+        const int t = 64 * (int)rank + (lane >> 2), oct = lane & 3;
+        unsigned char* dst0 = ring + oct * C::B_LBO + (lane >> 2) * 16;
         const uint32_t full0 = cta_addr(bar0, 0);                      // the first CTA's bfull(0)
-        // this thread's row at chunk 0 of pass ps of an item
-        auto row_of = [&](const Seg& sg, int F, int ps) {
-            return frame_row(sg, (long long)F * kFrame + (ps >> 1) * kUp + t) + 16 * oct;
-        };
-        // ... of the first pass of unit un (at or after the segment `from`)
-        auto row_of_unit = [&](int un, int from) {
-            int item, ps0, ps1;
-            pass_unit(units, un, item, ps0, ps1);
-            while (from + 1 < bt.n_segs && bt.segs[from + 1].item_begin <= item) ++from;
-            return row_of(bt.segs[from], (item - bt.segs[from].item_begin) >> 2, ps0);
-        };
-        uint32_t p_bempty = 0, s = 0;
-        bool wrapped = false, ok = true;
-        int sgi = 0;
-        const uint8_t *p = nullptr, *next = nullptr;                   // the current and the next block's row
-        RawT raw;
-        if (pair < units.n_units) {
-            p = row_of_unit(pair, 0);
-            load_raw(p, 0, raw);
-        }
-        for (int un = pair; un < units.n_units && ok; un += npairs) {
-            int item, ps0, ps1;
-            pass_unit(units, un, item, ps0, ps1);
+        // the next task, whose rows are loaded while the current one is built
+        int un = pair, ps = 0, ps1 = 0, kc = wu / kTGroups, g = wu % kTGroups, sgi = 0, F = 0, j = 0;
+        bool more = un < units.n_units, new_unit = true, new_pass = true;
+        auto enter_unit = [&] {
+            int item;
+            pass_unit(units, un, item, ps, ps1);
             while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
+            const int local = item - bt.segs[sgi].item_begin;
+            F = local >> 2;
+            j = local & 3;
+        };
+        // this thread's part of the rows of a block in the carried and in the new samples, and the first
+        // of its rows that is new
+        const uint8_t *carried = nullptr, *fresh = nullptr;
+        int first_fresh = 0;
+        auto enter_block = [&] {
             const Seg& sg = bt.segs[sgi];
-            const int local = item - sg.item_begin;
-            const int F = local >> 2, j = local & 3;
-            EwW w;
-            load_ew_frame(sg, bt.ew, F, j, w);
-            for (int ps = ps0; ps < ps1 && ok; ++ps) {
-                if (ps == ps0 || !(ps & 1)) {
-                    // the rows after this block's: the item's next block or the next unit's first
-                    next = (ps | 1) + 1 < ps1 ? row_of(sg, F, ps + 2)
-                           : un + npairs < units.n_units ? row_of_unit(un + npairs, sgi) : nullptr;
-                }
-                const PolSel sel = pol_sel(ps & 1);
-                // four chunks per loop body: the raw rows alternate between registers without copies
-                // (1.16 ms with a copy per chunk, 1.02 ms without, when this was taken)
-#pragma unroll 4
-                for (int kc = 0; kc < kTNch; ++kc) {
-                    if (wrapped) {
-                        // the MMAs have read stage s in both CTAs
-                        if (!mbar_wait(bempty((int)s), (p_bempty >> s) & 1u, wlim)) ok = false;
-                        p_bempty ^= 1u << s;
-                    }
-                    // the warp stops as one (a wait expired in any lane)
-                    if (!__all_sync(0xffffffffu, ok)) {
-                        ok = false;
-                        break;
-                    }
-                    if constexpr (C::A_LO) {
-                        if (tid == 0) {
-                            // the chunk's lo twiddles (second half of the image) into the stage
-                            const uint32_t bar = rank == 0 ? bfull((int)s) : lofull((int)s);
-                            expect_tx(bar, 2 * kTTw);
-                            bulk_g2s(smem0 + (uint32_t)C::SM_A + s * (uint32_t)C::STAGE + (uint32_t)C::B_STAGE,
-                                     sg.a_img + 2 * C::SM_A + (size_t)(kc * 2 + (int)rank) * (2 * kTTw), 2 * kTTw, bar);
-                        }
-                    }
-                    const RawT cur = raw;
-                    if (kc + 1 < kTNch) {
-                        load_raw(p, kc + 1, raw);
-                    } else {
-                        if ((ps & 1) || ps + 1 == ps1) p = next;
-                        if (p) load_raw(p, 0, raw);
-                    }
-                    build<TERMS>(cur, sel, w, dst0 + s * (uint32_t)C::STAGE);
-                    // the generic-proxy stores are visible to the tensor cores
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) arrive_cluster(full0 + 8u * s);
-                    if (++s == (uint32_t)NB) {
-                        s = 0;
-                        wrapped = true;
-                    }
-                }
+            const long long row0 = (long long)F * kFrame + (ps >> 1) * kUp;
+            const long long left = sg.carry_rows - row0;
+            first_fresh = left < 0 ? 0 : left < kUp ? (int)left : kUp;
+            carried = sg.carry + row0 * kInput + 16 * oct;
+            fresh = sg.vin - left * kInput + 16 * oct;
+        };
+        auto load_task = [&](RawT& r) {
+            const int row = t + 8 * g;
+            load_raw((row < first_fresh ? carried : fresh) + (uint32_t)(row * kInput), kc, r);
+        };
+        uint32_t s = (uint32_t)(wu / kTGroups), parity = 1;             // a fresh barrier passes a wait on parity 1
+        bool ok = true;
+        EwW w;
+        PolSel sel;
+        // builds the task whose rows are in cur and loads the one after it
+        auto task = [&](const RawT& cur, RawT& nxt) {
+            if (new_pass) {
+                if (new_unit) load_ew_frame(bt.segs[sgi], bt.ew, F, j, w);
+                sel = pol_sel(ps & 1);
                 if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;   // the warp stops as one
             }
+            const int g0 = g, kc0 = kc, sg0 = sgi;
+            new_unit = new_pass = false;
+            uint32_t ds = kTBuild / kTGroups;
+            g += kTBuild % kTGroups;
+            if (g >= kTGroups) {
+                g -= kTGroups;
+                ++ds;
+            }
+            kc += (int)ds;
+            if (kc >= kTNch) {
+                kc -= kTNch;
+                new_pass = true;
+                if (++ps == ps1) {
+                    un += npairs;
+                    new_unit = true;
+                    more = un < units.n_units;
+                    if (more) enter_unit();
+                }
+                if (more) enter_block();
+            }
+            if (more) load_task(nxt);
+            // the MMAs have read stage s in both CTAs
+            if (!mbar_wait(bempty((int)s), parity, wlim)) ok = false;
+            // the warp stops as one (a wait expired in any lane)
+            if (!__all_sync(0xffffffffu, ok)) {
+                ok = false;
+                return;
+            }
+            if constexpr (C::A_LO) {
+                if (g0 == 0 && lane == 0) {
+                    // the chunk's lo twiddles (second half of the image) into the stage
+                    const uint32_t bar = rank == 0 ? bfull((int)s) : lofull((int)s);
+                    expect_tx(bar, 2 * kTTw);
+                    bulk_g2s(smem0 + (uint32_t)C::SM_A + s * (uint32_t)C::STAGE + (uint32_t)C::B_STAGE,
+                             bt.segs[sg0].a_img + 2 * C::SM_A + (size_t)(kc0 * 2 + (int)rank) * (2 * kTTw), 2 * kTTw, bar);
+                }
+            }
+            build<TERMS>(cur, sel, w, dst0 + s * (uint32_t)C::STAGE + g0 * C::B_SBO);
+            // the generic-proxy stores are visible to the tensor cores
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) arrive_cluster(full0 + 8u * s);
+            s += ds;
+            if (s >= (uint32_t)C::NB) {
+                s -= (uint32_t)C::NB;
+                parity ^= 1u;
+            }
+        };
+        // two tasks per loop body: the raw rows alternate between registers without copies
+        RawT ra, rb;
+        if (more) {
+            enter_unit();
+            enter_block();
+            load_task(ra);
+        }
+        while (more && ok) {
+            task(ra, rb);
+            if (!more || !ok) break;
+            task(rb, ra);
         }
         if (!ok) abort_s = 1;
     } else {
@@ -585,7 +611,7 @@ cudaError_t launch_tc(const Batch& b, int pairs, cudaStream_t s) {
     std::call_once(once[dev], [&] {
         cudaFuncAttributes fa;
         cudaError_t r = cudaFuncGetAttributes(&fa, fused_tc_kernel<TERMS, MODE>);
-        if (r == cudaSuccess && kTBuild * kTRegBuild + kTUp * kTRegUp > kTMma * fa.numRegs) r = cudaErrorInvalidConfiguration;
+        if (r == cudaSuccess && (kTBuild + 1) * kTRegBuild + kTUp * kTRegUp > kTThreads / 32 * fa.numRegs) r = cudaErrorInvalidConfiguration;
         if (r == cudaSuccess)
             r = cudaFuncSetAttribute(fused_tc_kernel<TERMS, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)TcCfg<TERMS>::SMEM);
