@@ -329,6 +329,22 @@ __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(mbar) : "memory");
 }
 
+// Segment of a work item, by halving: a launch of 160 two-frame channels spends 5.96 instead of 6.21 ms
+// per 1024 channels against a scan from its first segment, which each read of the table delays by a
+// trip to the constant cache.
+__device__ __forceinline__ int seg_of(const Batch& bt, int item) {
+    int lo = 0, hi = bt.n_segs;
+#pragma unroll 1
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (bt.segs[mid].item_begin <= item)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
 // Pass units (see PassUnits): item and pass range [ps0, ps1) of unit `un`.
 __device__ __forceinline__ void pass_unit(const PassUnits& u, int un, int& item, int& ps0, int& ps1) {
     constexpr int kPasses = kTds * kPol;

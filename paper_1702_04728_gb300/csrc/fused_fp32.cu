@@ -273,13 +273,10 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
         for (int un = blockIdx.x; un < units.n_units; un += gridDim.x) {
             int item, ps0, ps1;
             pass_unit(units, un, item, ps0, ps1);
-            int sgi = 0;
-            while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
+            const int sgi = seg_of(bt, item);
             const Seg& sg = bt.segs[sgi];
             const int local = item - sg.item_begin;
             const int F = local >> 2, j = local & 3;
-            EwW w;
-            load_ew_frame(sg, bt.ew, F, j, w);
             // time rows 16 a + 2 it + {0, 1} of row pairs a = 2 tw, 2 tw + 1
             const long long row0 = (long long)F * kFrame + 32 * tw;
             // this warp's four rows of iteration (ps, it) into its raw buffer
@@ -295,6 +292,8 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
                 cp_commit();
             };
             fetch(ps0, team);
+            EwW w;
+            load_ew_frame(sg, bt.ew, F, j, w);
             for (int ps = ps0; ps < ps1; ++ps) {
                 const PolSel sel = pol_sel(ps & 1);
 #pragma unroll 1
@@ -330,8 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
         for (int un = blockIdx.x; un < units.n_units; un += gridDim.x) {
             int item, ps0, ps1;
             pass_unit(units, un, item, ps0, ps1);
-            int sgi = 0;
-            while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
+            const int sgi = seg_of(bt, item);
             const Seg& sg = bt.segs[sgi];
             const int local = item - sg.item_begin;
             const int F = local >> 2, j = local & 3;
