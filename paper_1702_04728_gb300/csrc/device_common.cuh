@@ -19,7 +19,7 @@ struct cp {            // two complex values in SoA form
 };
 
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 bc(float v) { return make_float2(v, v); }
@@ -58,8 +58,7 @@ __device__ __forceinline__ void dft4(cp& a0, cp& a1, cp& a2, cp& a3) {
 // t = Im w / c with c as rounded, so both parts of w carry one rounding; the two
 // roundings of p and the sums are relative to |b|, whatever the size of t.
 template <bool kRot>
-__device__ __forceinline__ void bfly_ct(cp& a, cp& b, float c, float t) {
-    const float2 pre = fma2(b.im, bc(-t), b.re), pim = fma2(b.re, bc(t), b.im);
+__device__ __forceinline__ void bfly_p(cp& a, cp& b, float2 pre, float2 pim, float c) {
     if constexpr (kRot) {
         b = {fma2(pim, bc(-c), a.re), fma2(pre, bc(c), a.im)};
         a = {fma2(pim, bc(c), a.re), fma2(pre, bc(-c), a.im)};
@@ -67,6 +66,10 @@ __device__ __forceinline__ void bfly_ct(cp& a, cp& b, float c, float t) {
         b = {fma2(pre, bc(-c), a.re), fma2(pim, bc(-c), a.im)};
         a = {fma2(pre, bc(c), a.re), fma2(pim, bc(c), a.im)};
     }
+}
+template <bool kRot>
+__device__ __forceinline__ void bfly_ct(cp& a, cp& b, float c, float t) {
+    bfly_p<kRot>(a, b, fma2(b.im, bc(-t), b.re), fma2(b.re, bc(t), b.im), c);
 }
 
 // cos and sin of 2 pi e / 32, e = 0..8
@@ -92,6 +95,11 @@ __device__ __forceinline__ void bfly(cp& a, cp& b) {
         const cp z = {sub2(a.re, b.im), add2(a.im, b.re)};
         a = y;
         b = z;
+    } else if constexpr ((E & 7) == 4) {
+        // 45 degrees: the tangent is 1, so sums in place of two FMAs with a constant (the same bits;
+        // with the packed difference as an add 1.466 -> 1.462 ms per 4 x 49152 samples, 5.96 -> 5.94 ms
+        // per 1024 channels x 2 frames)
+        bfly_p<(E >= 8)>(a, b, add2(b.re, b.im), sub2(b.im, b.re), (float)cos32(4));
     } else {
         constexpr float c = (float)cos32(E & 7), t = (float)(-sin32(E & 7) / (double)c);
         bfly_ct<(E >= 8)>(a, b, c, t);
