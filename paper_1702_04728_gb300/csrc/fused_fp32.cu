@@ -120,11 +120,12 @@ __device__ __forceinline__ constexpr uint32_t tslot(int n2, int R) {
 // `before_tb` before the bin rows are first written.
 //
 // Bound: the FMA pipe with the register reads of its operands, 530 packed operations per row pair
-// here and 178 in the consumers.  Two warps per scheduler at 176 registers; one row pair per warp
-// and three warps at 128 registers (lane-dependent twiddles in both transforms) took 1.67 ms against
-// 1.57 ms here for 4 channels x 49152 samples.  The unpack straight from the transposing loads
-// replaced a store and two loads of the phased feeds per row pair and the odd half's divergent
-// twiddles (1.64 ms).
+// here and 178 in the consumers: 59 % of its cycles, with 49 % of the issue slots; the two producer
+// warps of a scheduler set the pace, the consumers wait for half of their time.  4 channels x 49152
+// samples take 1.46 ms.  One row pair per warp and three warps at 128 registers (lane-dependent
+// twiddles in both transforms) took 1.67 ms where this split took 1.57; the unpack straight from the
+// transposing loads replaced a store and two loads of the phased feeds per row pair and the odd half's
+// divergent twiddles (1.64 ms then).
 template <class AfterEw, class BeforeTb>
 __device__ __forceinline__ void phase_a(uint32_t raw, const PolSel& ps, const EwW& w, uint32_t twl,
                                         uint32_t rows, int lane, AfterEw after_ew, BeforeTb before_tb) {
