@@ -422,6 +422,10 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
             load_raw((row < first_fresh ? carried : fresh) + (uint32_t)(row * kInput), kc, r);
         };
         uint32_t s = (uint32_t)(wu / kTGroups), parity = 1;             // a fresh barrier passes a wait on parity 1
+        // A wait for a stage's previous use must not pass on the use before that one.  The warp's previous task
+        // saw the release of the stage NB chunks before it, and commits are in order, so that use is over
+        // if the warp advances by at most NB chunks at a time.
+        static_assert((kTBuild + kTGroups - 1) / kTGroups <= C::NB, "a builder's step between tasks");
         bool ok = true;
         EwW w;
         PolSel sel;
