@@ -51,13 +51,16 @@ __global__ void __launch_bounds__(kMapThreads) skymap_kernel(const float* __rest
 // row's spread instead of its level.  Valid for |x - mean| below ~1e18 (the
 // squares stay finite).  The sums run frame by frame, so a thread's two chains of
 // adds set the time of its row and rows in flight hide it: a CTA of four warps
-// stages 32 rows in shared memory of just their size (13 CTAs per SM at 128
+// stages 32 rows in shared memory of just their size (10 CTAs per SM at 128
 // frames), loads and reads 16 bytes at a time (rows padded to an odd number of
 // 16-byte words); one warp runs the sums, a thread per row, and all four write the
 // codes, a lane per four frames, straight to memory.  Rows longer than kU8Whole are
 // staged in chunks, once per sweep (sum, squares, codes), since whole rows would
-// leave too few CTAs.  65536 rows of 128 frames: 14.7 us (one warp per CTA, five CTAs
-// per SM, scalar accesses: 55 us); 42 MB, 6 us of HBM.
+// leave too few CTAs.  Bound by instructions (0.55 of the issue slots), so 16 / std is
+// formed once per row, the codes are rounded by an addition instead of two conversions,
+// and places in shared memory advance without products: 65536 rows of 128 frames 14.3 us
+// (16.6 without these; one warp per CTA, five CTAs per SM, scalar accesses: 55), eight times
+// as many 77 us (94); 42 and 336 MB, 6 and 49 us of HBM.
 constexpr int kU8Rows = 32;
 constexpr int kU8Threads = 128;
 constexpr int kU8Whole = 512;          // longest row staged whole
@@ -72,7 +75,7 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
                                                                   int chunk, uint8_t* __restrict__ codes,
                                                                   float* __restrict__ stats) {
     extern __shared__ __align__(16) float st[];
-    __shared__ float mean_s[kU8Rows], sd_s[kU8Rows];
+    __shared__ float2 fit_s[kU8Rows];                     // mean and 16 / std, -1 for a row without spread
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long r0 = (long long)blockIdx.x * kU8Rows;
     const int nr = (int)min((long long)kU8Rows, rows - r0);
@@ -85,18 +88,19 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
         __syncthreads();
         if (n == nf) {
             const int per = nf / V, total = nr * per, dr = kU8Threads / per, dc = kU8Threads % per;
-            int r = tid / per, c = tid % per;
+            const int step = dr * S + V * dc, wrap = S - V * per;
+            int c = tid % per, o = tid / per * S + V * c;     // o: the access's place among the staged rows
 #pragma unroll 8
             for (int i = tid; i < total; i += kU8Threads) {
                 if constexpr (kVec)
-                    *reinterpret_cast<float4*>(st + r * S + 4 * c) = __ldg(reinterpret_cast<const float4*>(src) + i);
+                    *reinterpret_cast<float4*>(st + o) = __ldg(reinterpret_cast<const float4*>(src) + i);
                 else
-                    st[r * S + c] = __ldg(src + i);
-                r += dr;
+                    st[o] = __ldg(src + i);
+                o += step;
                 c += dc;
                 if (c >= per) {
                     c -= per;
-                    ++r;
+                    o += wrap;
                 }
             }
         } else {
@@ -116,7 +120,7 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
     const float* row = st + lane * S;
     auto each = [&](int n, auto f) {
         if constexpr (kVec) {
-#pragma unroll 4
+#pragma unroll 8
             for (int k = 0; k < n; k += 4) {
                 const float4 v = *reinterpret_cast<const float4*>(row + k);
                 f(k, v.x);
@@ -156,8 +160,7 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
     }
     if (sums) {
         const float sd = sqrtf(q / (float)nf);
-        mean_s[lane] = mean;
-        sd_s[lane] = sd;
+        fit_s[lane] = make_float2(mean, sd > 0.f ? 16.f / sd : -1.f);
         if (stats) {
             stats[2 * (r0 + lane)] = mean;
             stats[2 * (r0 + lane) + 1] = sd;
@@ -167,24 +170,42 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
     for (int f0 = 0; f0 < nf; f0 += chunk) {
         const int n = min(chunk, nf - f0);
         if (!single) stage(f0, n);
-#pragma unroll 2
-        for (int r = warp; r < nr; r += kU8Threads / 32) {
-            const float m = mean_s[r], sd = sd_s[r];
-            const float scale = sd > 0.f ? 16.f / sd : 0.f;
-            auto code = [&](float x) -> uint32_t {
-                float v = 64.f;
-                if (sd > 0.f) v = floorf(fmaf(x - m, scale, 64.5f));
-                v = v < 0.f ? 0.f : (v > 255.f ? 255.f : v);
-                return (uint32_t)v;
-            };
-            uint8_t* dst = codes + (r0 + r) * nf + f0;
-            for (int i = lane; i < n / V; i += 32) {
+        uint8_t* dst = codes + r0 * nf + f0;
+        // the clamped value's floor sits in the low byte of its sum with 2^23, rounded down
+        auto code = [&](float2 fit, float x) -> uint32_t {
+            const float v = fit.y < 0.f ? 64.f : fminf(fmaxf(fmaf(x - fit.x, fit.y, 64.5f), 0.f), 255.f);
+            return __float_as_uint(__fadd_rd(v, 8388608.f));
+        };
+        if (kVec || single) {
+            const int per = n / V, total = nr * per, dr = kU8Threads / per, dc = kU8Threads % per;
+            const int step = dr * S + V * dc, wrap = S - V * per;
+            int r = tid / per, c = tid % per, o = r * S + V * c;
+#pragma unroll 4
+            for (int i = tid; i < total; i += kU8Threads) {
+                const float2 fit = fit_s[r];
                 if constexpr (kVec) {
-                    const float4 v = *reinterpret_cast<const float4*>(st + r * S + 4 * i);
-                    reinterpret_cast<uint32_t*>(dst)[i] = code(v.x) | code(v.y) << 8 | code(v.z) << 16 | code(v.w) << 24;
+                    const float4 v = *reinterpret_cast<const float4*>(st + o);
+                    const uint32_t lo = __byte_perm(code(fit, v.x), code(fit, v.y), 0x0040);
+                    const uint32_t hi = __byte_perm(code(fit, v.z), code(fit, v.w), 0x0040);
+                    uint8_t* to = single ? dst + 4 * (size_t)i : dst + (size_t)r * nf + 4 * c;
+                    *reinterpret_cast<uint32_t*>(to) = __byte_perm(lo, hi, 0x5410);
                 } else {
-                    dst[i] = (uint8_t)code(st[r * S + i]);
+                    dst[i] = (uint8_t)code(fit, st[o]);
                 }
+                r += dr;
+                c += dc;
+                o += step;
+                if (c >= per) {
+                    c -= per;
+                    ++r;
+                    o += wrap;
+                }
+            }
+        } else {
+#pragma unroll 2
+            for (int r = warp; r < nr; r += kU8Threads / 32) {
+                const float2 fit = fit_s[r];
+                for (int i = lane; i < n; i += 32) dst[(size_t)r * nf + i] = (uint8_t)code(fit, st[r * S + i]);
             }
         }
     }

@@ -214,3 +214,21 @@ def test_dedisperse_tiles(built_lib, n_chan, nf, dm):
         ser = p.dedisperse(torch.from_numpy(x).cuda(), freqs, dm).cpu().numpy()
     assert ser.shape == ref.shape and ref.shape[1] > 0
     assert np.max(np.abs(ser - ref) / ref) <= 1e-5
+
+
+@pytest.mark.parametrize("nf", [128, 41, 1017])
+def test_rescale_u8_rows_without_a_finite_spread(built_lib, nf):
+    """A row's code is 64 where its spread is zero, not a number or beyond FP32: constant rows, rows with a
+    NaN or an infinity, rows whose squares overflow.  The rows between keep their codes, both ends clipped."""
+    rng = np.random.default_rng(nf)
+    x = intensity_rows(rng, 70, nf)
+    plain = x.copy()
+    x[3], x[10, nf // 2], x[20, 0], x[30, nf - 1] = 5.0, np.nan, np.inf, -np.inf
+    x[40] = np.where(np.arange(nf) % 2 == 0, 1e30, -1e30)
+    odd = [3, 10, 20, 30, 40]
+    with B.Plan() as p:
+        got = p.rescale_u8(torch.from_numpy(x.reshape(1, 70, nf)).cuda())[0].cpu().numpy().reshape(70, nf)
+        want = p.rescale_u8(torch.from_numpy(plain.reshape(1, 70, nf)).cuda())[0].cpu().numpy().reshape(70, nf)
+    assert (got[odd] == 64).all()
+    rest = np.setdiff1d(np.arange(70), odd)
+    assert np.array_equal(got[rest], want[rest])
