@@ -116,8 +116,10 @@ __device__ __forceinline__ constexpr uint32_t tslot(int n2, int R) {
 //   raw    the lane's ldsm4t address (raw_lane)
 //   twl    shared address of the lane's first entry of the [8][32] twiddle table
 //   rows   the two row pairs' bins (2 x 8 KB; the transpose runs in place)
-// Only warp-level synchronisation.  Hooks: `after_ew` runs once the raw rows have been read,
-// `before_tb` before the bin rows are first written.
+// Only warp-level synchronisation.  Hooks: `before_tb` runs before the bin rows are first written,
+// `after_raw`, which requests the next raw rows, between the halves of the first transform, where half of
+// the registers are free (with all of them taken, right after the unpack, 1.460 ms for 4 channels x 49152
+// samples; here 1.453; after the second half 1.51 to 1.53, too late).
 //
 // Bound: the FMA pipe with the register reads of its operands, 530 packed operations per row pair
 // here and 178 in the consumers: 59 % of its cycles, with 49 % of the issue slots; the two producer
@@ -126,9 +128,9 @@ __device__ __forceinline__ constexpr uint32_t tslot(int n2, int R) {
 // twiddles in both transforms) took 1.67 ms where this split took 1.57; the unpack straight from the
 // transposing loads replaced a store and two loads of the phased feeds per row pair and the odd half's
 // divergent twiddles (1.64 ms then).
-template <class AfterEw, class BeforeTb>
+template <class AfterRaw, class BeforeTb>
 __device__ __forceinline__ void phase_a(uint32_t raw, const PolSel& ps, const EwW& w, uint32_t twl,
-                                        uint32_t rows, int lane, AfterEw after_ew, BeforeTb before_tb) {
+                                        uint32_t rows, int lane, AfterRaw after_raw, BeforeTb before_tb) {
     cp y[16];
 #pragma unroll
     for (int n1 = 0; n1 < 16; ++n1) {
@@ -146,7 +148,6 @@ __device__ __forceinline__ void phase_a(uint32_t raw, const PolSel& ps, const Ew
             }
         }
     }
-    after_ew();
     {
         const int n2 = (lane >> 2) + 4 * (lane & 2), R = lane & 1;
         const uint32_t tw_ = rows + (uint32_t)(R * kRowB) + 16u * tslot(n2, R);
@@ -158,6 +159,7 @@ __device__ __forceinline__ void phase_a(uint32_t raw, const PolSel& ps, const Ew
         before_tb();
 #pragma unroll
         for (int k1 = 0; k1 < 16; ++k1) sts_cp((tw_ ^ (uint32_t)(16 * ((2 * k1) & 7))) + 256u * (2 * k1), v[k1]);
+        after_raw();
         dft16<1>(y);                                     // odd outputs: k = 2 k1 + 1
 #pragma unroll
         for (int k1 = 0; k1 < 16; ++k1)
@@ -280,12 +282,19 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
             const int F = local >> 2, j = local & 3;
             // time rows 16 a + 2 it + {0, 1} of row pairs a = 2 tw, 2 tw + 1
             const long long row0 = (long long)F * kFrame + 32 * tw;
+            // this lane's part of row row0 in the carried and in the new samples, and the number of rows
+            // from it that are carried: a row's address is then a comparison and 32-bit arithmetic
+            // (1.453 -> 1.406 ms per 4 x 49152 samples, 5.88 -> 5.68 per 1024 channels x 2 frames)
+            const uint8_t* const carried = sg.carry + row0 * kInput + 16 * lane;
+            const uint8_t* const fresh = sg.vin + (row0 - sg.carry_rows) * kInput + 16 * lane;
+            const int left = row0 < sg.carry_rows ? (int)(sg.carry_rows - row0) : 0;
             // this warp's four rows of iteration (ps, it) into its raw buffer
             auto fetch = [&](int ps, int it) {
-                const long long r = row0 + (ps >> 1) * kUp + 2 * it;
+                const int r0 = (ps >> 1) * kUp + 2 * it;
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const uint8_t* p = frame_row(sg, r + 16 * (k >> 1) + (k & 1)) + 16 * lane;
+                    const int r = r0 + 16 * (k >> 1) + (k & 1);
+                    const uint8_t* p = (r < left ? carried : fresh) + (uint32_t)(r * kInput);
                     const uint32_t d = raw_sa + (uint32_t)(k * kRawRow) + 16u * lane;
 #pragma unroll
                     for (int c = 0; c < kCyl; ++c) cp16(d + c * (kFeed * kPol), p + c * (kFeed * kPol));

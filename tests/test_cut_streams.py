@@ -1,6 +1,7 @@
-"""Carried rows in the tensor-core forms: a build task takes 8 times of a block, each thread from the
-carried or from the new samples.  A stream cut at any sample (inside a group of 8, at a block's edge,
-one short of a frame, several cuts) gives the bits of the uncut one."""
+"""Carried rows: the kernels take each row of a frame from the carried or from the new samples (a
+tensor-core build task 8 times of a block, a producer warp of the FP32 form 4 rows).  A stream cut at
+any sample (inside such a group, at a block's edge, one short of a frame, several cuts) gives the bits
+of the uncut one."""
 import numpy as np
 import pytest
 
@@ -12,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("cuts", [(1,), (5,), (64,), (127,), (128,), (261,), (383,), (384 + 130,), (3, 390, 1000)])
-@pytest.mark.parametrize("form", [B.BF_TC_DFT256, B.BF_TC_DFT256_X2, B.BF_TC_DFT256_X1])
+@pytest.mark.parametrize("form", [B.BF_FP32_FFT, B.BF_TC_DFT256, B.BF_TC_DFT256_X2, B.BF_TC_DFT256_X1])
 def test_cut_streams_have_the_bits_of_the_whole(built_lib, form, cuts):
     freqs = [430e6, 760e6]
     n = 384 * 4 + 77
