@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
     float* park_s = reinterpret_cast<float*>(smem + kSmemBins + kSmemRaw + kSmemLut + kSmemTwl);
     __shared__ uint32_t tmem_base_s;
     __shared__ __align__(8) uint64_t empty_s[2];
-    __shared__ int expired_s;
+    __shared__ int expired_s, table_s;                       // table_s: the table in lut_s and beam_s
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t empty0 = smem_sa(&empty_s[0]);
@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(empty0 + 8u * i), "n"(kCons) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         expired_s = 0;
+        table_s = -1;
     }
     cta_sync();
     const uint32_t tmem = tmem_base_s;
@@ -343,14 +344,19 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
             const Seg& sg = bt.segs[sgi];
             const int local = item - sg.item_begin;
             const int F = local >> 2, j = local & 3;
-            bar_sync_n(kBarCons, 32 * kCons);             // the previous item's table reads are done
-            // consumer slot i (TMEM lane + 128 x half) takes beam order[i]
-            for (int i = ctid; i < kNs; i += 32 * kCons) {
-                const int bm = bt.order[sg.table * kNs + i];
-                beam_s[i] = bm;
-                lut_s[i] = bt.lut[sg.table * kNs + bm];
+            // the table changes with the channel only (reloaded for every item 1.408 ms per 4 x 49152
+            // samples, 1.397 so); its number is in shared memory because a register more costs 1 %
+            if (sg.table != *(volatile int*)&table_s) {
+                bar_sync_n(kBarCons, 32 * kCons);         // the previous table's reads are done
+                // consumer slot i (TMEM lane + 128 x half) takes beam order[i]
+                for (int i = ctid; i < kNs; i += 32 * kCons) {
+                    const int bm = bt.order[sg.table * kNs + i];
+                    beam_s[i] = bm;
+                    lut_s[i] = bt.lut[sg.table * kNs + bm];
+                }
+                if (ctid == 0) table_s = sg.table;
+                bar_sync_n(kBarCons, 32 * kCons);
             }
-            bar_sync_n(kBarCons, 32 * kCons);
             const bool whole = ps1 - ps0 == kPasses;
             const int Lsw0 = bsw(lut_s[m0]), Lsw1 = bsw(lut_s[m0 + 128]);
             // the slots' beams (gather order); output addresses are formed where they are used
