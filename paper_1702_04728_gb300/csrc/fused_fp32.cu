@@ -122,9 +122,9 @@ __device__ __forceinline__ constexpr uint32_t tslot(int n2, int R) {
 // samples; here 1.453; after the second half 1.51 to 1.53, too late).
 //
 // Bound: the FMA pipe with the register reads of its operands, 530 packed operations per row pair
-// here and 178 in the consumers: 59 % of its cycles, with 49 % of the issue slots; the two producer
-// warps of a scheduler set the pace, the consumers wait for half of their time.  4 channels x 49152
-// samples take 1.46 ms.  One row pair per warp and three warps at 128 registers (lane-dependent
+// here and 178 in the consumers: 64 % of its cycles, with 52 % of the issue slots; the two producer
+// warps of a scheduler set the pace, the consumers wait for a good third of their time.  4 channels x 49152
+// samples take 1.40 ms.  One row pair per warp and three warps at 128 registers (lane-dependent
 // twiddles in both transforms) took 1.67 ms where this split took 1.57; the unpack straight from the
 // transposing loads replaced a store and two loads of the phased feeds per row pair and the odd half's
 // divergent twiddles (1.64 ms then).
