@@ -228,7 +228,9 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
     float4* tw_s = reinterpret_cast<float4*>(ring + C::SM_RING);
     uint64_t* mbar_s = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(tw_s) + C::SM_TW);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // the warp number in a uniform register: the roles' branches are then uniform too, without which the nested
+    // ones cost the tensor-core forms 12, 15 and 17 % (1, 2 and 3 terms)
+    const int tid = threadIdx.x, warp = (int)uniform((uint32_t)tid >> 5), lane = tid & 31;
     const uint32_t rank = cluster_rank();
     const uint32_t smem0 = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
     const uint32_t bar0 = static_cast<uint32_t>(__cvta_generic_to_shared(&mbar_s[0]));
@@ -274,229 +276,233 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
     const int pair = (int)cluster_id(), npairs = (int)n_clusters();
     const PassUnits units = bt.units;
 
-    if (warp == kTMma) {
-        // ------------------------------ twiddle loads and MMAs ------------------------------
-        // The whole warp runs this and the leader lane issues: in a branch of one lane every descriptor
-        // would be computed in vector registers and moved over (3 % of the 1- and 2-term forms).
+    static_assert((kTBuild + 1) % 4 == 0 && kTUp % 4 == 0, "the register split is by warpgroup");
+    if (warp <= kTMma) {
+        // one setmaxnreg for all warps of a warpgroup, as the instruction requires: builders 8-10 share the MMA
+        // warp's.  (In branches that do not hold the warps' code the compiler keeps all of it to the launch's
+        // count and spills.)
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kTRegBuild) : "memory");
-        if (MODE != 3) {
-            const uint32_t leader = lane == 0;
-            uint32_t p_bfull = 0, p_tfree = 0, p_a = 0, p_lo = 0;
-            const unsigned char* a_cur = nullptr;
-            uint32_t s = 0, pass = 0;
-            bool ok = true;
-            // a wait of the whole warp
-            auto wait = [&](uint32_t bar, uint32_t parity) {
-                ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, wlim)) && ok;
-            };
-            const Desc da = tdesc(smem0, kTALbo, kTASbo), db = tdesc(smem0 + (uint32_t)C::SM_A, C::B_LBO, C::B_SBO);
-            const Desc dl = tdesc(smem0 + (uint32_t)C::SM_A + C::B_STAGE, kTALbo, kTASbo);    // lo twiddles
-            int seg_cursor = 0;
-            for (int un = pair; un < units.n_units && ok; un += npairs) {
-                int item, ps0, ps1;
-                pass_unit(units, un, item, ps0, ps1);
-                while (seg_cursor + 1 < bt.n_segs && bt.segs[seg_cursor + 1].item_begin <= item) ++seg_cursor;
-                const unsigned char* a_img = bt.segs[seg_cursor].a_img;
-                if (a_img != a_cur) {
-                    if (a_cur) {
-                        // the MMAs that read the old twiddles are complete before they are replaced
-                        if (rank == 0) tcommit(leader, adone);
-                        wait(adone, (p_a >> 1) & 1u);
-                        p_a ^= 2u;
-                    }
-                    if (leader) {
-                        expect_tx(afull, (uint32_t)C::SM_A);
-#pragma unroll 1
-                        for (int kc = 0; kc < kTNch; ++kc)
-                            bulk_g2s(smem0 + (uint32_t)(kc * 2 * kTTw), a_img + (size_t)(kc * 2 + (int)rank) * (2 * kTTw),
-                                     2 * kTTw, afull);
-                    }
-                    __syncwarp();
-                    wait(afull, p_a & 1u);
-                    if (rank == 1) {
-                        if (leader) arrive_cluster(cta_addr(aother, 0));
+        if (warp == kTMma) {
+            // ------------------------------ twiddle loads and MMAs ------------------------------
+            // The whole warp runs this and the leader lane issues: in a branch of one lane every descriptor
+            // would be computed in vector registers and moved over (3 % of the 1- and 2-term forms).
+            if (MODE != 3) {
+                const uint32_t leader = lane == 0;
+                uint32_t p_bfull = 0, p_tfree = 0, p_a = 0, p_lo = 0;
+                const unsigned char* a_cur = nullptr;
+                uint32_t s = 0, pass = 0;
+                bool ok = true;
+                // a wait of the whole warp
+                auto wait = [&](uint32_t bar, uint32_t parity) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, wlim)) && ok;
+                };
+                const Desc da = tdesc(smem0, kTALbo, kTASbo), db = tdesc(smem0 + (uint32_t)C::SM_A, C::B_LBO, C::B_SBO);
+                const Desc dl = tdesc(smem0 + (uint32_t)C::SM_A + C::B_STAGE, kTALbo, kTASbo);    // lo twiddles
+                int seg_cursor = 0;
+                for (int un = pair; un < units.n_units && ok; un += npairs) {
+                    int item, ps0, ps1;
+                    pass_unit(units, un, item, ps0, ps1);
+                    while (seg_cursor + 1 < bt.n_segs && bt.segs[seg_cursor + 1].item_begin <= item) ++seg_cursor;
+                    const unsigned char* a_img = bt.segs[seg_cursor].a_img;
+                    if (a_img != a_cur) {
+                        if (a_cur) {
+                            // the MMAs that read the old twiddles are complete before they are replaced
+                            if (rank == 0) tcommit(leader, adone);
+                            wait(adone, (p_a >> 1) & 1u);
+                            p_a ^= 2u;
+                        }
+                        if (leader) {
+                            expect_tx(afull, (uint32_t)C::SM_A);
+    #pragma unroll 1
+                            for (int kc = 0; kc < kTNch; ++kc)
+                                bulk_g2s(smem0 + (uint32_t)(kc * 2 * kTTw), a_img + (size_t)(kc * 2 + (int)rank) * (2 * kTTw),
+                                         2 * kTTw, afull);
+                        }
                         __syncwarp();
-                    } else {
-                        wait(aother, p_a & 1u);
-                    }
-                    p_a ^= 1u;
-                    a_cur = a_img;
-                }
-                for (int ps = ps0; ps < ps1 && ok; ++ps, ++pass) {
-                    if (rank == 1 && !C::A_LO) continue;
-                    const uint32_t buf = pass & 1u;
-                    if (rank == 0 && pass >= 2) {
-                        // the up-channel warps of both CTAs have read this accumulator half (pass - 2)
-                        wait(tfree((int)buf), (p_tfree >> buf) & 1u);
-                        p_tfree ^= 1u << buf;
-                    }
-                    const uint32_t re = tmem + 256u * buf, im = re + 128u;
-#pragma unroll 1
-                    for (int kc = 0; kc < kTNch && ok; ++kc) {
+                        wait(afull, p_a & 1u);
                         if (rank == 1) {
-                            // 3 terms: this CTA's lo twiddles of the stage have landed
-                            wait(lofull((int)s), (p_lo >> s) & 1u);
-                            p_lo ^= 1u << s;
-                            if (ok && leader) arrive_cluster(cta_addr(bfull((int)s), 0));
+                            if (leader) arrive_cluster(cta_addr(aother, 0));
                             __syncwarp();
                         } else {
-                            wait(bfull((int)s), (p_bfull >> s) & 1u);
-                            p_bfull ^= 1u << s;
-                            if (!ok) break;
-                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                            const uint32_t a0 = da.lo + (uint32_t)kc * (2 * kTTw / 16), b0 = db.lo + s * (C::STAGE / 16u);
-                            const uint32_t l0 = dl.lo + s * (C::STAGE / 16u);
-#pragma unroll
-                            for (int ks = 0; ks < kTFeeds / 16; ++ks) {
-                                const uint32_t c = a0 + ks * (2 * kTALbo / 16), sn = c + kTTw / 16;
-                                const uint32_t yr = b0 + ks * (2 * C::B_LBO / 16), yi = yr + 128 / 16;
-                                const uint32_t more = (kc | ks) ? 1u : 0u;
-                                tmma(leader, re, c, da.hi, yr, db.hi, kTIdesc, more);
-                                tmma(leader, im, c, da.hi, yi, db.hi, kTIdesc, more);
-                                tmma(leader, re, sn, da.hi, yi, db.hi, kTIdesc, 1u);
-                                tmma(leader, im, sn, da.hi, yr, db.hi, kTIdescNeg, 1u);
-                                if constexpr (C::B_LO) {
-                                    const uint32_t zr = yr + 256 / 16, zi = yr + 384 / 16;
-                                    tmma(leader, re, c, da.hi, zr, db.hi, kTIdesc, 1u);
-                                    tmma(leader, im, c, da.hi, zi, db.hi, kTIdesc, 1u);
-                                    tmma(leader, re, sn, da.hi, zi, db.hi, kTIdesc, 1u);
-                                    tmma(leader, im, sn, da.hi, zr, db.hi, kTIdescNeg, 1u);
-                                }
-                                if constexpr (C::A_LO) {
-                                    const uint32_t cl = l0 + ks * (2 * kTALbo / 16), sl = cl + kTTw / 16;
-                                    tmma(leader, re, cl, da.hi, yr, db.hi, kTIdesc, 1u);
-                                    tmma(leader, im, cl, da.hi, yi, db.hi, kTIdesc, 1u);
-                                    tmma(leader, re, sl, da.hi, yi, db.hi, kTIdesc, 1u);
-                                    tmma(leader, im, sl, da.hi, yr, db.hi, kTIdescNeg, 1u);
-                                }
-                            }
-                            tcommit(leader, bempty((int)s));
-                            if (kc == kTNch - 1) tcommit(leader, accfull((int)buf));
+                            wait(aother, p_a & 1u);
                         }
-                        if (++s == (uint32_t)NB) s = 0;
+                        p_a ^= 1u;
+                        a_cur = a_img;
                     }
-                    if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;
+                    for (int ps = ps0; ps < ps1 && ok; ++ps, ++pass) {
+                        if (rank == 1 && !C::A_LO) continue;
+                        const uint32_t buf = pass & 1u;
+                        if (rank == 0 && pass >= 2) {
+                            // the up-channel warps of both CTAs have read this accumulator half (pass - 2)
+                            wait(tfree((int)buf), (p_tfree >> buf) & 1u);
+                            p_tfree ^= 1u << buf;
+                        }
+                        const uint32_t re = tmem + 256u * buf, im = re + 128u;
+    #pragma unroll 1
+                        for (int kc = 0; kc < kTNch && ok; ++kc) {
+                            if (rank == 1) {
+                                // 3 terms: this CTA's lo twiddles of the stage have landed
+                                wait(lofull((int)s), (p_lo >> s) & 1u);
+                                p_lo ^= 1u << s;
+                                if (ok && leader) arrive_cluster(cta_addr(bfull((int)s), 0));
+                                __syncwarp();
+                            } else {
+                                wait(bfull((int)s), (p_bfull >> s) & 1u);
+                                p_bfull ^= 1u << s;
+                                if (!ok) break;
+                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                                const uint32_t a0 = da.lo + (uint32_t)kc * (2 * kTTw / 16), b0 = db.lo + s * (C::STAGE / 16u);
+                                const uint32_t l0 = dl.lo + s * (C::STAGE / 16u);
+    #pragma unroll
+                                for (int ks = 0; ks < kTFeeds / 16; ++ks) {
+                                    const uint32_t c = a0 + ks * (2 * kTALbo / 16), sn = c + kTTw / 16;
+                                    const uint32_t yr = b0 + ks * (2 * C::B_LBO / 16), yi = yr + 128 / 16;
+                                    const uint32_t more = (kc | ks) ? 1u : 0u;
+                                    tmma(leader, re, c, da.hi, yr, db.hi, kTIdesc, more);
+                                    tmma(leader, im, c, da.hi, yi, db.hi, kTIdesc, more);
+                                    tmma(leader, re, sn, da.hi, yi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, sn, da.hi, yr, db.hi, kTIdescNeg, 1u);
+                                    if constexpr (C::B_LO) {
+                                        const uint32_t zr = yr + 256 / 16, zi = yr + 384 / 16;
+                                        tmma(leader, re, c, da.hi, zr, db.hi, kTIdesc, 1u);
+                                        tmma(leader, im, c, da.hi, zi, db.hi, kTIdesc, 1u);
+                                        tmma(leader, re, sn, da.hi, zi, db.hi, kTIdesc, 1u);
+                                        tmma(leader, im, sn, da.hi, zr, db.hi, kTIdescNeg, 1u);
+                                    }
+                                    if constexpr (C::A_LO) {
+                                        const uint32_t cl = l0 + ks * (2 * kTALbo / 16), sl = cl + kTTw / 16;
+                                        tmma(leader, re, cl, da.hi, yr, db.hi, kTIdesc, 1u);
+                                        tmma(leader, im, cl, da.hi, yi, db.hi, kTIdesc, 1u);
+                                        tmma(leader, re, sl, da.hi, yi, db.hi, kTIdesc, 1u);
+                                        tmma(leader, im, sl, da.hi, yr, db.hi, kTIdescNeg, 1u);
+                                    }
+                                }
+                                tcommit(leader, bempty((int)s));
+                                if (kc == kTNch - 1) tcommit(leader, accfull((int)buf));
+                            }
+                            if (++s == (uint32_t)NB) s = 0;
+                        }
+                        if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;
+                    }
                 }
+                // every issued MMA is complete before shared and tensor memory are released
+                if (rank == 0) tcommit(leader, adone);
+                wait(adone, (p_a >> 1) & 1u);
+                if (!ok) abort_s = 1;
             }
-            // every issued MMA is complete before shared and tensor memory are released
-            if (rank == 0) tcommit(leader, adone);
-            wait(adone, (p_a >> 1) & 1u);
+        } else {
+            // ------------------------------ builders ------------------------------
+            // The warps take the CTA's tasks (unit, pass, chunk, group of 8 times) in turn.  Lane bits 0-1 take
+            // the four feed octets of a chunk, bits 2-4 eight times: a quarter warp loads 64 contiguous bytes
+            // of two rows (lanes on eight different lines at one offset instead take a pass of the L1 data
+            // banks each: 1.29 ms per 4 x 49152-sample request against 1.16)
+            const int t = 64 * (int)rank + (lane >> 2), oct = lane & 3;
+            unsigned char* dst0 = ring + oct * C::B_LBO + (lane >> 2) * 16;
+            const uint32_t full0 = cta_addr(bar0, 0);                      // the first CTA's bfull(0)
+            // the next task, whose rows are loaded while the current one is built
+            int un = pair, ps = 0, ps1 = 0, kc = warp / kTGroups, g = warp % kTGroups, sgi = 0, F = 0, j = 0;
+            bool more = un < units.n_units, new_unit = true, new_pass = true;
+            auto enter_unit = [&] {
+                int item;
+                pass_unit(units, un, item, ps, ps1);
+                while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
+                const int local = item - bt.segs[sgi].item_begin;
+                F = local >> 2;
+                j = local & 3;
+            };
+            // this thread's part of the rows of a block in the carried and in the new samples, and the first
+            // of its rows that is new
+            const uint8_t *carried = nullptr, *fresh = nullptr;
+            int first_fresh = 0;
+            auto enter_block = [&] {
+                const Seg& sg = bt.segs[sgi];
+                const long long row0 = (long long)F * kFrame + (ps >> 1) * kUp;
+                const long long left = sg.carry_rows - row0;
+                first_fresh = left < 0 ? 0 : left < kUp ? (int)left : kUp;
+                carried = sg.carry + row0 * kInput + 16 * oct;
+                fresh = sg.vin - left * kInput + 16 * oct;
+            };
+            auto load_task = [&](RawT& r) {
+                const int row = t + 8 * g;
+                load_raw((row < first_fresh ? carried : fresh) + (uint32_t)(row * kInput), kc, r);
+            };
+            uint32_t s = (uint32_t)(warp / kTGroups), parity = 1;             // a fresh barrier passes a wait on parity 1
+            // A wait for a stage's previous use must not pass on the use before that one.  The warp's previous task
+            // saw the release of the stage NB chunks before it, and commits are in order, so that use is over
+            // if the warp advances by at most NB chunks at a time.
+            static_assert((kTBuild + kTGroups - 1) / kTGroups <= C::NB, "a builder's step between tasks");
+            bool ok = true;
+            EwW w;
+            PolSel sel;
+            // builds the task whose rows are in cur and loads the one after it
+            auto task = [&](const RawT& cur, RawT& nxt) {
+                if (new_pass) {
+                    if (new_unit) load_ew_frame(bt.segs[sgi], bt.ew, F, j, w);
+                    sel = pol_sel(ps & 1);
+                    if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;   // the warp stops as one
+                }
+                const int g0 = g, kc0 = kc, sg0 = sgi;
+                new_unit = new_pass = false;
+                uint32_t ds = kTBuild / kTGroups;
+                g += kTBuild % kTGroups;
+                if (g >= kTGroups) {
+                    g -= kTGroups;
+                    ++ds;
+                }
+                kc += (int)ds;
+                if (kc >= kTNch) {
+                    kc -= kTNch;
+                    new_pass = true;
+                    if (++ps == ps1) {
+                        un += npairs;
+                        new_unit = true;
+                        more = un < units.n_units;
+                        if (more) enter_unit();
+                    }
+                    if (more) enter_block();
+                }
+                if (more) load_task(nxt);
+                // the MMAs have read stage s in both CTAs
+                if (!mbar_wait(bempty((int)s), parity, wlim)) ok = false;
+                // the warp stops as one (a wait expired in any lane)
+                if (!__all_sync(0xffffffffu, ok)) {
+                    ok = false;
+                    return;
+                }
+                if constexpr (C::A_LO) {
+                    if (g0 == 0 && lane == 0) {
+                        // the chunk's lo twiddles (second half of the image) into the stage
+                        const uint32_t bar = rank == 0 ? bfull((int)s) : lofull((int)s);
+                        expect_tx(bar, 2 * kTTw);
+                        bulk_g2s(smem0 + (uint32_t)C::SM_A + s * (uint32_t)C::STAGE + (uint32_t)C::B_STAGE,
+                                 bt.segs[sg0].a_img + 2 * C::SM_A + (size_t)(kc0 * 2 + (int)rank) * (2 * kTTw), 2 * kTTw, bar);
+                    }
+                }
+                build<TERMS>(cur, sel, w, dst0 + s * (uint32_t)C::STAGE + g0 * C::B_SBO);
+                // the generic-proxy stores are visible to the tensor cores
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) arrive_cluster(full0 + 8u * s);
+                s += ds;
+                if (s >= (uint32_t)C::NB) {
+                    s -= (uint32_t)C::NB;
+                    parity ^= 1u;
+                }
+            };
+            // two tasks per loop body: the raw rows alternate between registers without copies
+            RawT ra, rb;
+            if (more) {
+                enter_unit();
+                enter_block();
+                load_task(ra);
+            }
+            while (more && ok) {
+                task(ra, rb);
+                if (!more || !ok) break;
+                task(rb, ra);
+            }
             if (!ok) abort_s = 1;
         }
-    } else if (warp < kTBuild) {
-        // ------------------------------ builders ------------------------------
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" :: "n"(kTRegBuild) : "memory");
-        // The warps take the CTA's tasks (unit, pass, chunk, group of 8 times) in turn.  Lane bits 0-1 take
-        // the four feed octets of a chunk, bits 2-4 eight times: a quarter warp loads 64 contiguous bytes
-        // of two rows (lanes on eight different lines at one offset instead take a pass of the L1 data
-        // banks each: 1.29 ms per 4 x 49152-sample request against 1.16)
-        const int wu = (int)uniform((uint32_t)warp);
-        const int t = 64 * (int)rank + (lane >> 2), oct = lane & 3;
-        unsigned char* dst0 = ring + oct * C::B_LBO + (lane >> 2) * 16;
-        const uint32_t full0 = cta_addr(bar0, 0);                      // the first CTA's bfull(0)
-        // the next task, whose rows are loaded while the current one is built
-        int un = pair, ps = 0, ps1 = 0, kc = wu / kTGroups, g = wu % kTGroups, sgi = 0, F = 0, j = 0;
-        bool more = un < units.n_units, new_unit = true, new_pass = true;
-        auto enter_unit = [&] {
-            int item;
-            pass_unit(units, un, item, ps, ps1);
-            while (sgi + 1 < bt.n_segs && bt.segs[sgi + 1].item_begin <= item) ++sgi;
-            const int local = item - bt.segs[sgi].item_begin;
-            F = local >> 2;
-            j = local & 3;
-        };
-        // this thread's part of the rows of a block in the carried and in the new samples, and the first
-        // of its rows that is new
-        const uint8_t *carried = nullptr, *fresh = nullptr;
-        int first_fresh = 0;
-        auto enter_block = [&] {
-            const Seg& sg = bt.segs[sgi];
-            const long long row0 = (long long)F * kFrame + (ps >> 1) * kUp;
-            const long long left = sg.carry_rows - row0;
-            first_fresh = left < 0 ? 0 : left < kUp ? (int)left : kUp;
-            carried = sg.carry + row0 * kInput + 16 * oct;
-            fresh = sg.vin - left * kInput + 16 * oct;
-        };
-        auto load_task = [&](RawT& r) {
-            const int row = t + 8 * g;
-            load_raw((row < first_fresh ? carried : fresh) + (uint32_t)(row * kInput), kc, r);
-        };
-        uint32_t s = (uint32_t)(wu / kTGroups), parity = 1;             // a fresh barrier passes a wait on parity 1
-        // A wait for a stage's previous use must not pass on the use before that one.  The warp's previous task
-        // saw the release of the stage NB chunks before it, and commits are in order, so that use is over
-        // if the warp advances by at most NB chunks at a time.
-        static_assert((kTBuild + kTGroups - 1) / kTGroups <= C::NB, "a builder's step between tasks");
-        bool ok = true;
-        EwW w;
-        PolSel sel;
-        // builds the task whose rows are in cur and loads the one after it
-        auto task = [&](const RawT& cur, RawT& nxt) {
-            if (new_pass) {
-                if (new_unit) load_ew_frame(bt.segs[sgi], bt.ew, F, j, w);
-                sel = pol_sel(ps & 1);
-                if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;   // the warp stops as one
-            }
-            const int g0 = g, kc0 = kc, sg0 = sgi;
-            new_unit = new_pass = false;
-            uint32_t ds = kTBuild / kTGroups;
-            g += kTBuild % kTGroups;
-            if (g >= kTGroups) {
-                g -= kTGroups;
-                ++ds;
-            }
-            kc += (int)ds;
-            if (kc >= kTNch) {
-                kc -= kTNch;
-                new_pass = true;
-                if (++ps == ps1) {
-                    un += npairs;
-                    new_unit = true;
-                    more = un < units.n_units;
-                    if (more) enter_unit();
-                }
-                if (more) enter_block();
-            }
-            if (more) load_task(nxt);
-            // the MMAs have read stage s in both CTAs
-            if (!mbar_wait(bempty((int)s), parity, wlim)) ok = false;
-            // the warp stops as one (a wait expired in any lane)
-            if (!__all_sync(0xffffffffu, ok)) {
-                ok = false;
-                return;
-            }
-            if constexpr (C::A_LO) {
-                if (g0 == 0 && lane == 0) {
-                    // the chunk's lo twiddles (second half of the image) into the stage
-                    const uint32_t bar = rank == 0 ? bfull((int)s) : lofull((int)s);
-                    expect_tx(bar, 2 * kTTw);
-                    bulk_g2s(smem0 + (uint32_t)C::SM_A + s * (uint32_t)C::STAGE + (uint32_t)C::B_STAGE,
-                             bt.segs[sg0].a_img + 2 * C::SM_A + (size_t)(kc0 * 2 + (int)rank) * (2 * kTTw), 2 * kTTw, bar);
-                }
-            }
-            build<TERMS>(cur, sel, w, dst0 + s * (uint32_t)C::STAGE + g0 * C::B_SBO);
-            // the generic-proxy stores are visible to the tensor cores
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) arrive_cluster(full0 + 8u * s);
-            s += ds;
-            if (s >= (uint32_t)C::NB) {
-                s -= (uint32_t)C::NB;
-                parity ^= 1u;
-            }
-        };
-        // two tasks per loop body: the raw rows alternate between registers without copies
-        RawT ra, rb;
-        if (more) {
-            enter_unit();
-            enter_block();
-            load_task(ra);
-        }
-        while (more && ok) {
-            task(ra, rb);
-            if (!more || !ok) break;
-            task(rb, ra);
-        }
-        if (!ok) abort_s = 1;
     } else {
         // ------------------------------ up-channel warps ------------------------------
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" :: "n"(kTRegUp) : "memory");
