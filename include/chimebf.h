@@ -274,15 +274,17 @@ int bf_debug_gather_order(const bf_config* cfg, double freq_hz, int16_t* order_o
 int bf_debug_gemm(bf_plan_t p, double freq_hz, const uint8_t* d_vin, int64_t n_samples, float* d_out);
 
 /* Failure-detection check of the device-side waits (no counterpart in the
- * paper): runs a tensor-core kernel on one frame (d_vin: device, 384 x 2048
- * bytes, 16-byte aligned) with its MMA thread idle, so no pipeline stage is
- * ever released, and every mbarrier wait bounded by wait_ns (1 .. 2e9).  The
- * kernel is the 1-term tensor-core kernel (one cluster of two CTAs), whatever
- * the plan's form.  It neither traps nor spins unbounded: its waits run out, it frees its tensor
- * memory and reports through the plan's status word, and the call returns
- * BF_ETIMEDOUT, after which the plan and the CUDA context remain usable.
- * BF_OK would mean a wait did not expire.  Any plan form may call it; it
- * synchronises the plan's stream. */
+ * paper): runs the plan's tensor-core kernel (an FP32 plan: the 1-term one) on
+ * one frame (d_vin: device, 384 x 2048 bytes, 16-byte aligned) on one cluster of
+ * two CTAs, with every mbarrier wait bounded by wait_ns (1 .. 2e9) and a part of
+ * it stopped: its MMA warps, idle from the start and then again after some
+ * chunks, and the warps that build its data likewise (an FP32 plan: MMA warps
+ * idle only).  The kernel neither traps nor spins unbounded: its waits run out, it
+ * lets its copies and MMAs under way finish, frees its tensor memory and reports
+ * through the plan's status word, and the call returns BF_ETIMEDOUT, after which
+ * the plan and the CUDA context remain usable.  BF_OK would mean a run in
+ * which no wait expired.  Any plan form may call it; it synchronises the
+ * plan's stream. */
 int bf_debug_stall(bf_plan_t p, const uint8_t* d_vin, int64_t wait_ns);
 
 /* Device unpack of n bytes into 2n floats (re, im), with the same device

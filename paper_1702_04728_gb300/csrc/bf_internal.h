@@ -72,6 +72,8 @@ struct Batch {
     float2* dump;            // debug: up-channelised voltages instead of detection
     int* status;                 // set non-zero by a kernel whose bounded wait expired
     unsigned long long wait_ns;  // bound on each device-side wait (0: the default, 2 s)
+    int stall_mma;               // stall check: the MMA warps (else the builders) stop ...
+    int stall_chunks;            // ... after this many chunks of 32 feeds
     PassUnits units;             // work units of the launch
     float* part;                 // sums of split items' passes [CTAs][6][16][256]
     unsigned long long* part_tok;    // [CTAs][256] passes published (see add_passes)
@@ -88,9 +90,9 @@ cudaError_t debug_unpack_launch(const uint8_t* in, float* out, long long n, cuda
 int fused_fp32_max_grid(int device);   // CTAs that fit at once (1 per SM)
 
 // Tensor-core form on `pairs` clusters of two CTAs over b.units: `terms` = 1, 2 or 3 GEMM terms; mode
-// 0 = detect, 1 = dump up-channelised voltages, 2 = dump the N-S/E-W beams of the GEMM, 3 = stall check
-// (1 term only): the MMA thread stays idle, so the other waits run out and the kernel reports through
-// `status`.
+// 0 = detect, 1 = dump up-channelised voltages, 2 = dump the N-S/E-W beams of the GEMM, 3 = stall check:
+// the MMA warps or the builders stop (b.stall_mma, b.stall_chunks), so the other warps' waits run out and the
+// kernel reports through `status`.
 cudaError_t fused_tc_launch(const Batch& b, int terms, int mode, int pairs, cudaStream_t s);
 // Tensor-core form: a table's twiddle image, C (part 0) and S (part 1) = cos and sin of 2 pi n L(m) / 512
 // in FP16, in the order of the kernel's shared memory operand: chunks of kTFeeds feeds, the CTAs of a

@@ -75,9 +75,9 @@ struct TcCfg {
     static constexpr int B_STAGE = kTGroups * B_SBO;                   // 64 times
     static constexpr int STAGE = B_STAGE + (A_LO ? 2 * kTTw : 0);      // and the chunk's lo twiddles
     static constexpr int NB = TERMS == 1 ? 6 : TERMS == 2 ? 5 : 3;     // ring stages
-    // arrivals on "stage full" in the first CTA: the builder warps of both CTAs; 3 terms: both
-    // CTAs' lo twiddles
-    static constexpr int FULL = 2 * kTGroups + (A_LO ? 2 : 0);
+    // arrivals on "stage full" in the first CTA: the build tasks of both CTAs (one of the first CTA's also
+    // for its lo twiddles); 3 terms: the second CTA's lo twiddles
+    static constexpr int FULL = 2 * kTGroups + (A_LO ? 1 : 0);
     static constexpr int BARS = 3 * NB + 7;
     static constexpr size_t SM_A = (size_t)kTNch * 2 * kTTw;           // 128 KB
     static constexpr size_t SM_RING = (size_t)NB * STAGE;
@@ -215,8 +215,8 @@ __device__ __forceinline__ void build(const RawT& raw, const PolSel& ps, const E
 }
 
 // MODE: 0 = detect and integrate, 1 = dump up-channelised voltages, 2 = dump the N-S/E-W beams of
-//       the GEMM, 3 = stall check (the MMA thread stays idle, so no stage is ever released and
-//       every other wait runs out against the launch's bound).
+//       the GEMM, 3 = stall check (the MMA warps or the builders stop after bt.stall_chunks chunks, so
+//       the other warps' waits run out against the launch's bound).
 template <int TERMS, int MODE>
 __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_constant__ Batch bt) {
     using C = TcCfg<TERMS>;
@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
+    __shared__ uint32_t lo_last_s[NB];     // 3 terms: phase of lofull that the stage's last copy completes
     unsigned char* ring = smem + C::SM_A;
     float4* tw_s = reinterpret_cast<float4*>(ring + C::SM_RING);
     uint64_t* mbar_s = reinterpret_cast<uint64_t*>(reinterpret_cast<unsigned char*>(tw_s) + C::SM_TW);
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
     const uint32_t bar0 = static_cast<uint32_t>(__cvta_generic_to_shared(&mbar_s[0]));
     auto bfull = [&](int s) { return bar0 + 8u * (uint32_t)s; };               // first CTA: stage s of both CTAs
     auto bempty = [&](int s) { return bar0 + 8u * (uint32_t)(NB + s); };       // MMA commit
-    auto lofull = [&](int s) { return bar0 + 8u * (uint32_t)(2 * NB + s); };   // second CTA's lo twiddles
+    auto lofull = [&](int s) { return bar0 + 8u * (uint32_t)(2 * NB + s); };   // this CTA's lo twiddles
     auto accfull = [&](int b) { return bar0 + 8u * (uint32_t)(3 * NB + b); };  // last commit of a pass
     auto tfree = [&](int b) { return bar0 + 8u * (uint32_t)(3 * NB + 2 + b); };    // first CTA: both CTAs' up-channel warps
     const uint32_t afull = bar0 + 8u * (uint32_t)(3 * NB + 4);                 // this CTA's resident twiddles
@@ -255,6 +256,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
             init(bfull(i), C::FULL);
             init(bempty(i), 1);
             init(lofull(i), 1);
+            lo_last_s[i] = 1;              // a fresh barrier passes a wait on parity 1
         }
         for (int i = 0; i < 2; ++i) {
             init(accfull(i), 1);
@@ -286,12 +288,15 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
             // ------------------------------ twiddle loads and MMAs ------------------------------
             // The whole warp runs this and the leader lane issues: in a branch of one lane every descriptor
             // would be computed in vector registers and moved over (3 % of the 1- and 2-term forms).
-            if (MODE != 3) {
+            const int stall_at = MODE == 3 && bt.stall_mma ? bt.stall_chunks : -1;
+            if (stall_at != 0) {
                 const uint32_t leader = lane == 0;
                 uint32_t p_bfull = 0, p_tfree = 0, p_a = 0, p_lo = 0;
                 const unsigned char* a_cur = nullptr;
                 uint32_t s = 0, pass = 0;
-                bool ok = true;
+                uint32_t a_last = 1;               // phase that the last load of resident twiddles completes
+                bool ok = true, stalled = false;
+                int chunks = 0;
                 // a wait of the whole warp
                 auto wait = [&](uint32_t bar, uint32_t parity) {
                     ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, wlim)) && ok;
@@ -311,9 +316,10 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                             wait(adone, (p_a >> 1) & 1u);
                             p_a ^= 2u;
                         }
+                        a_last = p_a & 1u;
                         if (leader) {
                             expect_tx(afull, (uint32_t)C::SM_A);
-    #pragma unroll 1
+#pragma unroll 1
                             for (int kc = 0; kc < kTNch; ++kc)
                                 bulk_g2s(smem0 + (uint32_t)(kc * 2 * kTTw), a_img + (size_t)(kc * 2 + (int)rank) * (2 * kTTw),
                                          2 * kTTw, afull);
@@ -330,65 +336,79 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                         a_cur = a_img;
                     }
                     for (int ps = ps0; ps < ps1 && ok; ++ps, ++pass) {
-                        if (rank == 1 && !C::A_LO) continue;
+                        if (rank == 1) {
+                            if constexpr (C::A_LO) {
+#pragma unroll 1
+                                for (int kc = 0; kc < kTNch && ok; ++kc) {
+                                    // this CTA's lo twiddles of the stage have landed
+                                    wait(lofull((int)s), (p_lo >> s) & 1u);
+                                    p_lo ^= 1u << s;
+                                    if (ok && leader) arrive_cluster(cta_addr(bfull((int)s), 0));
+                                    __syncwarp();
+                                    if (++s == (uint32_t)NB) s = 0;
+                                }
+                                if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;
+                            }
+                            continue;
+                        }
                         const uint32_t buf = pass & 1u;
-                        if (rank == 0 && pass >= 2) {
+                        if (pass >= 2) {
                             // the up-channel warps of both CTAs have read this accumulator half (pass - 2)
                             wait(tfree((int)buf), (p_tfree >> buf) & 1u);
                             p_tfree ^= 1u << buf;
                         }
                         const uint32_t re = tmem + 256u * buf, im = re + 128u;
-    #pragma unroll 1
+#pragma unroll 1
                         for (int kc = 0; kc < kTNch && ok; ++kc) {
-                            if (rank == 1) {
-                                // 3 terms: this CTA's lo twiddles of the stage have landed
-                                wait(lofull((int)s), (p_lo >> s) & 1u);
-                                p_lo ^= 1u << s;
-                                if (ok && leader) arrive_cluster(cta_addr(bfull((int)s), 0));
-                                __syncwarp();
-                            } else {
-                                wait(bfull((int)s), (p_bfull >> s) & 1u);
-                                p_bfull ^= 1u << s;
-                                if (!ok) break;
-                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                const uint32_t a0 = da.lo + (uint32_t)kc * (2 * kTTw / 16), b0 = db.lo + s * (C::STAGE / 16u);
-                                const uint32_t l0 = dl.lo + s * (C::STAGE / 16u);
-    #pragma unroll
-                                for (int ks = 0; ks < kTFeeds / 16; ++ks) {
-                                    const uint32_t c = a0 + ks * (2 * kTALbo / 16), sn = c + kTTw / 16;
-                                    const uint32_t yr = b0 + ks * (2 * C::B_LBO / 16), yi = yr + 128 / 16;
-                                    const uint32_t more = (kc | ks) ? 1u : 0u;
-                                    tmma(leader, re, c, da.hi, yr, db.hi, kTIdesc, more);
-                                    tmma(leader, im, c, da.hi, yi, db.hi, kTIdesc, more);
-                                    tmma(leader, re, sn, da.hi, yi, db.hi, kTIdesc, 1u);
-                                    tmma(leader, im, sn, da.hi, yr, db.hi, kTIdescNeg, 1u);
-                                    if constexpr (C::B_LO) {
-                                        const uint32_t zr = yr + 256 / 16, zi = yr + 384 / 16;
-                                        tmma(leader, re, c, da.hi, zr, db.hi, kTIdesc, 1u);
-                                        tmma(leader, im, c, da.hi, zi, db.hi, kTIdesc, 1u);
-                                        tmma(leader, re, sn, da.hi, zi, db.hi, kTIdesc, 1u);
-                                        tmma(leader, im, sn, da.hi, zr, db.hi, kTIdescNeg, 1u);
-                                    }
-                                    if constexpr (C::A_LO) {
-                                        const uint32_t cl = l0 + ks * (2 * kTALbo / 16), sl = cl + kTTw / 16;
-                                        tmma(leader, re, cl, da.hi, yr, db.hi, kTIdesc, 1u);
-                                        tmma(leader, im, cl, da.hi, yi, db.hi, kTIdesc, 1u);
-                                        tmma(leader, re, sl, da.hi, yi, db.hi, kTIdesc, 1u);
-                                        tmma(leader, im, sl, da.hi, yr, db.hi, kTIdescNeg, 1u);
-                                    }
+                            if constexpr (MODE == 3) {
+                                if (chunks++ == stall_at) {
+                                    stalled = true;
+                                    ok = false;
+                                    break;
                                 }
-                                tcommit(leader, bempty((int)s));
-                                if (kc == kTNch - 1) tcommit(leader, accfull((int)buf));
                             }
+                            wait(bfull((int)s), (p_bfull >> s) & 1u);
+                            p_bfull ^= 1u << s;
+                            if (!ok) break;
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                            const uint32_t a0 = da.lo + (uint32_t)kc * (2 * kTTw / 16), b0 = db.lo + s * (C::STAGE / 16u);
+                            const uint32_t l0 = dl.lo + s * (C::STAGE / 16u);
+#pragma unroll
+                            for (int ks = 0; ks < kTFeeds / 16; ++ks) {
+                                const uint32_t c = a0 + ks * (2 * kTALbo / 16), sn = c + kTTw / 16;
+                                const uint32_t yr = b0 + ks * (2 * C::B_LBO / 16), yi = yr + 128 / 16;
+                                const uint32_t more = (kc | ks) ? 1u : 0u;
+                                tmma(leader, re, c, da.hi, yr, db.hi, kTIdesc, more);
+                                tmma(leader, im, c, da.hi, yi, db.hi, kTIdesc, more);
+                                tmma(leader, re, sn, da.hi, yi, db.hi, kTIdesc, 1u);
+                                tmma(leader, im, sn, da.hi, yr, db.hi, kTIdescNeg, 1u);
+                                if constexpr (C::B_LO) {
+                                    const uint32_t zr = yr + 256 / 16, zi = yr + 384 / 16;
+                                    tmma(leader, re, c, da.hi, zr, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, c, da.hi, zi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, re, sn, da.hi, zi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, sn, da.hi, zr, db.hi, kTIdescNeg, 1u);
+                                }
+                                if constexpr (C::A_LO) {
+                                    const uint32_t cl = l0 + ks * (2 * kTALbo / 16), sl = cl + kTTw / 16;
+                                    tmma(leader, re, cl, da.hi, yr, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, cl, da.hi, yi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, re, sl, da.hi, yi, db.hi, kTIdesc, 1u);
+                                    tmma(leader, im, sl, da.hi, yr, db.hi, kTIdescNeg, 1u);
+                                }
+                            }
+                            tcommit(leader, bempty((int)s));
+                            if (kc == kTNch - 1) tcommit(leader, accfull((int)buf));
                             if (++s == (uint32_t)NB) s = 0;
                         }
                         if (__any_sync(0xffffffffu, *(volatile int*)&abort_s != 0)) ok = false;
                     }
                 }
-                // every issued MMA is complete before shared and tensor memory are released
+                // every issued MMA and load is complete before shared and tensor memory are released
                 if (rank == 0) tcommit(leader, adone);
                 wait(adone, (p_a >> 1) & 1u);
-                if (!ok) abort_s = 1;
+                wait(afull, a_last);
+                if (!ok && !stalled) abort_s = 1;
             }
         } else {
             // ------------------------------ builders ------------------------------
@@ -432,6 +452,8 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
             // if the warp advances by at most NB chunks at a time.
             static_assert((kTBuild + kTGroups - 1) / kTGroups <= C::NB, "a builder's step between tasks");
             bool ok = true;
+            int chunks = warp / kTGroups;                               // of the task at hand, from the launch's first
+            const int stall_at = MODE == 3 && !bt.stall_mma ? bt.stall_chunks : -1;
             EwW w;
             PolSel sel;
             // builds the task whose rows are in cur and loads the one after it
@@ -472,18 +494,28 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                 if constexpr (C::A_LO) {
                     if (g0 == 0 && lane == 0) {
                         // the chunk's lo twiddles (second half of the image) into the stage
-                        const uint32_t bar = rank == 0 ? bfull((int)s) : lofull((int)s);
+                        const uint32_t bar = lofull((int)s);
+                        *(volatile uint32_t*)&lo_last_s[s] = parity ^ 1u;
                         expect_tx(bar, 2 * kTTw);
                         bulk_g2s(smem0 + (uint32_t)C::SM_A + s * (uint32_t)C::STAGE + (uint32_t)C::B_STAGE,
                                  bt.segs[sg0].a_img + 2 * C::SM_A + (size_t)(kc0 * 2 + (int)rank) * (2 * kTTw), 2 * kTTw, bar);
                     }
                 }
                 build<TERMS>(cur, sel, w, dst0 + s * (uint32_t)C::STAGE + g0 * C::B_SBO);
+                if constexpr (C::A_LO) {
+                    // in the first CTA the task that requested the chunk's lo twiddles stands for them too (a barrier more
+                    // for the MMA warp to test between two chunks' MMAs costs 2 %, the second CTA's done like this 1 %)
+                    if (rank == 0 && g0 == 0 && !__all_sync(0xffffffffu, mbar_wait(lofull((int)s), parity ^ 1u, wlim))) {
+                        ok = false;
+                        return;
+                    }
+                }
                 // the generic-proxy stores are visible to the tensor cores
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) arrive_cluster(full0 + 8u * s);
                 s += ds;
+                if constexpr (MODE == 3) chunks += (int)ds;
                 if (s >= (uint32_t)C::NB) {
                     s -= (uint32_t)C::NB;
                     parity ^= 1u;
@@ -497,8 +529,10 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                 load_task(ra);
             }
             while (more && ok) {
+                if (MODE == 3 && stall_at >= 0 && chunks >= stall_at) break;
                 task(ra, rb);
                 if (!more || !ok) break;
+                if (MODE == 3 && stall_at >= 0 && chunks >= stall_at) break;
                 task(rb, ra);
             }
             if (!ok) abort_s = 1;
@@ -596,6 +630,12 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if constexpr (C::A_LO) {
+        // no builder issues any more; copies under way when a wait ran out have to land before this memory is
+        // given up (after a run that completed there are none)
+        if (tid < NB) mbar_wait(lofull(tid), lo_last_s[tid], wlim);
+        __syncwarp();
+    }
     // both CTAs are done with each other's barriers and, in a run that completed, with the MMAs
     cluster_sync();
     if (abort_s && tid == 0 && bt.status) atomicExch(bt.status, 1);
@@ -656,9 +696,11 @@ cudaError_t fused_tc_launch(const Batch& b, int terms, int mode, int pairs, cuda
         case 20: return launch_tc<2, 0>(b, pairs, s);
         case 21: return launch_tc<2, 1>(b, pairs, s);
         case 22: return launch_tc<2, 2>(b, pairs, s);
+        case 23: return launch_tc<2, 3>(b, pairs, s);
         case 30: return launch_tc<3, 0>(b, pairs, s);
         case 31: return launch_tc<3, 1>(b, pairs, s);
         case 32: return launch_tc<3, 2>(b, pairs, s);
+        case 33: return launch_tc<3, 3>(b, pairs, s);
         default: return cudaErrorInvalidValue;
     }
 }

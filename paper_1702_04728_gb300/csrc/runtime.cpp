@@ -1283,13 +1283,22 @@ int bf_debug_stall(bf_plan_t p, const uint8_t* d_vin, int64_t wait_ns) {
     b.segs[0].n_frames = 1;
     b.wait_ns = (unsigned long long)wait_ns;
     b.units = pass_units(b.n_items, 1, 6);
-    CK(fused_tc_launch(b, 1, 3, 1, p->stream));
-    CK(cudaStreamSynchronize(p->stream));
-    if (p->h_status && *(volatile int*)p->h_status) {
+    // chunks before the stop: none, and some of the second pass (8 a pass), when the ring has been round and
+    // MMAs and copies are under way.  An FP32 plan has no twiddle image, which the MMA warps load
+    // before their first chunk.
+    const struct {
+        int mma, chunks;
+    } stops[] = {{1, 0}, {1, 13}, {0, 0}, {0, 13}};
+    for (const auto& st : stops) {
+        b.stall_mma = st.mma;
+        b.stall_chunks = st.chunks;
+        CK(fused_tc_launch(b, p->terms ? p->terms : 1, 3, 1, p->stream));
+        CK(cudaStreamSynchronize(p->stream));
+        if (!p->h_status || !*(volatile int*)p->h_status) return BF_OK;
         *(volatile int*)p->h_status = 0;
-        return fail(BF_ETIMEDOUT, "a bounded device-side wait expired (expected in the stall check)");
+        if (!p->terms) break;
     }
-    return BF_OK;
+    return fail(BF_ETIMEDOUT, "a bounded device-side wait expired (expected in the stall check)");
 }
 
 // ---- measurement aid ---------------------------------------------------------------------

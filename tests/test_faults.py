@@ -1,9 +1,10 @@
 """Failure detection without a GPU fault.
 
-* A device-side wait that nothing will release runs out: the tensor-core
-  kernel is launched with its MMA warp idle and a 2 ms bound on every
-  mbarrier wait; it must return BF_ETIMEDOUT quickly (no trap, no unbounded
-  spin), and the plan and the CUDA context must stay usable.
+* A device-side wait that nothing will release runs out: the plan's tensor-core
+  kernel is launched with a 2 ms bound on every mbarrier wait and its MMA warps
+  or its builders stopped, at once or with MMAs and copies under way; it must return
+  BF_ETIMEDOUT quickly (no trap, no unbounded spin), and the plan and the CUDA
+  context must stay usable.
 * A host producer that dies in the middle of its stream (never sends the end
   of the stream) does not hold up the other streams of a serving plan, and
   the plan still drains and frees everything at destroy.
@@ -30,9 +31,9 @@ def rel_err(got, ref):
     return float(np.max(np.abs(np.asarray(got, np.float64) - ref) / np.abs(ref)))
 
 
-# FP32 and 3-term plans run the single-CTA tensor-core kernel's check; the 1-term and
-# 512-row plans run their own cluster kernel's (CTA-to-CTA copies, then an abort drain)
-@pytest.mark.parametrize("form", [B.BF_FP32_FFT, B.BF_TC_DFT256, B.BF_TC_DFT256_X1, B.BF_TC_DFT512])
+# the kernel of the plan's own number of terms (three: low twiddles copied into the stages while the waits run
+# out); FP32 plans the 1-term kernel with its MMA warps idle, 512-row plans the 1-term one
+@pytest.mark.parametrize("form", [B.BF_FP32_FFT, B.BF_TC_DFT256, B.BF_TC_DFT256_X1, B.BF_TC_DFT512, B.BF_TC_DFT256_X2])
 def test_device_wait_expires_and_context_survives(built_lib, form):
     freq = 600e6
     raw = synth.noise_only([freq], 384, seed=60)
