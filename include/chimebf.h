@@ -287,6 +287,12 @@ int bf_debug_gemm(bf_plan_t p, double freq_hz, const uint8_t* d_vin, int64_t n_s
  * plan's stream. */
 int bf_debug_stall(bf_plan_t p, const uint8_t* d_vin, int64_t wait_ns);
 
+/* Bound on each device-side wait of the plan's later launches in nanoseconds (0:
+ * the default, 2 s; at most 2e9).  It is a bound on one hand-off between a
+ * kernel's warps, not on the launch: a launch that lasts longer but moves on stays
+ * below it.  For tests (no counterpart in the paper). */
+int bf_debug_wait_bound(bf_plan_t p, int64_t wait_ns);
+
 /* Device unpack of n bytes into 2n floats (re, im), with the same device
  * code the fused kernel uses.  d_in, d_out device pointers. */
 int bf_debug_unpack(bf_plan_t p, const uint8_t* d_in, float* d_out, int64_t n);

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
     constexpr int NB = C::NB;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s;
+    __shared__ int abort_s, passes_s;      // passes_s: passes that the first up-channel warp has read
     __shared__ uint32_t lo_last_s[NB];     // 3 terms: phase of lofull that the stage's last copy completes
     unsigned char* ring = smem + C::SM_A;
     float4* tw_s = reinterpret_cast<float4*>(ring + C::SM_RING);
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
         init(aother, 1);
         init(adone, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        abort_s = 0;
+        abort_s = passes_s = 0;
     }
     for (int i = tid; i < 64; i += kTThreads) tw_s[i] = kPairTw.w[i >> 3][i & 7];
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -301,6 +301,17 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                 auto wait = [&](uint32_t bar, uint32_t parity) {
                     ok = __all_sync(0xffffffffu, mbar_wait(bar, parity, wlim)) && ok;
                 };
+                // A wait for all MMAs issued so far.  The second CTA's warp comes here while the first has many
+                // passes to go, so the bound is on each pass.
+                auto wait_mma = [&](uint32_t parity) {
+                    bool done;
+                    int seen;
+                    do {
+                        seen = *(volatile int*)&passes_s;
+                        done = __all_sync(0xffffffffu, mbar_wait(adone, parity, wlim));
+                    } while (!done && __any_sync(0xffffffffu, *(volatile int*)&passes_s != seen));
+                    ok = done && ok;
+                };
                 const Desc da = tdesc(smem0, kTALbo, kTASbo), db = tdesc(smem0 + (uint32_t)C::SM_A, C::B_LBO, C::B_SBO);
                 const Desc dl = tdesc(smem0 + (uint32_t)C::SM_A + C::B_STAGE, kTALbo, kTASbo);    // lo twiddles
                 int seg_cursor = 0;
@@ -313,7 +324,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                         if (a_cur) {
                             // the MMAs that read the old twiddles are complete before they are replaced
                             if (rank == 0) tcommit(leader, adone);
-                            wait(adone, (p_a >> 1) & 1u);
+                            wait_mma((p_a >> 1) & 1u);
                             p_a ^= 2u;
                         }
                         a_last = p_a & 1u;
@@ -406,7 +417,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                 }
                 // every issued MMA and load is complete before shared and tensor memory are released
                 if (rank == 0) tcommit(leader, adone);
-                wait(adone, (p_a >> 1) & 1u);
+                wait_mma((p_a >> 1) & 1u);
                 wait(afull, a_last);
                 if (!ok && !stalled) abort_s = 1;
             }
@@ -589,6 +600,7 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) arrive_cluster(free0 + 8u * buf);
+                if (tid == 32 * (kTMma + 1)) *(volatile int*)&passes_s = (int)pass + 1;
                 if constexpr (MODE == 0) {
                     if (whole) {
 #pragma unroll

@@ -144,6 +144,7 @@ struct bf_plan_s {
     float* d_part = nullptr;                  // sums of split items (see Batch::part)
     unsigned long long* d_part_tok = nullptr;
     unsigned long long launches = 0;          // launch epochs handed to the kernels
+    unsigned long long wait_ns = 0;           // bound on the kernels' waits (0: 2 s; see bf_debug_wait_bound)
 
     std::mutex mu;
     std::condition_variable cv;
@@ -466,6 +467,7 @@ Batch make_batch(const bf_plan_s* p) {
     b.status = p->d_status;
     b.part = p->d_part;
     b.part_tok = p->d_part_tok;
+    b.wait_ns = p->wait_ns;
     return b;
 }
 
@@ -1299,6 +1301,13 @@ int bf_debug_stall(bf_plan_t p, const uint8_t* d_vin, int64_t wait_ns) {
         if (!p->terms) break;
     }
     return fail(BF_ETIMEDOUT, "a bounded device-side wait expired (expected in the stall check)");
+}
+
+int bf_debug_wait_bound(bf_plan_t p, int64_t wait_ns) {
+    if (!p || wait_ns < 0 || wait_ns > 2000000000LL) return fail(BF_EINVAL, "bad argument");
+    std::lock_guard<std::mutex> lk(p->mu);
+    p->wait_ns = (unsigned long long)wait_ns;
+    return BF_OK;
 }
 
 // ---- measurement aid ---------------------------------------------------------------------

@@ -51,12 +51,30 @@ def test_device_wait_expires_and_context_survives(built_lib, form):
         assert B.bf_debug_stall(p.handle, vin, 1_000_000) == B.BF_ETIMEDOUT
 
 
+@pytest.mark.parametrize("form", [B.BF_FP32_FFT, B.BF_TC_DFT256, B.BF_TC_DFT256_X2, B.BF_TC_DFT256_X1])
+def test_wait_bound_is_per_hand_off(built_lib, form):
+    """A launch that lasts many times the bound on a wait, but whose warps keep handing on (a pass takes some
+    20 us), completes: the second CTA of a tensor-core pair has no stage to wait for and follows the passes."""
+    n = 384 * 2048
+    gen = torch.Generator(device="cuda").manual_seed(62)
+    vin = torch.randint(0, 256, (1, n, 2048), generator=gen, device="cuda", dtype=torch.uint8)
+    with B.Plan(form=form) as p:
+        want = p.run(vin, [600e6])
+        B.bf_debug_wait_bound(p.handle, 400_000)
+        out = torch.empty_like(want)
+        _, t = p.submit(vin, [600e6], out, stream_id=9, flags=B.BF_END_OF_STREAM)
+        assert p.poll_timed(t)[2][4] > 2e-3
+        assert torch.equal(out, want)
+
+
 def test_stall_check_rejects_bad_bounds(built_lib):
     raw = synth.noise_only([600e6], 384, seed=61)
     with B.Plan() as p:
         vin = dev(raw[0])
         assert B.bf_debug_stall(p.handle, vin, 0) == B.BF_EINVAL
         assert B.bf_debug_stall(p.handle, vin, 3_000_000_000) == B.BF_EINVAL
+        with pytest.raises(B.BfError):
+            B.bf_debug_wait_bound(p.handle, 3_000_000_000)
 
 
 def test_dead_producer_does_not_block_other_streams(built_lib):
