@@ -161,6 +161,8 @@ int bf_submit(bf_plan_t p, const bf_request* r, uint64_t* ticket);
  * Wait up to timeout_us microseconds (0 = just test, <0 = forever) for a
  * ticket.  BF_OK: output written, *n_frames_out set, ticket released.
  * BF_PENDING: still running.  Negative: error (the ticket is released).
+ * On a direct plan the call tests for completion without sleeping for its first
+ * 3 ms (one core busy, the plan open to other threads), then every 60 us or so.
  */
 int bf_poll(bf_plan_t p, uint64_t ticket, int64_t timeout_us, int64_t* n_frames_out);
 

@@ -98,9 +98,13 @@ struct TrackBuf {
     float2* dev = nullptr;
 };
 
+// An event of the plan's pool, back in it with the last reference (dropped under the plan's lock): a batch
+// holds one, and a bf_poll that queries the event outside the lock another.
+using EventRef = std::shared_ptr<CUevent_st>;
+
 struct InflightBatch {
     uint64_t id;
-    cudaEvent_t ev;
+    EventRef ev;
     cudaEvent_t ev_start;                               // before the batch's first kernel (timing)
     std::vector<uint64_t> tickets;
     size_t bytes;
@@ -671,7 +675,8 @@ int launch_jobs(bf_plan_s* p, std::vector<Job>& jobs, size_t bytes) {
     }
     CK(cudaEventRecord(ev_end.ev, p->stream));
     ev_start.kept = ev_end.kept = true;
-    InflightBatch ib{p->next_batch++, ev_end.ev, ev_start.ev, {}, bytes, {}, tb, std::move(held)};
+    EventRef done(ev_end.ev, [p](cudaEvent_t ev) { p->event_pool.push_back(ev); });
+    InflightBatch ib{p->next_batch++, std::move(done), ev_start.ev, {}, bytes, {}, tb, std::move(held)};
     const double t_launch = now_s();
     for (auto& jb : jobs) {
         ib.tickets.push_back(jb.ticket);
@@ -696,13 +701,13 @@ bool retire(bf_plan_s* p) {
     bool any = false;
     while (!p->inflight.empty()) {
         InflightBatch& ib = p->inflight.front();
-        cudaError_t e = cudaEventQuery(ib.ev);
+        cudaError_t e = cudaEventQuery(ib.ev.get());
         if (e == cudaErrorNotReady) break;
         const bool expired = p->h_status && *(volatile int*)p->h_status != 0;
         if (expired) *(volatile int*)p->h_status = 0;
         const double t_done = now_s();
         float exec_ms = 0.f;
-        if (e == cudaSuccess && cudaEventElapsedTime(&exec_ms, ib.ev_start, ib.ev) != cudaSuccess) exec_ms = 0.f;
+        if (e == cudaSuccess && cudaEventElapsedTime(&exec_ms, ib.ev_start, ib.ev.get()) != cudaSuccess) exec_ms = 0.f;
         for (uint64_t t : ib.tickets) {
             auto it = p->tickets.find(t);
             if (it == p->tickets.end()) continue;
@@ -724,7 +729,6 @@ bool retire(bf_plan_s* p) {
         for (auto& r : ib.release) p->carry_pool.emplace(r.first, r.second);
         if (ib.track.host) p->track_pool.emplace(ib.track.bytes, ib.track);
         for (int t : ib.slots) release_table(p, t);
-        p->event_pool.push_back(ib.ev);
         p->event_pool.push_back(ib.ev_start);
         p->inflight.pop_front();
         any = true;
@@ -1008,11 +1012,19 @@ static int poll_ticket(bf_plan_t p, uint64_t ticket, int64_t timeout_us, int64_t
         if (timeout_us >= 0 && el >= timeout_us) return BF_PENDING;
         // inflight: poll the event; queued: wait for the worker.  A timed sleep lasts some 60 us (10 us
         // and the timer slack), as long as the kernel of a short request, so on a direct plan
-        // the first milliseconds are polled without sleeping, with the lock open in between.
+        // the first milliseconds are polled without sleeping and without the lock, which another thread's
+        // call on the plan would otherwise have to catch between two queries.
         if (it->second.state == T_INFLIGHT && p->cfg.mode == BF_MODE_DIRECT && el < kPollSpinUs) {
+            const auto batch = std::find_if(p->inflight.begin(), p->inflight.end(),
+                                            [&](const InflightBatch& ib) { return ib.id == it->second.batch; });
+            EventRef ev = batch->ev;
+            const auto end = t0 + std::chrono::microseconds(
+                                      timeout_us >= 0 ? std::min<int64_t>(timeout_us, kPollSpinUs) : kPollSpinUs);
             lk.unlock();
-            std::this_thread::yield();
+            while (cudaEventQuery(ev.get()) == cudaErrorNotReady && std::chrono::steady_clock::now() < end)
+                std::this_thread::yield();
             lk.lock();
+            ev.reset();
         } else {
             p->cv.wait_for(lk, std::chrono::microseconds(it->second.state == T_INFLIGHT ? 10 : 200));
         }
@@ -1046,11 +1058,11 @@ int bf_destroy(bf_plan_t p) {
         for (auto& kv : p->streams)
             if (kv.second.carry) cudaFree(kv.second.carry);
         for (auto& ib : p->inflight) {
-            cudaEventDestroy(ib.ev);
             cudaEventDestroy(ib.ev_start);
             for (auto& r : ib.release) cudaFree(r.second);
             if (ib.track.host) p->track_pool.emplace(ib.track.bytes, ib.track);
         }
+        p->inflight.clear();                 // their events to the pool
         for (auto& kv : p->carry_pool) cudaFree(kv.second);
         for (auto& kv : p->track_pool) {
             cudaFreeHost(kv.second.host);
