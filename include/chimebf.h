@@ -208,7 +208,9 @@ int bf_skymap(bf_plan_t p, const float* d_out, int64_t n_sub, int64_t n_frames, 
  * highest sub-channel is floor(((4.148808e3 * dm) * (1/(f f) - 1/(fmax fmax)))
  * / 0.98304e-3 + 1/2) with f in MHz (FP64, that order).  Writes
  * d_series float [1024][n_out] with n_out = n_frames - max delay (0 if
- * negative; *n_out reports it): series[b][t] = sum_s out[b][s][t + d_s].
+ * negative; *n_out reports it): series[b][t] = sum_s out[b][s][t + d_s], added
+ * in an order that depends on n_chan alone, so a sample has the same bits in a
+ * longer or shorter series at the same DM.
  * The delay table goes to plan-owned device memory; the kernel is enqueued
  * on the plan's stream and the call returns at once.
  */

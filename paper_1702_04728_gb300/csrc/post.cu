@@ -214,65 +214,77 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
 // Incoherent dedispersion to one DM: series[beam][t] = sum over sub-channels s
 // of in[beam][s][t + d_s], t < n_out.  Threads run along t, so each sub-channel row
 // is read with coalesced (unaligned) loads.  A CTA takes up to 1024 frames of a beam, kR of them per
-// thread and wt apart, so that a row is read as one piece; `groups` of wt threads take a contiguous
-// share of the sub-channels each (in order), added in order at the end.  A thread loads dd_unroll rows
-// at a time: eight of long rows keep some 100 KB in flight per SM, of short ones (many groups) two are
-// enough and better (54 us at 64 frames, four 61, eight 66).  1024 sub-channels x 1017 frames to 630:
-// 446 us (5.9 TB/s); 64 frames to 58: 54 us (128 frames per CTA, rows one after the other: 518 and
-// 136 us).
+// thread and wt apart, so that a row is read as one piece.
+//
+// The sub-channels are cut into `parts` runs (by their number alone), each summed in order, and the runs' sums
+// are added in order, so a sample has the same bits in a series of any length.  `groups` of wt threads share
+// the runs; the first one adds its own runs as they come, which keeps the sums of the longest tiles below
+// 48 KB.  Eight rows at a time, their delays in two loads, keep some 100 KB in flight per SM; short
+// series (kR = 1) need four CTAs for that, 32 registers a thread.
+//
+// Bound by HBM and, below some 200 frames, by latency.  1024 sub-channels x 1017 frames to 630: 435 us
+// (6.1 TB/s), 200 frames to 194: 156, 96 to 90: 76, 64 to 58: 56, 40 to 34: 50; a contiguous share of the
+// sub-channels per thread group, whose number follows the length, took 439, 155, 76, 55 and 45.  16 runs
+// instead of 20: 84 us at 90 frames (five groups); 24, one more than fits in 48 KB, 2 % more at 998.
 constexpr int kDdThreads = 512;
-constexpr int dd_unroll(int r) { return r == 1 ? 2 : 8; }
+constexpr int kDdParts = 20;           // most runs of sub-channels, each of 32 or more
+constexpr int kDdRows = 8;             // rows loaded at a time; a run is a multiple of them
+static_assert(kSub % kDdRows == 0, "a channel's sub-channels are whole loads");
 
 template <int kR>
-__global__ void __launch_bounds__(kDdThreads) dedisperse_kernel(const float* __restrict__ in,
+__global__ void __launch_bounds__(kDdThreads, kR == 1 ? 4 : 0) dedisperse_kernel(const float* __restrict__ in,
                                                                   const int* __restrict__ delays, int n_sub, long long nf,
-                                                                  long long n_out, int wt, int groups,
+                                                                  long long n_out, int wt, int groups, int parts,
                                                                   float* __restrict__ out) {
-    __shared__ float part[kR][kDdThreads];
+    extern __shared__ float run_s[];     // [..][kR][wt]: sum of the first group's runs, then of each other run
     const int g = threadIdx.x / wt, c = threadIdx.x - g * wt;     // wt is a multiple of 32
     const long long t0 = (long long)blockIdx.x * (kR * wt) + c;
     const int beam = blockIdx.y;
-    const int s0 = (int)((long long)n_sub * g / groups), s1 = (int)((long long)n_sub * (g + 1) / groups);
-    float acc[kR];
     bool in_range[kR];
 #pragma unroll
-    for (int r = 0; r < kR; ++r) {
-        acc[r] = 0.f;
-        in_range[r] = t0 + r * wt < n_out;
-    }
-    constexpr int kDdUnroll = dd_unroll(kR);
-    const float* row = in + ((long long)beam * n_sub + s0) * nf + t0;
-    int s = s0;
-    for (; s + kDdUnroll <= s1; s += kDdUnroll, row += kDdUnroll * nf) {
-        float v[kDdUnroll][kR];
+    for (int r = 0; r < kR; ++r) in_range[r] = t0 + r * wt < n_out;
+    auto first = [&](int q) { return n_sub / kDdRows * q / parts * kDdRows; };   // first sub-channel of run q
+    const int own = parts / groups;                               // runs of the first group
+    int q = parts * g / groups, s = first(q);
+    const int q1 = parts * (g + 1) / groups;
+    const float* row = in + ((long long)beam * n_sub + s) * nf + t0;
+#pragma unroll 1
+    for (; q < q1; ++q) {
+        const int s1 = first(q + 1);
+        float acc[kR];
 #pragma unroll
-        for (int k = 0; k < kDdUnroll; ++k) {
-            const float* p = row + k * nf + __ldg(delays + s + k);
+        for (int r = 0; r < kR; ++r) acc[r] = 0.f;
+#pragma unroll 1
+        for (; s < s1; s += kDdRows, row += kDdRows * nf) {
+            int d[kDdRows];
 #pragma unroll
-            for (int r = 0; r < kR; ++r) v[k][r] = in_range[r] ? __ldg(p + r * wt) : 0.f;
+            for (int k = 0; k < kDdRows; k += 4)
+                *reinterpret_cast<int4*>(d + k) = __ldg(reinterpret_cast<const int4*>(delays + s + k));
+            float v[kDdRows][kR];
+#pragma unroll
+            for (int k = 0; k < kDdRows; ++k) {
+                const float* p = row + k * nf + d[k];
+#pragma unroll
+                for (int r = 0; r < kR; ++r) v[k][r] = in_range[r] ? __ldg(p + r * wt) : 0.f;
+            }
+#pragma unroll
+            for (int k = 0; k < kDdRows; ++k)
+#pragma unroll
+                for (int r = 0; r < kR; ++r) acc[r] += v[k][r];
         }
 #pragma unroll
-        for (int k = 0; k < kDdUnroll; ++k)
-#pragma unroll
-            for (int r = 0; r < kR; ++r) acc[r] += v[k][r];
+        for (int r = 0; r < kR; ++r) {
+            float* to = run_s + (max(0, q - own + 1) * kR + r) * wt + c;
+            *to = q > 0 && q < own ? *to + acc[r] : acc[r];
+        }
     }
-    for (; s < s1; ++s, row += nf) {
-        const float* p = row + __ldg(delays + s);
-#pragma unroll
-        for (int r = 0; r < kR; ++r) acc[r] += in_range[r] ? __ldg(p + r * wt) : 0.f;
+    __syncthreads();
+    for (int r = g; r < kR; r += groups) {
+        if (t0 + r * wt >= n_out) continue;
+        float sum = run_s[r * wt + c];
+        for (int k = 1; k <= parts - own; ++k) sum += run_s[(k * kR + r) * wt + c];
+        out[(long long)beam * n_out + t0 + r * wt] = sum;
     }
-    if (groups > 1) {
-#pragma unroll
-        for (int r = 0; r < kR; ++r) part[r][threadIdx.x] = acc[r];
-        __syncthreads();
-        if (g) return;
-        for (int k = 1; k < groups; ++k)
-#pragma unroll
-            for (int r = 0; r < kR; ++r) acc[r] += part[r][k * wt + c];
-    }
-#pragma unroll
-    for (int r = 0; r < kR; ++r)
-        if (in_range[r]) out[(long long)beam * n_out + t0 + r * wt] = acc[r];
 }
 
 // Delay table of the allocation-free dedispersion entry point: one array per
@@ -336,14 +348,16 @@ cudaError_t dedisperse_static_table(int device, int** table) {
 cudaError_t dedisperse_launch(const float* in, const int* delays, int n_sub, long long nf, long long n_out,
                               float* out, cudaStream_t s) {
     if (n_out <= 0) return cudaSuccess;
-    // tiles of equal width up to 1024 frames, up to 256 threads along them; groups: as many as fill the
-    // CTA, each of 32 sub-channels or more
+    // tiles of equal width up to 1024 frames, up to 256 threads along them
     const long long tiles = (n_out + 1023) / 1024, width = (n_out + tiles - 1) / tiles;
     const int r = (int)((width + 255) / 256), wt = (int)(((width + r - 1) / r + 31) / 32 * 32);
-    const int groups = std::max(1, std::min(kDdThreads / wt, n_sub / 32));
+    // groups: as many as fill the CTA, fewer where that leaves the longest share of the runs as it is
+    const int parts = std::max(1, std::min(kDdParts, n_sub / 32)), most = std::min(kDdThreads / wt, parts);
+    const int share = (parts + most - 1) / most, groups = (parts + share - 1) / share;
     const dim3 grid((unsigned)((n_out + r * wt - 1) / (r * wt)), kBeams);
+    const size_t smem = (size_t)(parts - parts / groups + 1) * r * wt * sizeof(float);   // at most 45 KB: 11 sums of 1024 frames
     auto kernel = r == 1 ? dedisperse_kernel<1> : r == 2 ? dedisperse_kernel<2> : r == 3 ? dedisperse_kernel<3> : dedisperse_kernel<4>;
-    kernel<<<grid, wt * groups, 0, s>>>(in, delays, n_sub, nf, n_out, wt, groups, out);
+    kernel<<<grid, wt * groups, smem, s>>>(in, delays, n_sub, nf, n_out, wt, groups, parts, out);
     return cudaGetLastError();
 }
 

@@ -216,6 +216,22 @@ def test_dedisperse_tiles(built_lib, n_chan, nf, dm):
     assert np.max(np.abs(ser - ref) / ref) <= 1e-5
 
 
+@pytest.mark.parametrize("n_chan", [5, 9, 37])
+def test_dedispersed_samples_do_not_depend_on_the_series_length(built_lib, n_chan):
+    """A sample of a series has the bits that it has in a longer series at the same DM: lengths for every number
+    of frames per thread and of thread groups, and for several tiles; 2, 4 and 8 runs of sub-channels."""
+    gen = torch.Generator(device="cuda").manual_seed(n_chan)
+    freqs = [500e6 + 100e6 * k / n_chan for k in range(n_chan)]
+    x = torch.rand((1024, 16 * n_chan, 2060), generator=gen, device="cuda").mul_(1e6).add_(1e4)
+    with B.Plan() as p:
+        whole = p.dedisperse(x, freqs, 3.0)
+        lost = x.shape[2] - whole.shape[1]
+        assert 5 < lost < 60
+        for n in (1, 32, 33, 64, 97, 129, 161, 200, 257, 400, 513, 800, 1024, 1030, 1900):
+            part = p.dedisperse(x[:, :, :n + lost].contiguous(), freqs, 3.0)
+            assert torch.equal(part, whole[:, :n]), f"{n} of {whole.shape[1]} samples"
+
+
 @pytest.mark.parametrize("nf", [128, 41, 1017])
 def test_rescale_u8_rows_without_a_finite_spread(built_lib, nf):
     """A row's code is 64 where its spread is zero, not a number or beyond FP32: constant rows, rows with a
