@@ -344,6 +344,9 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
             const Seg& sg = bt.segs[sgi];
             const int local = item - sg.item_begin;
             const int F = local >> 2, j = local & 3;
+            // lanes may have parted in the last unit's add_passes; barriers and tensor memory want the whole warp
+            // (here 1.399 ms per 4 x 49152 samples, as without; behind add_passes 1.415)
+            __syncwarp();
             // the table changes with the channel only (reloaded for every item 1.408 ms per 4 x 49152
             // samples, 1.397 so); its number is in shared memory because a register more costs 1 %
             if (sg.table != *(volatile int*)&table_s) {
@@ -435,6 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
                                     ((v[0][s2] + v[1][s2]) + v[2][s2]) + ((v[3][s2] + v[4][s2]) + v[5][s2]);
                         }
                     }
+                    __syncwarp();        // as at the unit's start, for the next pass
                 }
                 if constexpr (kMode == kItems) {
                     if (whole && ps == kPasses / 2 - 1) {
