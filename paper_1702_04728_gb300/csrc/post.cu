@@ -69,9 +69,10 @@ constexpr int kU8Chunk = 256;          // frames per chunk of longer rows
 // floats between staged rows of up to n frames: a multiple of 4 whose quarter is odd
 __host__ __device__ constexpr int u8_stride(int n) { return 4 * (((n + 3) / 4) | 1); }
 
-// kVec: rows are a multiple of 4 frames and start on 16 bytes (codes: 4 bytes).
-template <bool kVec>
-__global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __restrict__ in, long long rows, int nf,
+// kVec: rows are a multiple of 4 frames and start on 16 bytes (codes: 4 bytes).  Len: numbers the frames of
+// a row, 64 bits for rows beyond 2^31 frames only (for all rows they cost up to 10 %).
+template <bool kVec, class Len>
+__global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __restrict__ in, long long rows, Len nf,
                                                                   int chunk, uint8_t* __restrict__ codes,
                                                                   float* __restrict__ stats) {
     extern __shared__ __align__(16) float st[];
@@ -84,10 +85,10 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
     constexpr int V = kVec ? 4 : 1;                       // frames per access
 
     // n frames from f0 of the CTA's rows; whole rows are one contiguous block, walked without divisions
-    auto stage = [&](int f0, int n) {
+    auto stage = [&](Len f0, int n) {
         __syncthreads();
         if (n == nf) {
-            const int per = nf / V, total = nr * per, dr = kU8Threads / per, dc = kU8Threads % per;
+            const int per = (int)nf / V, total = nr * per, dr = kU8Threads / per, dc = kU8Threads % per;
             const int step = dr * S + V * dc, wrap = S - V * per;
             int c = tid % per, o = tid / per * S + V * c;     // o: the access's place among the staged rows
 #pragma unroll 8
@@ -135,8 +136,8 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
     };
     const bool sums = warp == 0 && lane < nr, single = chunk >= nf;
     float x0 = 0.f, s = 0.f, q = 0.f;
-    for (int f0 = 0; f0 < nf; f0 += chunk) {
-        const int n = min(chunk, nf - f0);
+    for (Len f0 = 0; f0 < nf; f0 += chunk) {
+        const int n = (int)min((Len)chunk, nf - f0);
         stage(f0, n);
         if (!sums) continue;
         if (f0 == 0) {
@@ -149,8 +150,8 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
         }
     }
     const float mean = x0 + s / (float)nf;
-    for (int f0 = 0; f0 < nf; f0 += chunk) {
-        const int n = min(chunk, nf - f0);
+    for (Len f0 = 0; f0 < nf; f0 += chunk) {
+        const int n = (int)min((Len)chunk, nf - f0);
         if (!single) stage(f0, n);
         if (!sums) continue;
         each(n, [&](int, float v) {
@@ -167,8 +168,8 @@ __global__ void __launch_bounds__(kU8Threads) rescale_u8_kernel(const float* __r
         }
     }
     __syncthreads();
-    for (int f0 = 0; f0 < nf; f0 += chunk) {
-        const int n = min(chunk, nf - f0);
+    for (Len f0 = 0; f0 < nf; f0 += chunk) {
+        const int n = (int)min((Len)chunk, nf - f0);
         if (!single) stage(f0, n);
         uint8_t* dst = codes + r0 * nf + f0;
         // the clamped value's floor sits in the low byte of its sum with 2^23, rounded down
@@ -384,12 +385,11 @@ cudaError_t rescale_u8_launch(const float* in, long long rows, long long nf, uin
                               cudaStream_t s) {
     if (rows <= 0 || nf <= 0) return cudaSuccess;
     const long long ctas = (rows + kU8Rows - 1) / kU8Rows;
-    if (nf > 0x7fffff00LL || ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
+    if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;                  // more than any memory holds
     const bool vec = (nf & 3) == 0 && (reinterpret_cast<uintptr_t>(in) & 15) == 0 && (reinterpret_cast<uintptr_t>(codes) & 3) == 0;
     const int chunk = nf <= kU8Whole ? (int)nf : kU8Chunk;
     const size_t smem = (size_t)kU8Rows * u8_stride(chunk) * sizeof(float);
-    auto kernel = vec ? rescale_u8_kernel<true> : rescale_u8_kernel<false>;
-    // more shared memory than a launch gets by default, once per device
+    // more shared memory than a launch gets by default, once per device (rows of 2^31 frames go in chunks)
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -398,12 +398,18 @@ cudaError_t rescale_u8_launch(const float* in, long long rows, long long nf, uin
     static cudaError_t result[kMaxDevices];
     std::call_once(once[dev], [&] {
         const int most = (int)(kU8Rows * u8_stride(kU8Whole) * sizeof(float));
-        result[dev] = cudaFuncSetAttribute(rescale_u8_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        result[dev] = cudaFuncSetAttribute(rescale_u8_kernel<true, int>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (result[dev] == cudaSuccess)
-            result[dev] = cudaFuncSetAttribute(rescale_u8_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            result[dev] = cudaFuncSetAttribute(rescale_u8_kernel<false, int>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     });
     if (result[dev] != cudaSuccess) return result[dev];
-    kernel<<<(unsigned)ctas, kU8Threads, smem, s>>>(in, rows, (int)nf, chunk, codes, stats);
+    if (nf + kU8Chunk > 0x7fffffffLL) {
+        auto kernel = vec ? rescale_u8_kernel<true, long long> : rescale_u8_kernel<false, long long>;
+        kernel<<<(unsigned)ctas, kU8Threads, smem, s>>>(in, rows, nf, chunk, codes, stats);
+    } else {
+        auto kernel = vec ? rescale_u8_kernel<true, int> : rescale_u8_kernel<false, int>;
+        kernel<<<(unsigned)ctas, kU8Threads, smem, s>>>(in, rows, (int)nf, chunk, codes, stats);
+    }
     return cudaGetLastError();
 }
 
