@@ -61,6 +61,12 @@ inline PassUnits pass_units(int n_items, int slots, int least_g) {
         if (rem * (kPasses / g) <= slots) return {n_items - rem, g, n_items - rem + rem * (kPasses / g)};
     return {n_items, kPasses, n_items};
 }
+// Room for the sums of split items on `grid` CTAs (as many slots, or half as many of CTA pairs): every part has a
+// slot, so at most grid / 2 items are split (in halves), and they publish at most 2 grid sums of 16 x 256 floats:
+// grid / 3 items in thirds all six passes each, fewer in the other cases (items in halves publish two in
+// the FP32 form, and six, of grid / 4 items, in the tensor-core forms).
+inline size_t part_items(int grid) { return (size_t)grid / 2; }
+inline size_t part_sums(int grid) { return 2 * (size_t)grid; }
 
 struct Batch {
     int n_segs;
@@ -75,8 +81,8 @@ struct Batch {
     int stall_mma;               // stall check: the MMA warps (else the builders) stop ...
     int stall_chunks;            // ... after this many chunks of 32 feeds
     PassUnits units;             // work units of the launch
-    float* part;                 // sums of split items' passes [CTAs][6][16][256]
-    unsigned long long* part_tok;    // [CTAs][256] passes published (see add_passes)
+    float* part;                 // sums of split items' passes [item][6] or halves [item][2], each [16][256]
+    unsigned long long* part_tok;    // [item][256] passes published (see add_passes)
     unsigned long long epoch;        // this launch's number within the plan (from 1)
     Seg segs[kMaxSegs];
 };

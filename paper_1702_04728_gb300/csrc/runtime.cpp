@@ -889,12 +889,10 @@ int bf_plan(const bf_config* cfg, bf_plan_t* out) {
     CK(cudaHostAlloc(&p->h_status, sizeof(int), cudaHostAllocMapped));
     *p->h_status = 0;
     CK(cudaHostGetDevicePointer(&p->d_status, p->h_status, 0));
-    // a launch splits fewer items than it has CTAs: six passes of 16 x 256 floats each, and one token
-    // per bin
-    const size_t slots = (size_t)p->grid;
-    CK(cudaMalloc(&p->d_part, slots * kTds * kPol * kSub * kNs * sizeof(float)));
-    CK(cudaMalloc(&p->d_part_tok, slots * kNs * sizeof(unsigned long long)));
-    CK(cudaMemset(p->d_part_tok, 0, slots * kNs * sizeof(unsigned long long)));
+    // one sum is 16 x 256 floats, and an item has a token per bin
+    CK(cudaMalloc(&p->d_part, part_sums(p->grid) * kSub * kNs * sizeof(float)));
+    CK(cudaMalloc(&p->d_part_tok, part_items(p->grid) * kNs * sizeof(unsigned long long)));
+    CK(cudaMemset(p->d_part_tok, 0, part_items(p->grid) * kNs * sizeof(unsigned long long)));
 
     if (p->cfg.mode == BF_MODE_SERVING) {
         bf_plan_s* raw = p.get();
