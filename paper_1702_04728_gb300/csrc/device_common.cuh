@@ -34,7 +34,6 @@ __device__ __forceinline__ cp ld_cp(const float4* p) {
     const float4 v = *p;
     return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
 }
-__device__ __forceinline__ void st_cp(float4* p, cp a) { *p = make_float4(a.re.x, a.re.y, a.im.x, a.im.y); }
 
 __device__ __forceinline__ void dft4(cp& a0, cp& a1, cp& a2, cp& a3) {
     const cp s02 = cadd(a0, a2), d02 = csub(a0, a2), s13 = cadd(a1, a3);
@@ -402,39 +401,11 @@ __device__ __forceinline__ void cta_sync() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-__device__ __forceinline__ const uint8_t* frame_row(const Seg& sg, long long row) {
-    return row < sg.carry_rows ? sg.carry + row * kInput : sg.vin + (row - sg.carry_rows) * kInput;
-}
-
 // Second up-channel pass for one thread (TMEM lane, bin half hh): 16-point DFTs
 // over the residue b for fine channels q = c + 8 d, two c at a time (SoA), then
-// |.|^2 into the fftshifted sub-channels (d + 8) mod 16.  With `dump` set, the
-// up-channelised voltages of bin m are written instead (fine channel q' order).
-__device__ __forceinline__ void upchan_pass2(uint32_t tlane, int hh, float2 (&acc)[kSub], float2* dump) {
-#pragma unroll 1
-    for (int cpi = 0; cpi < 4; ++cpi) {
-        cp y[16];
-        tmem_ld64(tlane + hh * 256 + 64 * cpi, y);
-        dft16(y);
-        if (dump) {
-#pragma unroll
-            for (int dd = 0; dd < 16; ++dd) {
-                const int c0 = 2 * cpi;
-                dump[(c0 + 8 * dd + kUp / 2) & (kUp - 1)] = make_float2(y[dd].re.x, y[dd].im.x);
-                dump[(c0 + 1 + 8 * dd + kUp / 2) & (kUp - 1)] = make_float2(y[dd].re.y, y[dd].im.y);
-            }
-        } else {
-#pragma unroll
-            for (int dd = 0; dd < 16; ++dd) {
-                const float2 p = fma2(y[dd].im, y[dd].im, mul2(y[dd].re, y[dd].re));
-                acc[(dd + 8) & 15] = add2(acc[(dd + 8) & 15], p);
-            }
-        }
-    }
-}
-
-// The same with one float per sub-channel: the two fine channels of a SoA pair
-// are added before they join the running sum.
+// |.|^2 into the fftshifted sub-channels (d + 8) mod 16, the two fine channels of
+// a SoA pair added first.  With `dump` set, the up-channelised voltages of bin m
+// are written instead (fine channel q' order).
 __device__ __forceinline__ void upchan_pass2(uint32_t tlane, int hh, float (&acc)[kSub], float2* dump) {
 #pragma unroll 1
     for (int cpi = 0; cpi < 4; ++cpi) {

@@ -877,7 +877,7 @@ int bf_plan(const bf_config* cfg, bf_plan_t* out) {
     p->slot_used.assign(p->table_cap, 0);
     p->atc_blocks.assign((p->table_cap + kTcBlock - 1) / kTcBlock, nullptr);
     CK(cudaMalloc(&p->d_lut, (size_t)p->table_cap * kNs * sizeof(int16_t)));
-    CK(cudaMalloc(&p->d_order, (size_t)p->table_cap * kNs * sizeof(int16_t)));
+    if (!p->terms) CK(cudaMalloc(&p->d_order, (size_t)p->table_cap * kNs * sizeof(int16_t)));
     CK(cudaMalloc(&p->d_ew, (size_t)p->table_cap * kEw * kCyl * sizeof(float2)));
     CK(cudaMalloc(&p->d_twl, kLaneTwLen * sizeof(float2)));
     std::vector<float2> tw(kLaneTwLen);
