@@ -171,10 +171,9 @@ def test_node_slice_full_size_sampled(plan):
                                       (B.BF_TC_DFT256_X2, 1e-3)])
 def test_tail_split_items_match_whole_items(built_lib, form, rel):
     """A launch whose last round of items would leave at least half of the CTAs
-    idle runs each item of that round as two half units on two CTAs (the 2-term
-    form never splits).  The output must equal, bit for bit, a run of the same
-    stream in two requests whose items all run whole, and the oracle within the
-    form's tolerance."""
+    (or CTA pairs) idle runs each item of that round in parts on several of them.  The
+    output must equal, bit for bit, a run of the same stream in two requests, one
+    of whole items and one short one, and the oracle within the form's tolerance."""
     with B.Plan(form=form) as plan:
         _tail_split_case(plan, rel)
 

@@ -4,9 +4,8 @@ least recently used one that no open stream and no running batch references.
 
 A serving plan with 64 slots runs 1100 requests of distinct frequencies (more
 than 17 times its slots) with up to 24 in flight, for the FP32 form and the
-1-term tensor-core forms (256 rows: twiddle images per slot; 512 rows: the
-bin-to-beams tables per slot); sampled results match the oracle, and a frequency
-whose slot was refilled many times over gives the same bits as on first use.
+1-term tensor-core forms (256 and 512 rows by name, one kernel with a twiddle
+image per slot); sampled results match the oracle, and a frequency whose slot was refilled many times over gives the same bits as on first use.
 More distinct frequencies than slots in one request fail cleanly.
 """
 import collections

@@ -9,9 +9,10 @@ output element against the oracle):
 * BF_TC_DFT256 (3 terms: twiddles hi+lo, data hi+lo): 1e-5, as the FP32 path;
 * BF_TC_DFT256_X2 (2 terms: twiddles hi, data hi+lo): 1e-3;
 * BF_TC_DFT256_X1 (1 term: twiddles hi, data hi): 1e-3 (measured 3.3-3.5e-4);
-* BF_TC_DFT512 (all 512 rows of the zero-padded transform, 1 term, the clamp
-  applied to the result): 1e-3, and the same values as BF_TC_DFT256_X1, whose
-  rows are the kept rows of the same FP16 matrix.
+* BF_TC_DFT512 (the clamp of the 512-row zero-padded transform, 1 term; it runs
+  BF_TC_DFT256_X1's kernel, since rows that the clamp drops reach no output):
+  1e-3, and 2e-5 from the definition, all 512 rows with FP16 operands and the
+  clamp applied to them.
 """
 import numpy as np
 import pytest
@@ -99,8 +100,7 @@ def test_tc_multichannel_ragged_and_node_slice_sample(built_lib):
 
 
 def test_dft512_point_source(built_lib):
-    # the data of the point-source case (one channel at 600 MHz, 3072 samples) through the
-    # 512 x 256 DFT-matrix GEMM
+    # the data of the point-source case (one channel at 600 MHz, 3072 samples)
     raw, f = synth.config_point_source(0)
     with B.Plan(form=B.BF_TC_DFT512) as p:
         out = p.run(dev(raw), list(f)).cpu().numpy()
@@ -110,7 +110,41 @@ def test_dft512_point_source(built_lib):
     assert int(out.sum(axis=(1, 2)).argmax()) == 939
 
 
+def clamped_512_row_transform(raw, freq):
+    """float64 [1024][16][n_frames]: the 512 x 256 DFT matrix and the E-W phased feeds rounded to FP16, all 512
+    rows evaluated in FP64, the clamp as a gather of rows, then stages 3 to 5 in FP64."""
+    nf = raw.shape[0] // 384
+    b = torch.from_numpy(raw[:384 * nf]).cuda()
+    x = torch.complex((b >> 4).double() - 8, (b & 15).double() - 8).view(384 * nf, 4, 256, 2)
+    w = torch.from_numpy(np.ascontiguousarray(O.ew_weights(freq))).cuda()            # [c, j]
+    y = torch.einsum("cj,tcnp->jptn", w, x)
+    yr, yi = (v.float().half().double() for v in (y.real, y.imag))
+    th = 2 * np.pi * (np.outer(np.arange(512), np.arange(256)) % 512) / 512
+    C, S = (torch.from_numpy(f(th).astype(np.float16).astype(np.float64)).cuda() for f in (np.cos, np.sin))
+    X = torch.complex(yr @ C.T + yi @ S.T, yi @ C.T - yr @ S.T)                      # [j, p, t, 512]
+    X = X[..., torch.from_numpy(O.clamp_lut(freq).astype(np.int64)).cuda()]
+    Y = torch.fft.fft(X.view(4, 2, nf, 3, 128, 256), dim=4)
+    P = torch.fft.fftshift((Y.real ** 2 + Y.imag ** 2).sum(dim=(1, 3)), dim=2)       # [j, F, q', m]
+    return P.view(4, nf, 16, 8, 256).sum(dim=3).permute(0, 3, 2, 1).reshape(1024, 16, nf).cpu().numpy()
+
+
+def test_dft512_is_the_clamp_of_all_512_rows(built_lib):
+    """The form against its definition with the same operands' rounding: what remains are the FP32 sums and, where
+    the phased feeds in FP32 lie next to the middle of two FP16 values (one in 2^12), the other
+    neighbour: 2^-11 of one feed in eight rows or so, 1e-5 of a row and a tenth of that in an output's 96 squares.
+    2e-5 is far below the 3e-4 between the operands' rounding and FP64."""
+    freqs = [410e6, 600e6]
+    raw = synth.noise_only(freqs, 384 * 3, seed=36)
+    with B.Plan(form=B.BF_TC_DFT512) as p:
+        out = p.run(dev(raw), freqs).cpu().numpy()
+    for c, f in enumerate(freqs):
+        ref = clamped_512_row_transform(raw[c], f)
+        assert rel_err(out[:, 16 * c:16 * c + 16], ref) <= 2e-5
+        assert rel_err(ref, O.beamform(raw[c:c + 1], [f])) > 5e-5     # the rounding is what is compared
+
+
 def test_dft512_equals_the_256_row_form(built_lib):
+    # both names of the 1-term kernel, which takes the kept rows only: the plans' tables and images agree;
     # 410 MHz leaves bins that no beam takes; at 600 MHz aliasing gives some bins two beams
     freqs = [410e6, 600e6, 790e6]
     assert len(set(O.clamp_lut(600e6).tolist())) < 256
@@ -121,8 +155,6 @@ def test_dft512_equals_the_256_row_form(built_lib):
     with B.Plan(form=B.BF_TC_DFT256_X1) as p:
         o256 = p.run(dev(raw), freqs).cpu().numpy()
     assert o512.shape == (1024, 48, 5)
-    # the kept rows of the 512-row GEMM are the 256-row form's rows: same FP16 operands,
-    # same accumulation order, same epilogue
     assert np.array_equal(o512, o256)
     assert rel_err(o512, O.beamform(raw, freqs)) <= 1e-3
 
@@ -140,7 +172,7 @@ def test_dft512_streams_carry_dumps_and_stall_check(built_lib):
         with pytest.raises(B.BfError) as e:
             B.bf_debug_gemm(p.handle, freqs[0], vin, 384, out)
         assert e.value.code == B.BF_EINVAL
-        # the stall check runs the form's own kernel (clusters of four)
+        # the stall check runs the 1-term kernel
         assert B.bf_debug_stall(p.handle, vin, 1000000) == B.BF_ETIMEDOUT
     got = np.concatenate([a, b], axis=2)
     assert got.shape == (1024, 32, 4)

@@ -5,7 +5,7 @@ A request may carry one row of four E-W sines per output frame; the host
 turns each row into phases in FP64 and the fused kernels weight the
 cylinders of every frame with its own row.  Tolerances as for static beams:
 1e-5 relative for the FP32 form and the 3-term tensor-core form, 1e-3 for the
-1-term forms on CTA clusters (256 and 512 rows).
+1-term forms (256 and 512 rows by name, one kernel).
 """
 import numpy as np
 import pytest
