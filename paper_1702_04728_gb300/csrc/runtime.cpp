@@ -696,12 +696,13 @@ int launch_jobs(bf_plan_s* p, std::vector<Job>& jobs, size_t bytes) {
     return BF_OK;
 }
 
-// Retire finished batches (caller holds the lock).  Returns true if any.
-bool retire(bf_plan_s* p) {
+// Retire finished batches (caller holds the lock).  Returns true if any.  Batches up to `done` are known to
+// have completed (a batch's event stands for the earlier ones of the stream too).
+bool retire(bf_plan_s* p, uint64_t done = 0) {
     bool any = false;
     while (!p->inflight.empty()) {
         InflightBatch& ib = p->inflight.front();
-        cudaError_t e = cudaEventQuery(ib.ev.get());
+        cudaError_t e = ib.id <= done ? cudaSuccess : cudaEventQuery(ib.ev.get());
         if (e == cudaErrorNotReady) break;
         const bool expired = p->h_status && *(volatile int*)p->h_status != 0;
         if (expired) *(volatile int*)p->h_status = 0;
@@ -983,10 +984,11 @@ static int poll_ticket(bf_plan_t p, uint64_t ticket, int64_t timeout_us, int64_t
     if (!p) return fail(BF_EINVAL, "null plan");
     const auto t0 = std::chrono::steady_clock::now();
     std::unique_lock<std::mutex> lk(p->mu);
+    uint64_t done = 0;
     for (;;) {
         auto it = p->tickets.find(ticket);
         if (it == p->tickets.end()) return fail(BF_ENOTICKET, "unknown ticket");
-        if (it->second.state == T_INFLIGHT) retire(p);
+        if (it->second.state == T_INFLIGHT) retire(p, done);
         it = p->tickets.find(ticket);
         if ((it->second.state == T_DONE || it->second.state == T_ERROR) && times) {
             times[0] = it->second.t_submit;
@@ -1018,9 +1020,12 @@ static int poll_ticket(bf_plan_t p, uint64_t ticket, int64_t timeout_us, int64_t
             EventRef ev = batch->ev;
             const auto end = t0 + std::chrono::microseconds(
                                       timeout_us >= 0 ? std::min<int64_t>(timeout_us, kPollSpinUs) : kPollSpinUs);
+            const uint64_t id = batch->id;
             lk.unlock();
-            while (cudaEventQuery(ev.get()) == cudaErrorNotReady && std::chrono::steady_clock::now() < end)
+            cudaError_t q;
+            while ((q = cudaEventQuery(ev.get())) == cudaErrorNotReady && std::chrono::steady_clock::now() < end)
                 std::this_thread::yield();
+            if (q == cudaSuccess) done = id;
             lk.lock();
             ev.reset();
         } else {
