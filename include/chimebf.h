@@ -50,9 +50,9 @@ extern "C" {
  * line is split into FP16 hi + lo, the twiddles are FP16 hi (+ lo).
  * BF_TC_DFT512 is the clamp applied to all 512 rows of the zero-padded
  * transform (the 512 redundant beams of Sec. 3.1) with one GEMM term.  Rows that
- * no pointing keeps reach no output, so they are not computed: it runs the
- * BF_TC_DFT256_X1 kernel and gives its output bit for bit.  Its plans refuse
- * the stage dumps (BF_EINVAL). */
+ * no pointing keeps reach no output, so they are not computed: it is another
+ * name of BF_TC_DFT256_X1, whose kernel it runs and whose output it gives bit for
+ * bit.  Its plans refuse the stage dumps (BF_EINVAL), which would show 256 rows. */
 #define BF_FP32_FFT      0 /* FP32 zero-padded FFT on the CUDA cores                */
 #define BF_TC_DFT256     1 /* 3 GEMM terms: twiddles hi+lo x data hi+lo             */
 #define BF_TC_DFT512     2 /* clamp of all 512 padded rows, 1 GEMM term             */

@@ -46,9 +46,10 @@ struct Seg {
 // Work units of a launch whose items (six passes each) go to `slots` CTAs or CTA pairs in turn: whole
 // items, and the items of a last round that leaves slots idle in parts of g passes, g the smallest
 // from `least_g` that gives every part a slot of its own (parts in several rounds lose more between
-// units, most of a pass each, than they balance: 108 items on 152 CTAs took 181 us in single passes,
-// 121 us whole).  Every output adds the six passes' sums in one fixed order, whether or not its item
-// was split, so the result does not depend on how a request was batched.
+// units, most of a pass each, than they balance: FP32 form, 108 items on 152 CTAs, 181 us in single passes
+// and 121 whole; three terms, 48 items on 76 pairs, 64 and 62).  Every output adds the six passes' sums in
+// one fixed order, whether or not its item was split, so the result does not depend on how a request was
+// batched.
 struct PassUnits {
     int n_full;     // items run whole: 0 .. n_full - 1
     int g;          // passes of a part of the others (1, 2, 3; 6: none is split)

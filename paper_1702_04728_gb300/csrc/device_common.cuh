@@ -95,9 +95,8 @@ __device__ __forceinline__ void bfly(cp& a, cp& b) {
         a = y;
         b = z;
     } else if constexpr ((E & 7) == 4) {
-        // 45 degrees: the tangent is 1, so sums in place of two FMAs with a constant (the same bits;
-        // with the packed difference as an add 1.466 -> 1.462 ms per 4 x 49152 samples, 5.96 -> 5.94 ms
-        // per 1024 channels x 2 frames)
+        // 45 degrees: the tangent is 1, so sums in place of two FMAs with a constant (the same bits; 0.3 % of
+        // an FP32-form launch)
         bfly_p<(E >= 8)>(a, b, add2(b.re, b.im), sub2(b.im, b.re), (float)cos32(4));
     } else {
         constexpr float c = (float)cos32(E & 7), t = (float)(-sin32(E & 7) / (double)c);
@@ -183,7 +182,7 @@ struct PolSel {
     uint32_t mi, mr;
     float si, bi, sr, br;
 };
-// (called by whole warps; in uniform registers: 1.55 -> 1.49 ms per 4 x 49152 samples in the FP32 form)
+// (called by whole warps; uniform registers for these are worth 4 % of an FP32-form launch)
 __device__ __forceinline__ PolSel pol_sel(int pol) {
     const float s = pol ? 1.f / 256.f : 1.f;
     return {uniform(pol ? 0xF00u : 0xFu), uniform(pol ? 0xF000u : 0xF0u), uniform(s),
@@ -224,9 +223,8 @@ __device__ __forceinline__ void load_ew_frame(const Seg& sg, const float2* __res
 
 // Twiddles of the first up-channel pass: [b / 2][c] = (Re, Re', Im, Im') of exp(-2 pi i b c / 128) for b
 // and b + 1.  In constant memory: the FP32 form reads them by a warp-uniform index and so through
-// uniform registers (1.49 -> 1.47 ms per 4 x 49152 samples); the tensor-core forms, whose up-channel
-// warps have a scheduler's slots to themselves less often, from a copy in shared memory (constant reads
-// there: 1.01 -> 1.04 ms).
+// uniform registers (1.3 % of a launch); the tensor-core forms, whose up-channel warps have a scheduler's
+// slots to themselves less often, from a copy in shared memory (constant reads there cost 3 %).
 struct PairTw {
     float4 w[kUp / 16][8];
 };
@@ -336,9 +334,8 @@ __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(mbar) : "memory");
 }
 
-// Segment of a work item, by halving: a launch of 160 two-frame channels spends 5.96 instead of 6.21 ms
-// per 1024 channels against a scan from its first segment, which each read of the table delays by a
-// trip to the constant cache.
+// Segment of a work item, by halving: a scan from the first segment, each read of which is a trip to the
+// constant cache, costs launches of 160 two-frame channels 4 %.
 __device__ __forceinline__ int seg_of(const Batch& bt, int item) {
     int lo = 0, hi = bt.n_segs;
 #pragma unroll 1
@@ -386,7 +383,7 @@ __device__ __forceinline__ bool add_passes(unsigned long long* tok, unsigned lon
 
 // The published sums of an item's six passes for one beam (`in`: its place in pass 0).  All loads come
 // before the caller's first store, which could alias them as far as the compiler knows: with
-// stores in between, the adds of a one-frame request took 16 of its 43 us.
+// stores in between, the adds of a one-frame request take 8 us longer.
 __device__ __forceinline__ void load_passes(const float* in, float (&v)[kTds * kPol][kSub]) {
 #pragma unroll
     for (int k = 0; k < kTds * kPol; ++k)

@@ -118,16 +118,15 @@ __device__ __forceinline__ constexpr uint32_t tslot(int n2, int R) {
 //   rows   the two row pairs' bins (2 x 8 KB; the transpose runs in place)
 // Only warp-level synchronisation.  Hooks: `before_tb` runs before the bin rows are first written,
 // `after_raw`, which requests the next raw rows, between the halves of the first transform, where half of
-// the registers are free (with all of them taken, right after the unpack, 1.460 ms for 4 channels x 49152
-// samples; here 1.453; after the second half 1.51 to 1.53, too late).
+// the registers are free (right after the unpack, with all of them taken, 0.5 % slower; after the second
+// half, too late, 4 %).
 //
 // Bound: the FMA pipe with the register reads of its operands, 530 packed operations per row pair
 // here and 178 in the consumers: 64 % of its cycles, with 52 % of the issue slots; the two producer
 // warps of a scheduler set the pace, the consumers wait for a good third of their time.  4 channels x 49152
-// samples take 1.40 ms.  One row pair per warp and three warps at 128 registers (lane-dependent
-// twiddles in both transforms) took 1.67 ms where this split took 1.57; the unpack straight from the
-// transposing loads replaced a store and two loads of the phased feeds per row pair and the odd half's
-// divergent twiddles (1.64 ms then).
+// samples take 1.40 ms.  One row pair per warp and three warps at 128 registers, with lane-dependent twiddles
+// in both transforms, are 6 % slower; the unpack straight from the transposing loads spares a store and
+// two loads of the phased feeds per row pair and the odd half's divergent twiddles (4 %).
 template <class AfterRaw, class BeforeTb>
 __device__ __forceinline__ void phase_a(uint32_t raw, const PolSel& ps, const EwW& w, uint32_t twl,
                                         uint32_t rows, int lane, AfterRaw after_raw, BeforeTb before_tb) {
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
             const long long row0 = (long long)F * kFrame + 32 * tw;
             // this lane's part of row row0 in the carried and in the new samples, and the number of rows
             // from it that are carried: a row's address is then a comparison and 32-bit arithmetic
-            // (1.453 -> 1.406 ms per 4 x 49152 samples, 5.88 -> 5.68 per 1024 channels x 2 frames)
+            // (3 % of a launch against 64-bit products per row)
             const uint8_t* const carried = sg.carry + row0 * kInput + 16 * lane;
             const uint8_t* const fresh = sg.vin + (row0 - sg.carry_rows) * kInput + 16 * lane;
             const int left = row0 < sg.carry_rows ? (int)(sg.carry_rows - row0) : 0;
@@ -345,10 +344,10 @@ __global__ void __launch_bounds__(kThreads, 1) fused_fp32_kernel(const __grid_co
             const int local = item - sg.item_begin;
             const int F = local >> 2, j = local & 3;
             // lanes may have parted in the last unit's add_passes; barriers and tensor memory want the whole warp
-            // (here 1.399 ms per 4 x 49152 samples, as without; behind add_passes 1.415)
+            // (behind add_passes itself it costs 1 %, here nothing)
             __syncwarp();
-            // the table changes with the channel only (reloaded for every item 1.408 ms per 4 x 49152
-            // samples, 1.397 so); its number is in shared memory because a register more costs 1 %
+            // the table changes with the channel only (reloading it for every item costs 0.8 %); its number
+            // is in shared memory because a register more costs 1 %
             if (sg.table != *(volatile int*)&table_s) {
                 bar_sync_n(kBarCons, 32 * kCons);         // the previous table's reads are done
                 // consumer slot i (TMEM lane + 128 x half) takes beam order[i]

@@ -32,16 +32,15 @@
 // the twiddles and, in the first CTA, issues the MMAs of the pair, warps 12-15 (one per tensor-memory
 // lane quarter) run the up-channel passes and detection for one bin per thread.  16 warps is what the
 // register file gives at 128 a thread; with 8 builders, one per group of 8 times, the loads and the
-// arithmetic of two warps left each scheduler idle for half of its cycles: 0.98 / 1.33 / 1.69 ms for 1 /
-// 2 / 3 terms against 0.89 / 1.06 / 1.39 with 11 (4 x 49152 samples, 152 SMs).  Hand-offs are mbarriers
-// only; every wait is bounded by %globaltimer, and on expiry the CTA records the failure and leaves its
-// loops (the other CTA's waits then expire too).
+// arithmetic of two warps leave each scheduler idle for half of its cycles (10, 25 and 22 % slower with 1, 2
+// and 3 terms).  Hand-offs are mbarriers only; every wait is bounded by %globaltimer, and on expiry
+// the CTA records the failure, leaves its loops (the other CTA's waits then expire too) and waits for its
+// copies and MMAs under way.
 //
 // Bound: the issue slots and the FP32 pipe that the builders' unpack and E-W arithmetic and the one
 // up-channel warp of a scheduler share (61 % and 54 % of cycles for 1 term); the tensor pipe needs 512 x
 // terms cycles of a chunk (3 terms: it and the shared-memory reads of its operands).  Per 4 x
-// 49152-sample request on 152 SMs: 0.89 / 1.06 / 1.39 ms for 1 / 2 / 3 terms, where one CTA with streamed
-// twiddles took 1.89 (2) and 2.55 (3) and CTAs that copied the data tile to each other 1.36 (1).
+// 49152-sample request on 152 SMs: 0.88 / 1.05 / 1.36 ms for 1 / 2 / 3 terms.
 #include "device_common.cuh"
 
 #include <cuda_fp16.h>
@@ -61,7 +60,7 @@ constexpr int kTMma = kTBuild;                    // the MMA / twiddle warp
 constexpr int kTUp = 4;                           // up-channel warps
 constexpr int kTThreads = 32 * (kTBuild + 1 + kTUp);
 // Register split (setmaxnreg, by warpgroup): builders and the MMA warp kTRegBuild, up-channel warps
-// kTRegUp (104 and 200: 0.93 ms for 1 term against 0.89); the launcher checks that the launch gives
+// kTRegUp (104 and 200: 4 % slower with 1 term); the launcher checks that the launch gives
 // enough (with fewer, the up-channel warps' increase could never be granted).
 constexpr int kTRegBuild = 112, kTRegUp = 176;
 
@@ -149,8 +148,8 @@ __device__ __forceinline__ void cluster_sync() {
 }
 // Arrival on an mbarrier of any CTA of the cluster (shared::cluster address).  What it announces was
 // written for the asynchronous proxy (fence.proxy.async) or to tensor memory (tcgen05.fence), so no
-// cluster-wide release is needed; one here costs a memory barrier and an L1 invalidation per chunk
-// (1.83 ms per 4 x 49152-sample request against 1.30).
+// cluster-wide release of other memory is needed; one here is a memory barrier and an L1 invalidation per
+// chunk, 40 % of the time of a 1-term launch.
 __device__ __forceinline__ void arrive_cluster(uint32_t mbar) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" :: "r"(mbar) : "memory");
 }
@@ -425,8 +424,8 @@ __global__ void __launch_bounds__(kTThreads, 1) fused_tc_kernel(const __grid_con
             // ------------------------------ builders ------------------------------
             // The warps take the CTA's tasks (unit, pass, chunk, group of 8 times) in turn.  Lane bits 0-1 take
             // the four feed octets of a chunk, bits 2-4 eight times: a quarter warp loads 64 contiguous bytes
-            // of two rows (lanes on eight different lines at one offset instead take a pass of the L1 data
-            // banks each: 1.29 ms per 4 x 49152-sample request against 1.16)
+            // of two rows (lanes on eight different lines at one offset take a pass of the L1 data banks each, 11 %
+            // of the time of a 1-term launch)
             const int t = 64 * (int)rank + (lane >> 2), oct = lane & 3;
             unsigned char* dst0 = ring + oct * C::B_LBO + (lane >> 2) * 16;
             const uint32_t full0 = cta_addr(bar0, 0);                      // the first CTA's bfull(0)

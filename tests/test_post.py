@@ -234,8 +234,8 @@ def test_dedispersed_samples_do_not_depend_on_the_series_length(built_lib, n_cha
 
 @pytest.mark.parametrize("nf", [128, 41, 1017])
 def test_rescale_u8_rows_without_a_finite_spread(built_lib, nf):
-    """A row's code is 64 where its spread is zero, not a number or beyond FP32: constant rows, rows with a
-    NaN or an infinity, rows whose squares overflow.  The rows between keep their codes, both ends clipped."""
+    """A row's code is 64 where its spread is zero, not a number or, about a finite mean, beyond FP32: constant
+    rows, rows with a NaN or an infinity, rows whose squares overflow.  The rows between keep their codes, both ends clipped."""
     rng = np.random.default_rng(nf)
     x = intensity_rows(rng, 70, nf)
     plain = x.copy()
