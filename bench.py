@@ -38,9 +38,9 @@ FORM_NAMES = {"BF_FP32_FFT": "fp32_fft", "BF_TC_DFT256": "tc_dft256_3term",
               "BF_TC_DFT256_X2": "tc_dft256_2term", "BF_TC_DFT256_X1": "tc_dft256_1term",
               "BF_TC_DFT512": "tc_dft512_1term"}
 # tensor flop per input-sample of each tensor-core form: 8 real flop per (row, feed) and
-# term, over the 256 clamped rows or all 512 rows of the zero-padded transform
+# term, over the 256 rows that the clamp keeps (the 512-row form is another name of the 1-term one)
 TC_FLOP = {"tc_dft256_3term": 3 * 2048, "tc_dft256_2term": 2 * 2048, "tc_dft256_1term": 2048,
-           "tc_dft512_1term": 2048}      # of the 512 rows only the 256 that the clamp keeps
+           "tc_dft512_1term": 2048}
 
 
 def bench_config(form: str) -> dict:
