@@ -113,8 +113,8 @@ int bf_config_default(bf_config* cfg);
  * Create a plan: validates cfg, precomputes in FP64 the twiddle tables and
  * allocates device memory for per-frequency tables (clamp table of Eq. (1)
  * and E-W phases, filled lazily per channel frequency) and stream carry state.
- * An FP32 plan holds some 10 MB of device memory from the start (5 MB of it for
- * the sums of work items that several CTAs share), a tensor-core plan 8 MB and
+ * An FP32 plan holds some 11 MB of device memory from the start (5 MB of it for
+ * the sums of work items that several CTAs share), a tensor-core plan 9 MB and
  * then 16 MB (3 terms: 32) for every 64 distinct frequencies; open streams hold
  * their leftover samples beside that.
  * On success *out owns everything and must be released with bf_destroy.
